@@ -88,12 +88,13 @@ __host__ __device__ __forceinline__ int64_t row_off3(int m, int M2, int M3, int6
 
 // Launch helpers implemented in kernels.cu / solve.cu.  All return a
 // cudaError_t from the launch.
-// CUDA-core complex GEMM (kernels.cu); with part != nullptr (part_cap floats) a
+// CUDA-core complex GEMM (simt_gemm.cu); with part != nullptr (part_cap floats) a
 // launch whose grid is under one wave is split over K into partials (cgemm_plan
 // gives the count and the partial floats) and summed by the fixed-order reduce.
 // force_splits > 0 replaces the heuristic split count (the autotuner's
 // choice); a count whose partials would not fit part_cap falls back to one.
 int cgemm_plan(const GemmDesc& d, size_t* part_floats, int force_splits = 0);
+cudaError_t simt_prepare();  // kernel attributes, once, before any stream capture
 cudaError_t launch_cgemm(const GemmDesc& d, cudaStream_t s, float* part = nullptr,
                          size_t part_cap = 0, int* n_kernels = nullptr, int force_splits = 0);
 // Tensor-core version (tc_gemm.cu) for TN_TF32 / TN_BF16 descriptors.  part:

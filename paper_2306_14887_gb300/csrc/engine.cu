@@ -1694,7 +1694,8 @@ tn_status tn_create(const tn_graph* graph, const tn_config* cfg, const tn_alloca
     return fail(TN_ENOMEM);
   }
   h->h_stats = new double[4 * std::max(1, h->max_layer)];
-  if ((use_tensor_cores(h) && tc_prepare() != cudaSuccess) || normalise_prepare(chi) != cudaSuccess) {
+  if ((use_tensor_cores(h) && tc_prepare() != cudaSuccess) || simt_prepare() != cudaSuccess ||
+      normalise_prepare(chi) != cudaSuccess) {
     cudaGetLastError();
     set_error("setting kernel attributes failed");
     delete[] h->h_stats;

@@ -1,7 +1,6 @@
-// CUDA-core kernels of the tnbp library: the plain-FP32 batched complex GEMM
-// that carries every contraction of the message and gate updates in the
-// TN_FP32 mode, the physical-leg gate, message normalisation with the FP64
-// residual, the single-site reduced density matrix and a batched block copy.
+// CUDA-core kernels of the tnbp library besides the FP32 GEMM: the physical-leg
+// gate, message normalisation with the FP64 residual, the single-site reduced
+// density matrix and a batched block copy.
 #include <algorithm>
 #include <mutex>
 
@@ -9,207 +8,6 @@
 #include "tnbp.h"
 
 namespace tnbp {
-
-// ---------------------------------------------------------------------------
-// Plain FP32 complex GEMM, 64 x 64 output tile per CTA, 16-deep K slices
-// staged in shared memory, 4 x 4 complex outputs per thread (planar re/im
-// accumulators).  Operand loads pick the thread-to-element map that makes
-// consecutive threads read consecutive addresses of whichever index of the
-// operand is contiguous.
-//
-// Summation: each 16-deep slice is summed into fresh registers and the slice
-// sums are added to the running total with an error-free two-sum whose
-// rounding errors are carried in a compensation term (Knuth's TwoSum).  The
-// contractions here run over K up to 2 chi^2 (8192 at chi = 64); a single
-// running FP32 sum would carry an error growing with K, while this keeps it
-// at the 32-term slice plus a few roundings of the total.
-// ---------------------------------------------------------------------------
-namespace {
-constexpr int BM = 64, BN = 64, BK = 16;
-
-// s + c += b with s the rounded sum and c the accumulated rounding errors.
-__device__ __forceinline__ void two_sum_acc(float& s, float& c, float b) {
-  const float t = __fadd_rn(s, b);
-  const float bb = __fsub_rn(t, s);
-  const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(b, bb));
-  s = t;
-  c = __fadd_rn(c, e);
-}
-
-__device__ __forceinline__ int64_t koff(int k, int K2, int64_t s1, int64_t s2) {
-  int k1 = k / K2;
-  int k2 = k - k1 * K2;
-  return (int64_t)k1 * s1 + (int64_t)k2 * s2;
-}
-
-__global__ void __launch_bounds__(256) cgemm_simt_kernel(GemmDesc d, float* part, int splits,
-                                                          int k_per_split) {
-  __shared__ float As[2][BK][BM + 1];
-  __shared__ float Bs[2][BK][BN + 1];
-  int z = blockIdx.z;
-  const int split = z % splits;
-  z /= splits;
-  const int outer = z / d.n_inner;
-  const int inner = z - outer * d.n_inner;
-  if (outer_frozen(d, outer)) return;  // a converged component of a union
-  const float* A = d.A[outer] + inner * d.a_in;
-  const float* B = d.B[outer] + inner * d.b_in;
-  float* C = d.C[outer] + inner * d.c_in;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const int Kall = d.K1 * d.K2;
-  // this CTA's K range (all of K without split-K)
-  const int kb = split * k_per_split;
-  const int K = min(Kall, kb + k_per_split);
-  const bool a_kfast = (d.a_k2 == 1) && !(d.M2 > 1 && d.M3 <= 1 && d.a_m2 == 1) &&
-                       !(d.M3 > 1 && d.a_m3 == 1);
-  const bool b_nfast = (d.b_n == 1);
-  const float sa = d.conj_a ? -1.f : 1.f;
-  const float sb = d.conj_b ? -1.f : 1.f;
-
-  float accr[4][4], acci[4][4], cmpr[4][4], cmpi[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) accr[i][j] = acci[i][j] = cmpr[i][j] = cmpi[i][j] = 0.f;
-
-  for (int k0 = kb; k0 < K; k0 += BK) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int idx = tid + r * 256;
-      int mm, kk;
-      if (a_kfast) { kk = idx & (BK - 1); mm = idx >> 4; }
-      else { mm = idx & (BM - 1); kk = idx >> 6; }
-      const int m = m0 + mm, k = k0 + kk;
-      float re = 0.f, im = 0.f;
-      if (m < d.M && k < K) {
-        const int64_t off = ROW_A(d, m) + koff(k, d.K2, d.a_k1, d.a_k2);
-        re = A[off];
-        im = sa * A[off + d.plane_a];
-      }
-      As[0][kk][mm] = re;
-      As[1][kk][mm] = im;
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int idx = tid + r * 256;
-      int nn, kk;
-      if (b_nfast) { nn = idx & (BN - 1); kk = idx >> 6; }
-      else { kk = idx & (BK - 1); nn = idx >> 4; }
-      const int n = n0 + nn, k = k0 + kk;
-      float re = 0.f, im = 0.f;
-      if (n < d.N && k < K) {
-        const int64_t off = (int64_t)n * d.b_n + koff(k, d.K2, d.b_k1, d.b_k2);
-        re = B[off];
-        im = sb * B[off + d.plane_b];
-      }
-      Bs[0][kk][nn] = re;
-      Bs[1][kk][nn] = im;
-    }
-    __syncthreads();
-    float pr[4][4], pi[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) pr[i][j] = pi[i][j] = 0.f;
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float ar[4], ai[4], br[4], bi[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        ar[i] = As[0][kk][ty + 16 * i];
-        ai[i] = As[1][kk][ty + 16 * i];
-        br[i] = Bs[0][kk][tx + 16 * i];
-        bi[i] = Bs[1][kk][tx + 16 * i];
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          pr[i][j] = fmaf(ar[i], br[j], pr[i][j]);
-          pr[i][j] = fmaf(-ai[i], bi[j], pr[i][j]);
-          pi[i][j] = fmaf(ar[i], bi[j], pi[i][j]);
-          pi[i][j] = fmaf(ai[i], br[j], pi[i][j]);
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        two_sum_acc(accr[i][j], cmpr[i][j], pr[i][j]);
-        two_sum_acc(acci[i][j], cmpi[i][j], pi[i][j]);
-      }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      accr[i][j] = __fadd_rn(accr[i][j], cmpr[i][j]);
-      acci[i][j] = __fadd_rn(acci[i][j], cmpi[i][j]);
-    }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty + 16 * i;
-    if (m >= d.M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx + 16 * j;
-      if (n >= d.N) continue;
-      if (splits > 1) {
-        // split-K partial [split][outer][inner][re|im][M][N], summed by the reduce
-        float* q = part + ((((int64_t)split * d.n_outer + outer) * d.n_inner + inner) * 2) *
-                              (int64_t)d.M * d.N;
-        q[(int64_t)m * d.N + n] = accr[i][j];
-        q[(int64_t)d.M * d.N + (int64_t)m * d.N + n] = acci[i][j];
-        continue;
-      }
-      const int64_t off = ROW_C(d, m) + (int64_t)n * d.c_n;
-      if (d.accumulate) {
-        C[off] += accr[i][j];
-        C[off + d.plane_c] += acci[i][j];
-      } else {
-        C[off] = accr[i][j];
-        C[off + d.plane_c] = acci[i][j];
-      }
-    }
-  }
-}
-}  // namespace
-
-// Split-K for the CUDA-core GEMM: a launch whose grid is under one wave (152
-// CTAs: a few sites with a long contraction, e.g. the closes) is split into at
-// most 64 pieces of at least 256 K values, each summed with the compensated
-// slices, the pieces then summed in FP64 in a fixed order by the reduce.
-int cgemm_plan(const GemmDesc& d, size_t* part_floats, int force_splits) {
-  const int64_t K = (int64_t)d.K1 * d.K2;
-  const int64_t ctas = (int64_t)((d.N + BN - 1) / BN) * ((d.M + BM - 1) / BM) * d.n_outer * d.n_inner;
-  int s = 1;
-  if (force_splits > 0)
-    s = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)force_splits, 64, (K + BK - 1) / BK}));
-  else if (ctas < 152)
-    while (s < 64 && ctas * s * 2 <= 2 * 152 && K / (2 * s) >= 256) s *= 2;
-  *part_floats = s > 1 ? (size_t)s * d.n_outer * d.n_inner * 2 * d.M * d.N : 0;
-  return s;
-}
-
-cudaError_t launch_cgemm(const GemmDesc& d, cudaStream_t s, float* part, size_t part_cap,
-                         int* n_kernels, int force_splits) {
-  if (n_kernels) *n_kernels = 0;
-  if (d.M <= 0 || d.N <= 0 || d.n_outer <= 0 || d.n_inner <= 0) return cudaSuccess;
-  size_t pf = 0;
-  int splits = part ? cgemm_plan(d, &pf, force_splits) : 1;
-  if (splits > 1 && pf > part_cap) splits = 1;  // the caller's partial buffer is too small
-  const int K = d.K1 * d.K2;
-  const int kps = splits > 1 ? ((K + splits - 1) / splits + BK - 1) / BK * BK : K;
-  dim3 grid((d.N + BN - 1) / BN, (d.M + BM - 1) / BM, d.n_outer * d.n_inner * splits);
-  cgemm_simt_kernel<<<grid, 256, 0, s>>>(d, part, splits, kps);
-  if (n_kernels) *n_kernels = splits > 1 ? 2 : 1;
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || splits == 1) return e;
-  return launch_tc_reduce(d, part, splits, s);
-}
 
 // ---------------------------------------------------------------------------
 // 2x2 gate on the physical leg of a list of sites (all of one degree).

@@ -1,0 +1,50 @@
+"""The CUDA-core FP32 GEMM at the edges of its tiles and slices: one BP sweep of
+a degree-3 star (its mode products, rows- and column-contiguous outputs, and the
+split-K closes) against the FP64 oracle's sweep.
+
+Tolerance: the messages have unit Frobenius norm, and each goes through two mode
+products and a close.  Every sum is taken in 16-deep complex slices, 32 FP32
+products each, whose worst-case relative error is 32 * 2^-24 = 1.9e-6; the slice
+sums are added error-free.  Three stages: 6e-6.
+"""
+import numpy as np
+import pytest
+
+from oracle import bptn as OB
+from oracle import graph as OG
+from workloads import random_state
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tnlib():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2306_14887_gb300 import build
+    build.build()
+    import paper_2306_14887_gb300 as tn
+    return tn
+
+
+def one_sweep(tn, g, chi, tensors, msgs, prec):
+    with tn.TNState(g.n, g.edges, g.colours, chi=chi, prec=prec) as s:
+        for v in range(g.n):
+            s.set_site(v, tensors[v])
+        for (src, e), m in msgs.items():
+            s.set_message(e, src, m)
+        s.bp_converge(tol=1e30, max_iters=1)
+        return {k: s.get_message(k[1], k[0]) for k in msgs}, s.expect_z_all()
+
+
+@pytest.mark.parametrize("chi", [1, 2, 3, 8, 15, 16, 17, 31, 32, 33, 48, 63, 64, 65, 96])
+def test_sweep_matches_oracle(tnlib, chi):
+    g = OG.star3_tree()
+    tensors, msgs = random_state([g.degree(v) for v in range(g.n)], g.edges, chi, seed=chi)
+    got, z = one_sweep(tnlib, g, chi, tensors, msgs, "fp32")
+    o = OB.BPState(g, chi)
+    o.T = [t.astype(np.complex64).astype(complex) for t in tensors]
+    o.M = {k: m.astype(np.complex64).astype(complex) for k, m in msgs.items()}
+    o.bp_sweep()
+    assert max(float(np.linalg.norm(got[k] - o.M[k])) for k in o.M) < 6e-6
