@@ -87,7 +87,10 @@ typedef struct {
  *              with hi = round(x), lo = round(x - hi) in the operand format, and
  *              the product is accumulated as hi*hi + hi*lo + lo*hi (three
  *              tensor-core products; the dropped lo*lo term is below FP32
- *              rounding for TF32X3, about 2^-16 relative for BF16X3). */
+ *              rounding for TF32X3, about 2^-16 relative for BF16X3).  Under
+ *              TN_KERNELS_AUTO they run as plain FP32 products, which are no
+ *              less accurate and take less time; TN_KERNELS_TILE forms the
+ *              split products. */
 typedef enum {
   TN_FP32 = 0,
   TN_TF32 = 1,
@@ -117,8 +120,9 @@ typedef struct {
  * TN_KERNELS_AUTO: with TN_TF32 and chi = 32 or 64, the mode products (one leg
  *   of a site tensor times a chi x chi matrix: the BP sweep's first two
  *   contractions per chain, the gate environments and rebuilds) run in the
- *   persistent TMA-fed streaming kernel; every other contraction, and every
- *   contraction of the other modes, in the generic tile kernel.
+ *   persistent TMA-fed streaming kernel; every other contraction of TN_TF32
+ *   and TN_BF16 in the generic tile kernel, those of the split modes on the
+ *   CUDA cores.
  * TN_KERNELS_TILE: the generic tile kernel for every contraction.
  * The two give the same sums in different rounding orders. */
 #define TN_KERNELS_AUTO 0

@@ -453,6 +453,23 @@ bool use_tensor_cores(const tn_handle* h) {
   return h->cfg.prec != TN_FP32;
 }
 
+// Whether a contraction without TMA maps runs in the tensor-core tile kernel;
+// otherwise the CUDA-core GEMM takes it.
+//  - Contractions too small to fill a tile pipeline (the degree-1 closes: chi^2
+//    outputs over K = 2) never do.
+//  - The split modes stage both parts of every operand through registers there,
+//    three products each: the CUDA-core GEMM gives FP32-accurate products in
+//    less time at every chi measured (ms a sweep, tile against CUDA cores:
+//    union of 338 sites chi = 16 1.04 / 0.22, 65 sites chi = 23 0.77 / 0.19,
+//    127 sites chi = 32 1.02 / 0.33, chi = 64 6.99 / 2.61).
+// TN_KERNELS_TILE keeps every contraction that is large enough on the tile kernel.
+bool on_tile_kernel(const tn_handle* h, const GemmDesc& d) {
+  if (!use_tensor_cores(h)) return false;
+  const double macs = (double)d.n_outer * d.n_inner * d.M * d.N * d.K1 * d.K2;
+  if (macs < 262144.0) return false;
+  return h->cfg.kernels == TN_KERNELS_TILE || d.prec == TN_TF32 || d.prec == TN_BF16;
+}
+
 tn_status run_plan(tn_handle* h, const Plan& P, int cls, size_t begin = 0,
                    size_t end = (size_t)-1, bool on_side = false) {
   const cudaStream_t stream = on_side ? h->side : h->stream;
@@ -477,10 +494,6 @@ tn_status run_plan(tn_handle* h, const Plan& P, int cls, size_t begin = 0,
       h->stats.kernel_launches += 1;
       continue;
     }
-    // contractions too small to fill a tensor-core tile pipeline (the
-    // degree-1 closes: chi^2 outputs over K = 2) run on the CUDA cores in FP32
-    const double macs = (double)L.d.n_outer * L.d.n_inner * L.d.M * L.d.N * L.d.K1 * L.d.K2;
-    const bool tiny = macs < 262144.0;
     if (L.sp.maps && L.sp.kind == 1) {
       TN_CUDA_TRY(launch_tc_close(L.d, L.sp, h->part, h->flags, stream));
       h->stats.tma_launches++;
@@ -488,7 +501,7 @@ tn_status run_plan(tn_handle* h, const Plan& P, int cls, size_t begin = 0,
     } else if (L.sp.maps) {
       TN_CUDA_TRY(launch_tc_stream(L.d, L.sp, h->flags, stream));
       h->stats.tma_launches++;
-    } else if (use_tensor_cores(h) && !tiny) {
+    } else if (on_tile_kernel(h, L.d)) {
       TN_CUDA_TRY(launch_cgemm_tc(L.d, h->part, h->flags, stream, &nk, L.tuned, h->part_floats));
     } else {
       // a tiny-grid launch on the main stream may split K into the partial buffer
@@ -515,8 +528,7 @@ bool side_safe(const tn_handle* h, const Plan& P, size_t begin) {
       if (L.sp.kind == 2 || (L.sp.kind == 1 && L.sp.splits > 1)) return false;
       continue;
     }
-    const double macs = (double)L.d.n_outer * L.d.n_inner * L.d.M * L.d.N * L.d.K1 * L.d.K2;
-    if (use_tensor_cores(h) && !(macs < 262144.0)) {
+    if (on_tile_kernel(h, L.d)) {
       int q = 0, sp = 1;
       size_t pf = 0;
       tc_plan(L.d, &q, &sp, &pf, L.tuned);
@@ -1245,8 +1257,7 @@ const char* kTuneNames[] = {"none", "close", "tile", "simt"};
 int tune_kind(const tn_handle* h, const HostLaunch& L) {
   if (L.skip) return TUNE_NONE;
   if (L.sp.maps) return L.sp.kind == 1 ? TUNE_CLOSE : TUNE_NONE;
-  const double macs = (double)L.d.n_outer * L.d.n_inner * L.d.M * L.d.N * L.d.K1 * L.d.K2;
-  return (use_tensor_cores(h) && !(macs < 262144.0)) ? TUNE_TILE : TUNE_SIMT;
+  return on_tile_kernel(h, L.d) ? TUNE_TILE : TUNE_SIMT;
 }
 
 // The split count a launch runs with now, and whether `s` is a valid count

@@ -48,3 +48,7 @@ def test_sweep_matches_oracle(tnlib, chi):
     o.M = {k: m.astype(np.complex64).astype(complex) for k, m in msgs.items()}
     o.bp_sweep()
     assert max(float(np.linalg.norm(got[k] - o.M[k])) for k in o.M) < 6e-6
+    # the split modes run their contractions in the same kernel
+    for prec in ("tf32x3", "bf16x3"):
+        same, z2 = one_sweep(tnlib, g, chi, tensors, msgs, prec)
+        assert all(np.array_equal(same[k], got[k]) for k in got) and np.array_equal(z, z2)
