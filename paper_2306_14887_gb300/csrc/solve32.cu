@@ -28,6 +28,7 @@
 
 #include <mutex>
 
+#include "chol_rows.cuh"
 #include "common.cuh"
 #include "tnbp.h"
 
@@ -166,10 +167,25 @@ __device__ void pivoted_cholesky32(float2* A, int m, int ld, int* perm, float re
   g.sync();
 }
 
+// Entry (i, j), i = (k, e), of G_w from the open-q environments conj(N_q^w):
+// conj(b_ki(q)) b_kj(q) = exp(s i pi/4 (s_kj - s_ki) s_q) is 1 on the diagonal
+// blocks, -s i s_q at (0, 1) and +s i s_q at (1, 0), so the off-diagonal blocks
+// are -+ s i (G_0 - G_1).
+__device__ __forceinline__ float2 gw_entry(const float* gw, int chi, int i, int j, float sg) {
+  const int64_t c2 = (int64_t)chi * chi;
+  const int ki = i / chi, ei = i % chi, kj = j / chi, ej = j % chi;
+  const int64_t o = (int64_t)ei * chi + ej;
+  const float2 g0 = make_float2(gw[o], -gw[c2 + o]);
+  const float2 g1 = make_float2(gw[2 * c2 + o], -gw[3 * c2 + o]);
+  if (ki == kj) return make_float2(g0.x + g1.x, g0.y + g1.y);
+  const float2 d = make_float2(g0.x - g1.x, g0.y - g1.y);
+  const float f = (ki == 0) ? -sg : sg;
+  return make_float2(-f * d.y, f * d.x);
+}
+
 struct Smem {
   float2* X;       // n x n: G_w -> L_w -> K^T -> rotated columns of K
   float2* Lv;      // 2 blocks chi x (chi + 1): L_0, L_1 (padded rows)
-  int* perm_w;     // n
   int* perm_v;     // 2 chi
   int* src;        // n: K^T gather map
   int* order;      // n: rows by decreasing norm
@@ -181,7 +197,7 @@ struct Smem {
   double* sig;     // n
   double* scal;    // 4
   double* red_d;   // 32
-  float2* colk;    // 2 n (one column buffer per concurrent factorisation)
+  float2* colk;    // 2 n (column buffers of the factorisations)
   float* nrm;      // n: squared row norms during the Jacobi
 };
 
@@ -196,7 +212,6 @@ __device__ Smem carve(unsigned char* base, int chi) {
   s.red_d = reinterpret_cast<double*>(p); p += sizeof(double) * 32;
   s.colk = reinterpret_cast<float2*>(p); p += sizeof(float2) * 2 * n;
   s.nrm = reinterpret_cast<float*>(p); p += sizeof(float) * n;
-  s.perm_w = reinterpret_cast<int*>(p); p += sizeof(int) * n;
   s.perm_v = reinterpret_cast<int*>(p); p += sizeof(int) * 2 * chi;
   s.src = reinterpret_cast<int*>(p); p += sizeof(int) * n;
   s.order = reinterpret_cast<int*>(p); p += sizeof(int) * n;
@@ -332,39 +347,25 @@ __global__ void __launch_bounds__(kThreads) solve32_kernel(SolveArgs a) {
           make_float2(gv[p * 2 * c2 + o], -gv[p * 2 * c2 + c2 + o]);
     }
   }
-  for (int idx = tid; idx < n * n; idx += blockDim.x) {
-    const int i = idx / n, j = idx % n;
-    const int ki = i / chi, ei = i % chi, kj = j / chi, ej = j % chi;
-    const int64_t o = (int64_t)ei * chi + ej;
-    const float2 g0 = make_float2(gw[o], -gw[c2 + o]);
-    const float2 g1 = make_float2(gw[2 * c2 + o], -gw[3 * c2 + o]);
-    float2 v;
-    if (ki == kj) {
-      v = make_float2(g0.x + g1.x, g0.y + g1.y);
-    } else {
-      // conj(b_ki(q)) b_kj(q) = exp(s i pi/4 (s_kj - s_ki) s_q): (0,1) -> -s i s_q,
-      // (1,0) -> +s i s_q, so the block is -+ s i (G_0 - G_1)
-      const float2 d = make_float2(g0.x - g1.x, g0.y - g1.y);
-      const float f = (ki == 0) ? -sg : sg;
-      v = make_float2(-f * d.y, f * d.x);
-    }
-    X[idx] = v;
-  }
+  for (int idx = tid; idx < n * n; idx += blockDim.x) X[idx] = make_float2(0.f, 0.f);
   __syncthreads();
   const float ctol = 1e-7f;
-  float2* colk = reinterpret_cast<float2*>(s.colk);
-  {
-    // the two v-side blocks concurrently on the two halves of the block, then G_w
+  if (!a.basis) {
+    // the two v-side blocks concurrently on the two halves of the block
     const int half_t = kThreads / 2;
     const int h = tid >= half_t;
     const Group gh{h * half_t, half_t, 1 + h};
-    if (!a.basis)
-      pivoted_cholesky32(s.Lv + h * chi * ldv, chi, ldv, s.perm_v + h * chi, ctol, &s.rank[h],
-                         s.red_i + h, s.red_v + h, s.dmax0 + h, colk + h * n, gh);
+    pivoted_cholesky32(s.Lv + h * chi * ldv, chi, ldv, s.perm_v + h * chi, ctol, &s.rank[h],
+                       s.red_i + h, s.red_v + h, s.dmax0 + h, s.colk + h * n, gh);
     __syncthreads();
-    const Group gall{0, kThreads, 0};
-    pivoted_cholesky32(X, n, n, s.perm_w, ctol, &s.rank[2], s.red_i, s.red_v, s.dmax0 + 2, colk,
-                       gall);
+  }
+  {
+    // G_w, its rows in registers; X receives R_w = L_w^H P_w^T as conj(L_w) with
+    // row = pivot, column = original index
+    chol::pivoted_cholesky<kMaxChi / 16, 5>(
+        n, 1, 0, s.colk, ctol, [&](int i, int j) { return gw_entry(gw, chi, i, j, sg); },
+        [&](int i, int k, float2 l) { X[k * n + i] = cconjf(l); }, nullptr);
+    __syncthreads();
   }
   if (a.basis) {
     // wait for chol64_kernel (all of its writes visible), then take its factors
@@ -383,29 +384,10 @@ __global__ void __launch_bounds__(kThreads) solve32_kernel(SolveArgs a) {
     __syncthreads();
   }
 
-  // 2. K^T = R_w R_v^T.  First X <- conj(L_w^T) so that row j of X holds
-  //    R_w[j][perm_w[t]] at column t.  Then with c = perm_b[t'] (block b):
-  //    K^T[j][(b, i)] = sum_t' X[j][pinv_w(b chi + perm_b[t'])] conj(L_b[t'][i]).
-  for (int idx = tid; idx < n * n; idx += blockDim.x) {
-    const int i = idx / n, j = idx % n;
-    if (i < j) {
-      const float2 u = X[i * n + j], l = X[j * n + i];
-      X[i * n + j] = cconjf(l);
-      X[j * n + i] = cconjf(u);
-    } else if (i == j) {
-      X[idx] = cconjf(X[idx]);
-    }
-  }
-  // src[(b, t')] = pinv_w(b chi + perm_b[t'])
-  for (int t = tid; t < n; t += blockDim.x) s.src[s.perm_w[t]] = -1 - t;  // temp: pinv_w
-  __syncthreads();
-  for (int bt = tid; bt < n; bt += blockDim.x) {
-    const int b = bt / chi, tp = bt % chi;
-    const int c = b * chi + s.perm_v[b * chi + tp];
-    s.order[bt] = -1 - s.src[c];  // pinv_w(c), staged in order[]
-  }
-  __syncthreads();
-  for (int bt = tid; bt < n; bt += blockDim.x) s.src[bt] = s.order[bt];
+  // 2. K^T = R_w R_v^T: with c = perm_b[t'] (block b),
+  //    K^T[j][(b, i)] = sum_t' R_w[j][b chi + perm_b[t']] conj(L_b[t'][i]).
+  for (int bt = tid; bt < n; bt += blockDim.x)
+    s.src[bt] = bt - bt % chi + s.perm_v[bt];
   __syncthreads();
   const int npl = n / 32 > 0 ? (n + 31) / 32 : 1;  // values per lane (<= 4)
   if (n % 32 == 0) {
@@ -892,130 +874,174 @@ __global__ void __launch_bounds__(kThreads) solve32_kernel(SolveArgs a) {
 
 // ----------------------------------------------------------------------
 // The FP32 starting basis of the refined solve for 2 chi > 128, where the
-// bond matrix no longer fits in shared memory: the same steps as basis mode of
-// solve32_kernel, with G_w, its Cholesky factor and K^T in the edge's global
-// workspace (L2-resident) and a round-robin pair order.  One CTA of
-// kGThreads threads per edge.
+// bond matrix no longer fits one SM's shared memory: the same steps as basis
+// mode of solve32_kernel in three launches, with G_w, its Cholesky factor and
+// K^T in the edge's global workspace between them and a round-robin pair order.
 constexpr int kGThreads = 512;
+constexpr int kGWarps = kGThreads / 32;
 constexpr int kGMaxN = 512;           // 2 chi <= 512 (chi <= 256)
 constexpr int kGVals = kGMaxN / 32;   // row values per lane
 
-__global__ void __launch_bounds__(kGThreads, 1) basis_gmem_kernel(SolveArgs a) {
-  __shared__ double sig[kGMaxN];
-  __shared__ int order[kGMaxN], perm_w[kGMaxN], src[kGMaxN];
-  __shared__ float2 colk[kGMaxN];
-  __shared__ int counter[4], red_i[4], rank_s[4];
-  __shared__ float red_v[4], dmax0[4];
-  __shared__ double red_d[kGThreads / 32];
-  const int chi = a.chi, n = 2 * chi, half = n / 2;
+// G_w's pivoted Cholesky factor and K^T, one cluster per edge (CV columns of
+// G_w per lane, two rows per row warp).  At chi = 128, two edges: 0.86 ms, with
+// one CTA per edge exchanging rows in global memory 5.8 ms.
+constexpr int kBThreads = kGThreads + 32;  // the Cholesky's row warps and its pivot warp
+
+template <int CV>
+__global__ void __launch_bounds__(kBThreads, 1) basis_bond_kernel(SolveArgs a, int ctas) {
+  __shared__ float2 colk[2 * kGMaxN];
+  __shared__ int src[kGMaxN];
+  const int chi = a.chi, n = 2 * chi;
   const int64_t c2 = (int64_t)chi * chi;
-  const int edge = blockIdx.x;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = kGThreads / 32;
+  const int edge = blockIdx.x / ctas;
+  const int rank = blockIdx.x - edge * ctas;
+  const int tid = threadIdx.x;
   const RefineLayout lay = refine_layout(chi);
   double* rbase = a.work + (int64_t)edge * lay.stride;
   const int* rints = reinterpret_cast<const int*>(rbase + lay.ints);
   const double2* L64 = reinterpret_cast<const double2*>(rbase + lay.L);
-  float2* Gw = reinterpret_cast<float2*>(rbase + lay.S);   // n x n: G_w, then L_w
-  float2* X = reinterpret_cast<float2*>(rbase + lay.U1);   // n x n: K^T, then its rotations
+  float2* Lw = reinterpret_cast<float2*>(rbase + lay.S);   // [original row][pivot]
+  float2* X = reinterpret_cast<float2*>(rbase + lay.U1);   // n x n: K^T
   const float* gw = a.gram + (int64_t)edge * 8 * c2 + 4 * c2;
   const float sg = (float)a.sign;
-  // 1. G_w from conj(N_q^w) with the phases of the gate split (as solve32_kernel)
-  for (int idx = tid; idx < n * n; idx += blockDim.x) {
-    const int i = idx / n, j = idx % n;
-    const int ki = i / chi, ei = i % chi, kj = j / chi, ej = j % chi;
-    const int64_t o = (int64_t)ei * chi + ej;
-    const float2 g0 = make_float2(gw[o], -gw[c2 + o]);
-    const float2 g1 = make_float2(gw[2 * c2 + o], -gw[3 * c2 + o]);
-    float2 v;
-    if (ki == kj) {
-      v = make_float2(g0.x + g1.x, g0.y + g1.y);
-    } else {
-      const float2 d = make_float2(g0.x - g1.x, g0.y - g1.y);
-      const float f = (ki == 0) ? -sg : sg;
-      v = make_float2(-f * d.y, f * d.x);
-    }
-    Gw[idx] = v;
-  }
+  for (int idx = rank * kBThreads + tid; idx < n * n; idx += ctas * kBThreads)
+    Lw[idx] = make_float2(0.f, 0.f);
+  chol::cluster_sync();
+  chol::pivoted_cholesky<CV, 2>(
+      n, ctas, rank, colk, 1e-7f, [&](int i, int j) { return gw_entry(gw, chi, i, j, sg); },
+      [&](int i, int k, float2 l) { Lw[(int64_t)i * n + k] = l; }, (int*)nullptr);
+  chol::cluster_sync();
+  // K^T[j][(b, i)] = sum_{t' >= i} conj(L_w[src(b, t')][j]) conj(L_b[t'][i]) with
+  // src(b, t') = b chi + perm_b[t'] (as solve32_kernel, R_w = L_w^H P_w^T)
+  for (int bt = tid; bt < n; bt += blockDim.x) src[bt] = bt - bt % chi + rints[bt];
   __syncthreads();
-  // 2. FP32 pivoted Cholesky of G_w in place (global memory)
-  const Group gall{0, kGThreads, 0};
-  pivoted_cholesky32(Gw, n, n, perm_w, 1e-7f, &rank_s[2], red_i, red_v, dmax0, colk, gall);
-  // 3. K^T[j][(b, i)] = sum_{t' >= i} conj(L_w[src(b, t')][j]) conj(L_b[t'][i]) with
-  //    src(b, t') = pinv_w(b chi + perm_b[t']) (as solve32_kernel, R_w = L_w^H P_w^T)
-  for (int t = tid; t < n; t += blockDim.x) order[perm_w[t]] = t;  // pinv_w
-  __syncthreads();
-  for (int bt = tid; bt < n; bt += blockDim.x) {
-    const int b = bt / chi, tp = bt % chi;
-    src[bt] = order[b * chi + rints[b * chi + tp]];
-  }
-  __syncthreads();
-  for (int idx = tid; idx < n * n; idx += blockDim.x) {
+  for (int idx = rank * kBThreads + tid; idx < n * n; idx += ctas * kBThreads) {
     const int o = idx / n, j = idx % n;   // output column (b, i) = o, row j: consecutive j per warp
     const int b = o / chi, i = o % chi;
     const double2* Lb = L64 + b * c2;
     float2 acc = make_float2(0.f, 0.f);
     for (int tp = i; tp < chi; ++tp) {
       const double2 l = Lb[(int64_t)tp * chi + i];
-      const float2 w = Gw[(int64_t)src[b * chi + tp] * n + j];
+      const float2 w = Lw[(int64_t)src[b * chi + tp] * n + j];
       // conj(w) conj(l) = conj(w l)
       const float lx = (float)l.x, ly = (float)l.y;
-      acc.x += w.x * lx - w.y * ly;
-      acc.y -= w.x * ly + w.y * lx;
+      acc.x = __fadd_rn(acc.x, chol::sum2(w.x, lx, -w.y, ly));
+      acc.y = __fsub_rn(acc.y, chol::sum2(w.x, ly, w.y, lx));
     }
     X[(int64_t)j * n + o] = acc;
   }
-  __syncthreads();
-  // 4. One-sided Jacobi on the rows of X (columns of K), round-robin pairs;
-  //    pairs orthogonal to orth_tol, or with an overlap below 1e-12 ||K||_F^2,
-  //    are left alone; a sweep that rotates nothing ends the iteration
-  {
-    double acc = 0.0;
-    for (int idx = tid; idx < n * n; idx += blockDim.x) {
+  chol::cluster_sync();
+  // ||K||_F^2 for the absolute floor of the rotations
+  if (rank != 0) return;
+  __shared__ double red_d[kGWarps];
+  double acc = 0.0;
+  if (tid < kGThreads) {
+    for (int idx = tid; idx < n * n; idx += kGThreads) {
       const float2 v = X[idx];
       acc += (double)v.x * v.x + (double)v.y * v.y;
     }
     acc = warp_sum_d(acc);
-    if (lane == 0) red_d[warp] = acc;
-    __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      for (int w = 0; w < nwarps; ++w) t += red_d[w];
-      sig[0] = t;
-    }
-    __syncthreads();
+    if ((tid & 31) == 0) red_d[tid >> 5] = acc;
   }
-  const float abs_floor = (float)(kAbsTol * sig[0]);
+  __syncthreads();
+  if (tid == 0) {
+    double t = 0.0;
+    for (int w = 0; w < kGWarps; ++w) t += red_d[w];
+    rbase[lay.misc + 2] = t;
+  }
+}
+
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+using chol::in_cta;
+using chol::sum2;
+
+// One-sided Jacobi on the rows of X (columns of K), round-robin pairs, one
+// cluster per edge.  A round's n / 2 pairs are disjoint, and from one round to
+// the next every row moves to a neighbouring pair (the circle method's fixed
+// rotation), so the rows stay in the cluster's shared memory: a warp owns one
+// pair slot, reads its two rows, rotates them and stores them into the
+// neighbouring slots, of which only the outermost lie in another CTA.  Two
+// split cluster barriers a round separate the reads from the stores that
+// replace the rows.  A round is then bound by the latency of read, dot
+// product, shuffles, rotation and barrier instead of one CTA passing every row
+// through L2.  Measured at chi = 128, two edges (ncu): 4.25 ms, where one CTA
+// per edge with the rows in L2 took about 31 ms; the same rotations bit for bit
+// (the FMA forms are written out).
+// Pairs orthogonal to orth_tol, or with an overlap below 1e-12 ||K||_F^2, are
+// left alone; a sweep that rotates nothing ends the iteration.
+__global__ void __launch_bounds__(kGThreads, 1) basis_jacobi_kernel(SolveArgs a, int ctas) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int rotated;
+  __shared__ int any_s;
+  float2* rows = reinterpret_cast<float2*>(smem_raw);  // [slot][top, bottom][n]
+  const int chi = a.chi, n = 2 * chi, half = n / 2;
+  const int edge = blockIdx.x / ctas;
+  const int rank = blockIdx.x - edge * ctas;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int per = (half + ctas - 1) / ctas;  // slots per CTA, at most one per warp
+  const RefineLayout lay = refine_layout(chi);
+  double* rbase = a.work + (int64_t)edge * lay.stride;
+  float2* X = reinterpret_cast<float2*>(rbase + lay.U1);
+  const float abs_floor = (float)(kAbsTol * rbase[lay.misc + 2]);
   const float orth_tol = a.orth_tol > 0.f ? a.orth_tol : 2e-6f;
   const int npl = n / 32;  // n is a multiple of 32 here
+  const int k = rank * per + warp;
+  const bool active = warp < per && k < half;
+  // rows of slot k in round 0, and where each goes after a round
+  const int row_t = k, row_b = k == 0 ? n - 1 : n - 1 - k;
+  float2 *mine_t = rows + (int64_t)(2 * warp) * n, *mine_b = mine_t + n;
+  float2 *to_t = mine_t, *to_b = mine_b;
+  if (active) {
+    // top: to the top of slot k - 1, from slot 0 to the bottom of slot 1;
+    // bottom: to the bottom of slot k + 1, from the last slot to its own top,
+    // and the last row stays at the bottom of slot 0
+    const int kt = k > 0 ? k - 1 : (half > 1 ? 1 : 0), st = k > 0 ? 0 : 1;
+    const int kb = k == 0 ? 0 : (k < half - 1 ? k + 1 : k), sb = k == 0 || k < half - 1 ? 1 : 0;
+    float2* lt = rows + (int64_t)(2 * (kt % per) + st) * n;
+    float2* lb = rows + (int64_t)(2 * (kb % per) + sb) * n;
+    to_t = kt / per == rank ? lt : in_cta(lt, kt / per);
+    to_b = kb / per == rank ? lb : in_cta(lb, kb / per);
+    for (int c = lane; c < n; c += 32) {
+      mine_t[c] = X[(int64_t)row_t * n + c];
+      mine_b[c] = X[(int64_t)row_b * n + c];
+    }
+  }
+  if (tid == 0) rotated = 0;
+  cluster_arrive();
+  cluster_wait();
   int sweeps = 0;
   for (int sweep = 0; sweep < a.max_sweeps; ++sweep) {
     ++sweeps;
-    if (tid == 0) counter[0] = 0;
-    __syncthreads();
+    int count = 0;
     for (int r = 0; r < n - 1; ++r) {
-      for (int k = warp; k < half; k += nwarps) {
-        int p, q;
-        if (k == 0) { p = r; q = n - 1; }
-        else { p = (r + k) % (n - 1); q = (r - k + (n - 1)) % (n - 1); }
-        float2 xp[kGVals], xq[kGVals];
-        float al = 0.f, be = 0.f, gr = 0.f, gi = 0.f;
+      float2 xp[kGVals], xq[kGVals];
+      float al = 0.f, be = 0.f, gr = 0.f, gi = 0.f;
+      if (active) {
 #pragma unroll
         for (int u = 0; u < kGVals; ++u) {
           if (u < npl) {
             const int c = u * 32 + lane;
-            xp[u] = X[(int64_t)p * n + c];
-            xq[u] = X[(int64_t)q * n + c];
-            al += xp[u].x * xp[u].x + xp[u].y * xp[u].y;
-            be += xq[u].x * xq[u].x + xq[u].y * xq[u].y;
-            gr += xp[u].x * xq[u].x + xp[u].y * xq[u].y;
-            gi += xp[u].x * xq[u].y - xp[u].y * xq[u].x;
+            xp[u] = mine_t[c];
+            xq[u] = mine_b[c];
+            al = __fadd_rn(al, sum2(xp[u].x, xp[u].x, xp[u].y, xp[u].y));
+            be = __fadd_rn(be, sum2(xq[u].x, xq[u].x, xq[u].y, xq[u].y));
+            gr = __fadd_rn(gr, sum2(xp[u].x, xq[u].x, xp[u].y, xq[u].y));
+            gi = __fadd_rn(gi, sum2(xp[u].x, xq[u].y, -xp[u].y, xq[u].x));
           }
         }
+      }
+      cluster_arrive();  // this warp's rows are in registers
+      if (active) {
         al = warp_sum(al);
         be = warp_sum(be);
         gr = warp_sum(gr);
         gi = warp_sum(gi);
-        const float gm = sqrtf(gr * gr + gi * gi);
+        const float gm = sqrtf(sum2(gr, gr, gi, gi));
         if (gm > orth_tol * sqrtf(al * be) && gm > abs_floor && gm > 0.f) {
           const float2 ph = make_float2(gr / gm, -gi / gm);  // e^{-i phi}
           const float tau = (be - al) / (2.f * gm);
@@ -1025,22 +1051,68 @@ __global__ void __launch_bounds__(kGThreads, 1) basis_gmem_kernel(SolveArgs a) {
 #pragma unroll
           for (int u = 0; u < kGVals; ++u) {
             if (u < npl) {
-              const int c = u * 32 + lane;
-              const float2 pq = cmulf(ph, xq[u]);
-              X[(int64_t)p * n + c] = make_float2(cs * xp[u].x - sn * pq.x, cs * xp[u].y - sn * pq.y);
-              X[(int64_t)q * n + c] = make_float2(sn * xp[u].x + cs * pq.x, sn * xp[u].y + cs * pq.y);
+              const float2 p = xp[u], q = xq[u];
+              const float2 pq = make_float2(sum2(ph.x, q.x, -ph.y, q.y),
+                                            sum2(ph.y, q.x, ph.x, q.y));
+              xp[u] = make_float2(sum2(cs, p.x, -sn, pq.x), sum2(cs, p.y, -sn, pq.y));
+              xq[u] = make_float2(sum2(cs, pq.x, sn, p.x), sum2(cs, pq.y, sn, p.y));
             }
           }
-          if (lane == 0) atomicAdd(&counter[0], 1);
+          ++count;
         }
       }
-      __syncthreads();
+      cluster_wait();  // every row of the cluster has been read
+      if (active) {
+#pragma unroll
+        for (int u = 0; u < kGVals; ++u) {
+          if (u < npl) {
+            const int c = u * 32 + lane;
+            to_t[c] = xp[u];
+            to_b[c] = xq[u];
+          }
+        }
+      }
+      cluster_arrive();
+      cluster_wait();  // the rows of the next round are in place
     }
-    const int rotated = counter[0];
-    __syncthreads();
-    if (rotated == 0) break;
+    // the cluster's rotations of this sweep
+    if (lane == 0 && count) atomicAdd(&rotated, count);
+    cluster_arrive();
+    cluster_wait();
+    if (tid == 0) {
+      int t = 0;
+      for (int c = 0; c < ctas; ++c) t += *in_cta(&rotated, c);
+      any_s = t;
+    }
+    cluster_arrive();
+    cluster_wait();
+    const int any = any_s;
+    if (tid == 0) rotated = 0;
+    cluster_arrive();
+    cluster_wait();
+    if (any == 0) break;
   }
-  // 5. sigma_j = ||row j|| (FP64), decreasing order, then the basis
+  // after whole sweeps every row is back in its first slot
+  if (active)
+    for (int c = lane; c < n; c += 32) {
+      X[(int64_t)row_t * n + c] = mine_t[c];
+      X[(int64_t)row_b * n + c] = mine_b[c];
+    }
+  if (rank == 0 && tid == 0) rbase[lay.misc + 3] = sweeps;
+}
+
+// sigma_j = ||row j|| (FP64), decreasing order, then the basis; one CTA per edge.
+__global__ void __launch_bounds__(kGThreads, 1) basis_out_kernel(SolveArgs a) {
+  __shared__ double sig[kGMaxN];
+  __shared__ int order[kGMaxN];
+  __shared__ int counter[4];
+  const int chi = a.chi, n = 2 * chi;
+  const int edge = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = kGWarps;
+  const RefineLayout lay = refine_layout(chi);
+  double* rbase = a.work + (int64_t)edge * lay.stride;
+  float2* X = reinterpret_cast<float2*>(rbase + lay.U1);
+  const int sweeps = (int)rbase[lay.misc + 3];
   for (int j = warp; j < n; j += nwarps) {
     double acc = 0.0;
     for (int c = lane; c < n; c += 32) {
@@ -1082,8 +1154,43 @@ bool solve32_supported(int chi) { return chi >= 1 && chi <= kMaxChi; }
 
 cudaError_t launch_basis_gmem(const SolveArgs& a, cudaStream_t st) {
   if (a.n_edges <= 0) return cudaSuccess;
-  if (a.chi < 16 || 2 * a.chi > kGMaxN || (2 * a.chi) % 32 != 0) return cudaErrorInvalidValue;
-  basis_gmem_kernel<<<a.n_edges, kGThreads, 0, st>>>(a);
+  const int n = 2 * a.chi;
+  if (a.chi < 16 || n > kGMaxN || n % 32 != 0) return cudaErrorInvalidValue;
+  // one pair slot per warp: 8 CTAs (the portable cluster size) hold n <= 256,
+  // 16 hold the rest
+  const int ctas = n <= 256 ? 8 : 16;
+  static std::once_flag once;
+  static cudaError_t attr = cudaSuccess;
+  std::call_once(once, [] {
+    attr = cudaFuncSetAttribute(basis_jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(sizeof(float2) * 2 * kGWarps * kGMaxN));
+    if (attr == cudaSuccess)
+      attr = cudaFuncSetAttribute(basis_jacobi_kernel,
+                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (attr == cudaSuccess)
+      attr = cudaFuncSetAttribute(basis_bond_kernel<16>,
+                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  });
+  if (attr != cudaSuccess) return attr;
+  const int per = (n / 2 + ctas - 1) / ctas;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(a.n_edges * ctas);
+  cfg.stream = st;
+  cudaLaunchAttribute cl[1];
+  cl[0].id = cudaLaunchAttributeClusterDimension;
+  cl[0].val.clusterDim.x = ctas;
+  cl[0].val.clusterDim.y = 1;
+  cl[0].val.clusterDim.z = 1;
+  cfg.attrs = cl;
+  cfg.numAttrs = 1;
+  cfg.blockDim = dim3(kBThreads);
+  cudaError_t e = n <= 256 ? cudaLaunchKernelEx(&cfg, basis_bond_kernel<8>, a, ctas)
+                           : cudaLaunchKernelEx(&cfg, basis_bond_kernel<16>, a, ctas);
+  if (e != cudaSuccess) return e;
+  cfg.blockDim = dim3(kGThreads);
+  cfg.dynamicSmemBytes = sizeof(float2) * 2 * (size_t)per * n;
+  if ((e = cudaLaunchKernelEx(&cfg, basis_jacobi_kernel, a, ctas)) != cudaSuccess) return e;
+  basis_out_kernel<<<a.n_edges, kGThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -49,6 +49,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "chol_rows.cuh"
 #include "common.cuh"
 #include "tnbp.h"
 
@@ -104,127 +105,75 @@ constexpr double kHead = 1e-6;
 constexpr double kNoise = 2e-6;
 
 // ------------------------------------------------------------ FP64 Cholesky
-// Pivoted Cholesky of the Hermitian PSD m x m matrix A (row stride ld, both
-// triangles stored) in place by the whole block: afterwards the first `rank`
-// columns of the lower triangle hold L with P^T A P = L L^H, perm[t] is the
-// original index of pivot t, and everything else is zero.  A pivot at or below
-// rel_tol * (largest initial diagonal) ends the factorisation.
-__device__ void pivoted_cholesky64(cd* A, int m, int ld, int* perm, double rel_tol, int* rank_out,
-                                   int* piv_s, double* pv_s, double* d0_s) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int i = tid; i < m; i += blockDim.x) perm[i] = i;
-  __syncthreads();
-  int r = m;
-  for (int k = 0; k < m; ++k) {
-    if (warp == 0) {
-      double best = -1.0;
-      int bi = k;
-      for (int i = k + lane; i < m; i += 32) {
-        const double d = A[i * ld + i].x;
-        if (d > best) { best = d; bi = i; }
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (lane == 0) {
-        *pv_s = best;
-        *piv_s = bi;
-        if (k == 0) *d0_s = best > 0.0 ? best : 0.0;
-      }
-    }
-    __syncthreads();
-    const double pv = *pv_s;
-    const int piv = *piv_s;
-    const double d0 = *d0_s;
-    if (!(d0 > 0.0) || !(pv > rel_tol * d0)) { r = k; break; }
-    if (piv != k) {
-      // symmetric exchange of rows and columns k and piv (the 2 x 2 block of
-      // the two indices by one thread afterwards)
-      for (int j = tid; j < m; j += blockDim.x) {
-        if (j == k || j == piv) continue;
-        const cd t = A[k * ld + j];
-        A[k * ld + j] = A[piv * ld + j];
-        A[piv * ld + j] = t;
-        const cd u = A[j * ld + k];
-        A[j * ld + k] = A[j * ld + piv];
-        A[j * ld + piv] = u;
-      }
-      __syncthreads();
-      if (tid == 0) {
-        const cd kk = A[k * ld + k], pp = A[piv * ld + piv];
-        const cd kp = A[k * ld + piv], pk = A[piv * ld + k];
-        A[k * ld + k] = pp;
-        A[piv * ld + piv] = kk;
-        A[k * ld + piv] = pk;
-        A[piv * ld + k] = kp;
-        const int t = perm[k];
-        perm[k] = perm[piv];
-        perm[piv] = t;
-      }
-      __syncthreads();
-    }
-    const double d = sqrt(A[k * ld + k].x);
-    const double inv = 1.0 / d;
-    for (int i = k + 1 + tid; i < m; i += blockDim.x) A[i * ld + k] = cscale(A[i * ld + k], inv);
-    __syncthreads();
-    if (tid == 0) A[k * ld + k] = {d, 0.0};
-    // trailing update of the full Hermitian block: A[i][j] -= l_i conj(l_j)
-    const int rem = m - k - 1;
-    for (int idx = tid; idx < rem * rem; idx += blockDim.x) {
-      const int i = k + 1 + idx / rem, j = k + 1 + idx % rem;
-      const cd li = A[i * ld + k], lj = A[j * ld + k];
-      cd v = A[i * ld + j];
-      v.x = fma(-li.x, lj.x, v.x);
-      v.x = fma(-li.y, lj.y, v.x);
-      v.y = fma(-li.y, lj.x, v.y);
-      v.y = fma(li.x, lj.y, v.y);
-      A[i * ld + j] = v;
-    }
-    __syncthreads();
-  }
-  for (int idx = tid; idx < m * m; idx += blockDim.x) {
-    const int i = idx / m, j = idx % m;
-    if (j > i || j >= r) A[i * ld + j] = cz();
-  }
-  if (tid == 0) *rank_out = r;
-  __syncthreads();
-}
+// Block b = blockIdx.y of edge blockIdx.z: G_b = conj(N_b^v) -> L_b, perm_b,
+// rank_b; ctas CTAs per block (one up to kSmemChi, a cluster above), CV columns
+// per lane and RW rows per row warp.  The factor is collected by original row, in
+// shared memory or in the edge's S block of the workspace, and copied to pivot
+// order at the end.
+constexpr int kCholThreads = 512 + 32;  // 16 row warps and the pivot warp
 
-// Block b = blockIdx.x of edge blockIdx.y: G_b = conj(N_b^v) -> L_b, perm_b, rank_b.
-__global__ void __launch_bounds__(kThreads) chol64_kernel(SolveArgs a) {
+template <int CV, int RW>
+__global__ void __launch_bounds__(kCholThreads, 1) chol64_kernel(SolveArgs a, int ctas) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int piv_s, rank_s;
-  __shared__ double pv_s, d0_s;
-  const int b = blockIdx.x, edge = blockIdx.y, chi = a.chi;
+  __shared__ double2 column[2 * 32 * CV];
+  __shared__ int perm_s[32 * CV];
+  const int rank = blockIdx.x, b = blockIdx.y, edge = blockIdx.z, chi = a.chi;
   const int64_t c2 = (int64_t)chi * chi;
   const float* g = a.gram + (int64_t)edge * 8 * c2 + (int64_t)b * 2 * c2;
   const RefineLayout lay = refine_layout(chi);
   double* base = a.work + (int64_t)edge * lay.stride;
   int* ints = reinterpret_cast<int*>(base + lay.ints);
-  // the factorisation runs in shared memory (padded rows) up to kSmemChi and in
-  // place in the edge's L block of the workspace above
   // the basis kernel that follows may start (its first phase does not read
   // these factors; it waits for this grid before it does)
   cudaTriggerProgrammaticLaunchCompletion();
-  const bool in_smem = chi <= kSmemChi;
-  const int ld = in_smem ? chi + 1 : chi;
-  cd* A = in_smem ? reinterpret_cast<cd*>(smem_raw)
-                  : reinterpret_cast<cd*>(base + lay.L) + (int64_t)b * c2;
-  for (int idx = threadIdx.x; idx < chi * chi; idx += blockDim.x) {
-    const int i = idx / chi, j = idx - i * chi;
-    A[i * ld + j] = {(double)g[idx], -(double)g[c2 + idx]};
+  double2* rows = ctas == 1 ? reinterpret_cast<double2*>(smem_raw)
+                            : reinterpret_cast<double2*>(base + lay.S) + (int64_t)b * c2;
+  const int first = rank * kCholThreads + threadIdx.x, step = ctas * kCholThreads;
+  for (int64_t idx = first; idx < c2; idx += step) rows[idx] = make_double2(0.0, 0.0);
+  if (ctas == 1) __syncthreads();
+  else chol::cluster_sync();
+  const int r = chol::pivoted_cholesky<CV, RW>(
+      chi, ctas, rank, column, a.gram_cut,
+      [&](int i, int j) {
+        const int64_t o = (int64_t)i * chi + j;
+        return make_double2((double)g[o], -(double)g[c2 + o]);
+      },
+      [&](int i, int k, double2 l) { rows[(int64_t)i * chi + k] = l; }, perm_s);
+  if (ctas == 1) __syncthreads();
+  else chol::cluster_sync();
+  double2* L = reinterpret_cast<double2*>(base + lay.L) + (int64_t)b * c2;
+  for (int64_t idx = first; idx < c2; idx += step) {
+    const int t = (int)(idx / chi);
+    L[idx] = rows[(int64_t)perm_s[t] * chi + (idx - (int64_t)t * chi)];
   }
-  __syncthreads();
-  pivoted_cholesky64(A, chi, ld, ints + b * chi, a.gram_cut, &rank_s, &piv_s, &pv_s, &d0_s);
-  cd* L = reinterpret_cast<cd*>(base + lay.L) + (int64_t)b * c2;
-  if (in_smem)
-    for (int idx = threadIdx.x; idx < chi * chi; idx += blockDim.x) {
-      const int i = idx / chi, j = idx - i * chi;
-      L[idx] = A[i * ld + j];
-    }
-  if (threadIdx.x == 0) ints[2 * chi + b] = rank_s;
+  if (rank == 0) {
+    for (int t = threadIdx.x; t < chi; t += kCholThreads) ints[b * chi + t] = perm_s[t];
+    if (threadIdx.x == 0) ints[2 * chi + b] = r;
+  }
+}
+
+// One CTA per block holds chi <= 64 (16 row warps x 4 rows); a cluster of 4
+// holds chi <= 128 and one of 8 chi <= 256 at two rows per warp.  Measured (ncu):
+// chi = 64, 51 edges 0.23 ms (0.27 with the block in shared memory and four
+// barriers a step); chi = 128, two edges 0.61 ms (1.82 with one CTA per block in
+// global memory).  Bound by the FP64 pipe at chi = 64 (two DFMAs a clock).
+cudaError_t launch_chol64(const SolveArgs& a, cudaStream_t st) {
+  const int ctas = a.chi <= kSmemChi ? 1 : a.chi <= 128 ? 4 : 8;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas, 2, a.n_edges);
+  cfg.blockDim = dim3(kCholThreads);
+  cfg.dynamicSmemBytes = ctas == 1 ? sizeof(double2) * (size_t)a.chi * a.chi : 0;
+  cfg.stream = st;
+  cudaLaunchAttribute cl[1];
+  cl[0].id = cudaLaunchAttributeClusterDimension;
+  cl[0].val.clusterDim.x = ctas;
+  cl[0].val.clusterDim.y = 1;
+  cl[0].val.clusterDim.z = 1;
+  cfg.attrs = cl;
+  cfg.numAttrs = ctas > 1 ? 1 : 0;
+  if (ctas == 1) return cudaLaunchKernelEx(&cfg, chol64_kernel<2, 4>, a, ctas);
+  if (ctas == 4) return cudaLaunchKernelEx(&cfg, chol64_kernel<4, 2>, a, ctas);
+  return cudaLaunchKernelEx(&cfg, chol64_kernel<8, 2>, a, ctas);
 }
 
 // ------------------------------------------------------------ refinement
@@ -713,7 +662,7 @@ __global__ void __launch_bounds__(kThreads, 2) legs_kernel(SolveArgs a, int cwma
 // Shared-memory limits of the refined solve's kernels, raised once to the
 // largest request any chi <= kMaxChi makes, so that concurrent launches (the
 // job server's slots) never lower a limit another thread relies on.
-constexpr size_t kCholSmemMax = sizeof(cd) * kSmemChi * (kSmemChi + 1);
+constexpr size_t kCholSmemMax = sizeof(double2) * kSmemChi * kSmemChi;
 constexpr size_t kRefineSmemMax = kSmemBudget + 4096;
 constexpr size_t kLegsSmemMax = kSmemBudget / 2 + 8192;
 
@@ -721,7 +670,7 @@ cudaError_t refine_prepare() {
   static std::once_flag once;
   static cudaError_t result = cudaSuccess;
   std::call_once(once, [] {
-    result = cudaFuncSetAttribute(chol64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    result = cudaFuncSetAttribute(chol64_kernel<2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)kCholSmemMax);
     if (result == cudaSuccess)
       result = cudaFuncSetAttribute(refine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -750,17 +699,14 @@ bool solve_refined_supported(int chi) {
 cudaError_t launch_solve_refined_basis(const SolveArgs& a, cudaStream_t st) {
   if (a.n_edges <= 0) return cudaSuccess;
   if (!solve_refined_supported(a.chi)) return cudaErrorInvalidValue;
-  const int chi = a.chi;
   // 1. FP64 Cholesky of the v-side Gram blocks
-  const size_t sm_chol = chi <= kSmemChi ? sizeof(cd) * (size_t)chi * (chi + 1) : 0;
   cudaError_t e = refine_prepare();
   if (e != cudaSuccess) return e;
-  chol64_kernel<<<dim3(2, a.n_edges), kThreads, sm_chol, st>>>(a);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = launch_chol64(a, st)) != cudaSuccess) return e;
   // 2. FP32 starting basis
   SolveArgs b = a;
   b.basis = 1;
-  return chi <= kSmemChi ? launch_solve32(b, st) : launch_basis_gmem(b, st);
+  return a.chi <= kSmemChi ? launch_solve32(b, st) : launch_basis_gmem(b, st);
 }
 
 cudaError_t launch_solve_refined_newton(const SolveArgs& a, cudaStream_t st) {
