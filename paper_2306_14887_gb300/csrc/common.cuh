@@ -62,6 +62,8 @@ struct GemmDesc {
   // the CUDA-core GEMM and the split-K reduce.
   const int* outer_comp;
   const double* comp_state;
+  // fused mode products only: store the output rounded to TF32 (nearest)
+  int32_t round_c;
 };
 // true when the outer entry's component has met the BP stop rule
 __device__ __forceinline__ bool outer_frozen(const GemmDesc& d, int outer) {
@@ -197,7 +199,7 @@ cudaError_t launch_bp_stop(int n_comp, double* state, unsigned long long* res,
 // Realified transposed copies of n planar complex chi x chi matrices (each at
 // src + i*src_stride): dst + i*4chi^2 holds Bt[(t,n)][(s,k)] as in GemmDesc::b_pre.
 cudaError_t launch_realify(const float* src, int64_t src_stride, float* dst, int n, int chi,
-                           cudaStream_t s);
+                           cudaStream_t s, bool tf32 = false);
 
 // TA copies of site tensors with the first leg moved last:
 // TA[pl][p][l1..l_{d-1}][l0] = T[pl][p][l0][l1..l_{d-1}] (planar).
@@ -212,6 +214,7 @@ cudaError_t launch_rho(const float* X, const float* T, const int64_t* x_off,
                        double* rho, double* part, cudaStream_t s);
 
 // Batched copy of equally sized blocks: dst[i][0..n) = src[i][0..n).
+// tf32: every value rounded to TF32 (nearest).
 cudaError_t launch_copy_blocks(float* const* dst, const float* const* src, int n_blocks,
                                int64_t n_floats, cudaStream_t s);
 

@@ -50,6 +50,7 @@ struct HostLaunch {
   TcStreamPlan sp;         // maps set: the launch runs in a TMA kernel
   bool fuse_next = false;  // the next launch contracts this one's output (chain stages)
   bool skip = false;       // carried out by the previous launch's fused kernel
+  bool cuda_cores = false; // runs in the CUDA-core GEMM whatever the precision
   int tuned = 0;           // split-K count chosen by tn_autotune (0: the heuristic)
   std::vector<int> outer_site;  // sweep launches: the site of each outer entry
 };
@@ -95,6 +96,8 @@ struct tn_handle {
   float* part = nullptr;          // K-split partials of tensor-core closes
   float* TA = nullptr;            // site tensors with the first leg moved last
   float* mrt = nullptr;           // realified transposed messages [2E][2chi][2chi]
+  float* mrt_tf32 = nullptr;      // the same rounded to TF32, for the site density matrices
+                                  // (TF32 with the fused mode products only)
   float* drt = nullptr;           // realified transposed leg matrices [slot][side][p][2chi][2chi]
   bool ta_valid = false, mrt_valid = false;
   double* work = nullptr;
@@ -345,7 +348,7 @@ tn_status upload_plans(tn_handle* h) {
       for (size_t li = 0; li < p->L.size(); ++li) {
         HostLaunch& L = p->L[li];
         TcStreamPlan sp;
-        if (L.skip) continue;
+        if (L.skip || L.cuda_cores) continue;
         // two chain stages in one pass: the intermediate never reaches HBM
         if (L.fuse_next && li + 1 < p->L.size()) {
           HostLaunch& L2 = p->L[li + 1];
@@ -501,7 +504,7 @@ tn_status run_plan(tn_handle* h, const Plan& P, int cls, size_t begin = 0,
     } else if (L.sp.maps) {
       TN_CUDA_TRY(launch_tc_stream(L.d, L.sp, h->flags, stream));
       h->stats.tma_launches++;
-    } else if (on_tile_kernel(h, L.d)) {
+    } else if (!L.cuda_cores && on_tile_kernel(h, L.d)) {
       TN_CUDA_TRY(launch_cgemm_tc(L.d, h->part, h->flags, stream, &nk, L.tuned, h->part_floats));
     } else {
       // a tiny-grid launch on the main stream may split K into the partial buffer
@@ -879,16 +882,46 @@ void build_rho_plan(tn_handle* h) {
   const HostGraph& g = h->g;
   Plan& P = h->rho_prep;
   std::vector<Ent> a, b, c;
-  // degree 3: Y1 = T x_2 M2 ; Y2 = Y1 x_1 M1 ; Y1 = Y2 x_0 M0
-  for (int v : h->sites_by_deg[3]) {
-    const auto& lg = g.legs[v];
-    a.push_back({site_ptr(h, h->T, v), in_msg(h, v, lg[2]), site_ptr(h, h->Y1, v)});
-    b.push_back({site_ptr(h, h->Y1, v), in_msg(h, v, lg[1]), site_ptr(h, h->Y2, v)});
-    c.push_back({site_ptr(h, h->Y2, v), in_msg(h, v, lg[0]), site_ptr(h, h->Y1, v)});
+  if (h->mrt_tf32) {
+    // Y2 = T x_2 M2 x_1 M1 in the fused tensor-core kernel, Y1 = Y2 x_0 M0 on
+    // the CUDA cores.  Every operand is rounded to TF32 as the tile kernel
+    // rounds it (messages and intermediates to nearest before they are
+    // stored, T by the tensor core), so the products are the same.  At chi =
+    // 64 on 127 qubits the three products took 2.0 ms as strided tile GEMMs
+    // (operands staged element by element); fused they take 0.06 ms and the
+    // third one 0.3 ms (9.7 GFLOP at the FP32 rate, the larger part now).
+    const int64_t x = chi, x2 = x * x, x3 = x2 * x, plane = 2 * x3;
+    auto m_in = [&](int v, int j) {
+      const int e = g.legs[v][j];
+      return h->mrt_tf32 + (int64_t)dir_id(g, g.other(e, v), e) * 4 * x2;
+    };
+    for (int v : h->sites_by_deg[3]) {
+      a.push_back({site_ptr(h, h->T, v), m_in(v, 2), site_ptr(h, h->Y1, v)});
+      b.push_back({site_ptr(h, h->Y1, v), m_in(v, 1), site_ptr(h, h->Y2, v)});
+      c.push_back({site_ptr(h, h->Y2, v), m_in(v, 0), site_ptr(h, h->Y1, v)});
+    }
+    // the first two as in the first degree-3 chain: Y2 at a 2x^2 + p x^2 + b' x + c'
+    add_spec(P, mode_spec(chi, plane, (int)(2 * x2), chi, 1, x2, x, 0, x2, 1, 0, x), prec, a);
+    if (!a.empty()) P.L.back().fuse_next = true;
+    add_spec(P, mode_spec(chi, plane, (int)(2 * x2), chi, chi, x3, x2, x, x2, 2 * x2, 1, x), prec, b);
+    if (!a.empty()) P.L.back().d.round_c = 1;
+    // rows (p, bc) contiguous on both sides, the contracted leg a at stride 2x^2
+    Spec sp = mode_spec(chi, plane, (int)(2 * x2), (int)x2, 1, x2, 1, 0, x3, 1, 0, x2);
+    sp.a_k2 = 2 * x2;
+    add_spec(P, sp, prec, c);
+    if (!a.empty()) P.L.back().cuda_cores = true;
+  } else {
+    // degree 3: Y1 = T x_2 M2 ; Y2 = Y1 x_1 M1 ; Y1 = Y2 x_0 M0
+    for (int v : h->sites_by_deg[3]) {
+      const auto& lg = g.legs[v];
+      a.push_back({site_ptr(h, h->T, v), in_msg(h, v, lg[2]), site_ptr(h, h->Y1, v)});
+      b.push_back({site_ptr(h, h->Y1, v), in_msg(h, v, lg[1]), site_ptr(h, h->Y2, v)});
+      c.push_back({site_ptr(h, h->Y2, v), in_msg(h, v, lg[0]), site_ptr(h, h->Y1, v)});
+    }
+    add_mode_product(P, 3, 2, chi, prec, a);
+    add_mode_product(P, 3, 1, chi, prec, b);
+    add_mode_product(P, 3, 0, chi, prec, c);
   }
-  add_mode_product(P, 3, 2, chi, prec, a);
-  add_mode_product(P, 3, 1, chi, prec, b);
-  add_mode_product(P, 3, 0, chi, prec, c);
   a.clear(); b.clear();
   // degree 2: Y1 = T x_0 M0 ; Y2 = Y1 x_1 M1 -> result in Y2, copy pointer for rho
   for (int v : h->sites_by_deg[2]) {
@@ -1391,6 +1424,11 @@ tn_status bp_converge_impl(tn_handle* h, double tol, int max_iters, int* iters, 
 }
 
 tn_status compute_rho(tn_handle* h, std::vector<double>* rho_out) {
+  if (h->mrt_tf32) {
+    TN_CUDA_TRY(launch_realify(h->msg, 2LL * h->chi * h->chi, h->mrt_tf32,
+                               2 * (int)h->g.eu.size(), h->chi, h->stream, true));
+    h->stats.kernel_launches++;
+  }
   tn_status st = run_plan(h, h->rho_prep, P_RHO);
   if (st) return st;
   const int n = h->g.n;
@@ -1453,7 +1491,18 @@ tn_status init_state(tn_handle* h) {
   return TN_OK;
 }
 
-size_t footprint_of(const HostGraph& g, int chi) {
+// The site density matrices of degree-3 sites go through the fused mode
+// products (TF32, chi = 32 or 64) from messages rounded to TF32.
+bool fused_rho(const HostGraph& g, const tn_config& cfg) {
+  if (cfg.prec != TN_TF32 || cfg.kernels != TN_KERNELS_AUTO || (cfg.chi != 32 && cfg.chi != 64))
+    return false;
+  for (int v = 0; v < g.n; ++v)
+    if (g.degree(v) == 3) return true;
+  return false;
+}
+
+size_t footprint_of(const HostGraph& g, const tn_config& cfg) {
+  const int chi = cfg.chi;
   int64_t tf = 0;
   for (int v = 0; v < g.n; ++v) tf += 4 * ipow(chi, g.degree(v));
   const int64_t c2 = (int64_t)chi * chi;
@@ -1467,6 +1516,7 @@ size_t footprint_of(const HostGraph& g, int chi) {
   b += 2 * sizeof(float) * maxl * 8 * c2;                  // gram, dmat
   b += sizeof(double) * maxl * solve_work_doubles(chi);    // work
   b += sizeof(double) * g.eu.size() * (size_t)chi;        // bond spectra
+  if (fused_rho(g, cfg)) b += sizeof(float) * (size_t)(2 * g.eu.size()) * 4 * c2;  // rounded messages
   return b;
 }
 
@@ -1512,7 +1562,7 @@ tn_status tn_footprint_estimate(const tn_graph* graph, const tn_config* cfg, siz
     set_error(why);
     return TN_EINVAL;
   }
-  *out = footprint_of(g, cfg->chi);
+  *out = footprint_of(g, *cfg);
   return TN_OK;
 }
 
@@ -1592,6 +1642,15 @@ tn_status tn_create(const tn_graph* graph, const tn_config* cfg, const tn_alloca
   h->Y2 = (float*)dev_alloc(h, sizeof(float) * off);
   h->TA = (float*)dev_alloc(h, sizeof(float) * off);
   h->mrt = (float*)dev_alloc(h, sizeof(float) * nmsg * 4 * c2);
+  if (fused_rho(g, *cfg)) {
+    h->mrt_tf32 = (float*)dev_alloc(h, sizeof(float) * nmsg * 4 * c2);
+    if (!h->mrt_tf32) {
+      set_error("device allocation failed");
+      dev_free_all(h);
+      delete h;
+      return TN_ENOMEM;
+    }
+  }
   h->msg = (float*)dev_alloc(h, sizeof(float) * nmsg * 2 * c2);
   h->raw = (float*)dev_alloc(h, sizeof(float) * nmsg * 2 * c2);
   h->gram = (float*)dev_alloc(h, sizeof(float) * h->max_layer * 8 * c2);
@@ -1661,7 +1720,7 @@ tn_status tn_create(const tn_graph* graph, const tn_config* cfg, const tn_alloca
       !h->comp_of_msg || !h->comp_state || !h->comp_res || !h->loop_par || !h->loop_out ||
       !h->rx_cs ||
       !h->spectra) {
-    set_error("device allocation failed (footprint " + std::to_string(footprint_of(g, chi)) +
+    set_error("device allocation failed (footprint " + std::to_string(footprint_of(g, *cfg)) +
               " bytes)");
     return fail(TN_ENOMEM);
   }

@@ -5,6 +5,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "tc_common.cuh"
 #include "tnbp.h"
 
 namespace tnbp {
@@ -367,6 +368,7 @@ __global__ void dot_msgs_kernel(const float* R, const float* M, int chi, double*
 }
 
 // Realified transposed copies (see GemmDesc::b_pre).
+template <bool TF32>
 __global__ void realify_kernel(const float* src, int64_t stride, float* dst, int chi) {
   const int64_t n2 = (int64_t)chi * chi;
   const float* a = src + blockIdx.y * stride;
@@ -375,7 +377,11 @@ __global__ void realify_kernel(const float* src, int64_t stride, float* dst, int
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n2;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(idx / chi), j = (int)(idx - (int64_t)i * chi);  // element [k = i][n = j]
-    const float re = a[idx], im = a[n2 + idx];
+    float re = a[idx], im = a[n2 + idx];
+    if (TF32) {
+      re = __uint_as_float(tc::to_tf32(re));
+      im = __uint_as_float(tc::to_tf32(im));
+    }
     q[(int64_t)j * w + i] = re;
     q[(int64_t)(chi + j) * w + chi + i] = re;
     q[(int64_t)(chi + j) * w + i] = im;
@@ -451,13 +457,14 @@ cudaError_t launch_dot_msgs(const float* R, const float* M, int chi, double* out
 }
 
 cudaError_t launch_realify(const float* src, int64_t src_stride, float* dst, int n, int chi,
-                           cudaStream_t s) {
+                           cudaStream_t s, bool tf32) {
   if (n <= 0) return cudaSuccess;
   const int64_t n2 = (int64_t)chi * chi;
   int64_t bx = (n2 + 255) / 256;
   if (bx > 64) bx = 64;
   dim3 grid((unsigned)bx, n);
-  realify_kernel<<<grid, 256, 0, s>>>(src, src_stride, dst, chi);
+  if (tf32) realify_kernel<true><<<grid, 256, 0, s>>>(src, src_stride, dst, chi);
+  else realify_kernel<false><<<grid, 256, 0, s>>>(src, src_stride, dst, chi);
   return cudaGetLastError();
 }
 

@@ -751,7 +751,8 @@ __global__ void __launch_bounds__(kFThreads, 1) tc_chain_kernel(GemmDesc d, Fuse
         tmem_ld32(lane_base + (uint32_t)(4 * CHI + h * CHI + cc * 32), v);
         float* Cc = C + cc * 32 * CHI;  // columns n2 = cc * 32 + jj at stride CHI
 #pragma unroll
-        for (int jj = 0; jj < 32; ++jj) Cc[jj * CHI] = v[jj];
+        for (int jj = 0; jj < 32; ++jj)
+          Cc[jj * CHI] = d.round_c ? __uint_as_float(to_tf32(v[jj])) : v[jj];
       }
       tc_fence_before();
       __syncwarp();
