@@ -99,6 +99,22 @@ int cgemm_plan(const GemmDesc& d, size_t* part_floats, int force_splits = 0);
 cudaError_t simt_prepare();  // kernel attributes, once, before any stream capture
 cudaError_t launch_cgemm(const GemmDesc& d, cudaStream_t s, float* part = nullptr,
                          size_t part_cap = 0, int* n_kernels = nullptr, int force_splits = 0);
+// One site's chain to one open leg (site_sweep.cu): the message contractions of
+// a BP sweep at chi <= 16 in one launch, FP32, the same sums as the CUDA-core
+// GEMM.  Degree 3: open-leg values o0 .. o0 + on - 1 (at most
+// site_sweep_open(chi)); mf, mg the incoming messages (planar chi x chi) on the
+// first and second contracted legs.  splits: the split-K counts of the three
+// degree-3 closes; comp_state: as in GemmDesc (null: no skipping).
+struct SiteJob {
+  const float *T, *mf, *mg;
+  float* out;
+  int32_t deg, open, o0, on, comp, pad;
+};
+bool site_sweep_supported(int chi);
+int site_sweep_open(int chi);
+cudaError_t site_sweep_prepare();
+cudaError_t launch_site_sweep(const SiteJob* jobs, int n_jobs, int chi, const int splits[3],
+                              const double* comp_state, cudaStream_t s);
 // Tensor-core version (tc_gemm.cu) for TN_TF32 / TN_BF16 descriptors.  part:
 // scratch for K-split partial products (tc_plan gives the size, part_cap the
 // floats the caller holds: a plan that needs more is refused); err: bit 1 is
@@ -198,6 +214,7 @@ cudaError_t launch_bp_stop(int n_comp, double* state, unsigned long long* res,
 
 // Realified transposed copies of n planar complex chi x chi matrices (each at
 // src + i*src_stride): dst + i*4chi^2 holds Bt[(t,n)][(s,k)] as in GemmDesc::b_pre.
+// tf32: every value rounded to TF32 (nearest).
 cudaError_t launch_realify(const float* src, int64_t src_stride, float* dst, int n, int chi,
                            cudaStream_t s, bool tf32 = false);
 
@@ -214,7 +231,6 @@ cudaError_t launch_rho(const float* X, const float* T, const int64_t* x_off,
                        double* rho, double* part, cudaStream_t s);
 
 // Batched copy of equally sized blocks: dst[i][0..n) = src[i][0..n).
-// tf32: every value rounded to TF32 (nearest).
 cudaError_t launch_copy_blocks(float* const* dst, const float* const* src, int n_blocks,
                                int64_t n_floats, cudaStream_t s);
 

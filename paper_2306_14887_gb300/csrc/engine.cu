@@ -134,6 +134,10 @@ struct tn_handle {
   // degree-2 chains and degree-1 closes, which share no scratch with the
   // degree-3 chains) runs beside sweep.L[..sweep_split].
   size_t sweep_split = 0;
+  // chi <= 16 on the CUDA cores: the sweep's contractions as one launch (one job
+  // per site, open leg and block of open-leg values) instead of sweep.L
+  tnbp::SiteJob* site_jobs = nullptr;
+  int n_site_jobs = 0;
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 
@@ -774,6 +778,71 @@ void build_sweep_plan(tn_handle* h) {
   tag(from, h->sites_by_deg[1]);
 }
 
+// Whether every contraction of the handle runs on the CUDA cores (FP32, and the
+// split modes, see on_tile_kernel).
+bool cuda_core_mode(const tn_config& c) {
+  return c.prec == TN_FP32 ||
+         (c.kernels == TN_KERNELS_AUTO && (c.prec == TN_TF32X3 || c.prec == TN_BF16X3));
+}
+
+// The sweep as one launch (site_sweep.cu): the degree-3 chains first, the
+// longest jobs.  Legs contracted in the order of the chains above.
+tn_status build_site_jobs(tn_handle* h) {
+  if (!cuda_core_mode(h->cfg) || !site_sweep_supported(h->chi)) return TN_OK;
+  const HostGraph& g = h->g;
+  std::vector<SiteJob> jobs;
+  for (int d = 3; d >= 1; --d)
+    for (int v : h->sites_by_deg[d])
+      for (int j = 0; j < d; ++j) {
+        SiteJob q{};
+        q.T = site_ptr(h, h->T, v);
+        q.out = (float*)msg_ptr(h, h->raw, dir_id(g, v, g.legs[v][j]));
+        q.deg = d;
+        q.open = j;
+        q.comp = h->comp_of_vertex[v];
+        if (d == 3) {
+          q.mf = in_msg(h, v, g.legs[v][j == 2 ? 0 : 2]);
+          q.mg = in_msg(h, v, g.legs[v][j == 1 ? 0 : 1]);
+        } else if (d == 2) {
+          q.mf = in_msg(h, v, g.legs[v][1 - j]);
+        }
+        const int step = d == 3 ? site_sweep_open(h->chi) : h->chi;
+        for (int o = 0; o < h->chi; o += step) {
+          q.o0 = o;
+          q.on = std::min(step, h->chi - o);
+          jobs.push_back(q);
+        }
+      }
+  if (jobs.empty()) return TN_OK;
+  h->site_jobs = (SiteJob*)dev_alloc(h, sizeof(SiteJob) * jobs.size());
+  if (!h->site_jobs) { set_error("device allocation of the sweep jobs failed"); return TN_ENOMEM; }
+  if (cudaMemcpy(h->site_jobs, jobs.data(), sizeof(SiteJob) * jobs.size(),
+                 cudaMemcpyHostToDevice) != cudaSuccess ||
+      site_sweep_prepare() != cudaSuccess) {
+    set_error("preparing the sweep jobs failed");
+    return TN_ECUDA;
+  }
+  h->n_site_jobs = (int)jobs.size();
+  return TN_OK;
+}
+
+// The sweep's contractions at small chi, with the split-K counts the plan's
+// degree-3 closes (every third launch) have.
+tn_status run_site_sweep(tn_handle* h) {
+  int splits[3] = {1, 1, 1};
+  if (!h->sites_by_deg[3].empty())
+    for (int j = 0; j < 3; ++j) {
+      const HostLaunch& L = h->sweep.L[3 * j + 2];
+      size_t pf = 0;
+      const int s = cgemm_plan(L.d, &pf, L.tuned);
+      splits[j] = pf > h->part_floats ? 1 : s;
+    }
+  TN_CUDA_TRY(launch_site_sweep(h->site_jobs, h->n_site_jobs, h->chi, splits,
+                                h->n_comp > 1 ? h->comp_state : nullptr, h->stream));
+  h->stats.kernel_launches++;
+  return TN_OK;
+}
+
 // A union of several components: every sweep launch gets the component of
 // each of its outer entries, so that the kernels that honour it skip the
 // components that have met the stop rule.
@@ -1163,7 +1232,12 @@ tn_status gate_layer(tn_handle* h, int li, int sign) {
 tn_status enqueue_sweep(tn_handle* h, bool fork, bool in_loop, cudaGraphConditionalHandle cond = 0) {
   const int nmsg = 2 * (int)h->g.eu.size();
   tn_status st;
-  if (fork) {
+  if (h->n_site_jobs) {
+    const int pb = prof_begin(h, P_BP);
+    st = run_site_sweep(h);
+    if (st) return st;
+    prof_end(h, pb, h->sweep_flops, h->sweep_bytes);
+  } else if (fork) {
     // degree-2 and degree-1 launches on the side stream, beside the degree-3 chains
     TN_CUDA_TRY(cudaEventRecord(h->ev_fork, h->stream));
     TN_CUDA_TRY(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
@@ -1205,7 +1279,7 @@ tn_status loop_graph(tn_handle* h, bool* use) {
     if (!h->stream || h->loop_unavailable) return TN_OK;  // the legacy default stream cannot be captured
     const bool prof = h->prof_on;
     h->prof_on = false;
-    bool fork = h->sweep_split > 0 && h->sweep_split < h->sweep.L.size() &&
+    bool fork = !h->n_site_jobs && h->sweep_split > 0 && h->sweep_split < h->sweep.L.size() &&
                 side_safe(h, h->sweep, h->sweep_split);
     if (fork && !h->side) {
       if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
@@ -1361,7 +1435,7 @@ tn_status bp_converge_impl(tn_handle* h, double tol, int max_iters, int* iters, 
   // exactly the sweeps it would receive alone.
   const double floor = precision_floor(h);
   {
-    tn_status st0 = ensure_ta(h);
+    tn_status st0 = h->n_site_jobs ? TN_OK : ensure_ta(h);
     if (st0) return st0;
     st0 = ensure_mrt(h);
     if (st0) return st0;
@@ -1800,6 +1874,8 @@ tn_status tn_create(const tn_graph* graph, const tn_config* cfg, const tn_alloca
     if (!h->part) { delete[] h->h_stats; set_error("device allocation failed"); return fail(TN_ENOMEM); }
   }
   tn_status st = upload_plans(h);
+  if (st) { delete[] h->h_stats; return fail(st); }
+  st = build_site_jobs(h);
   if (st) { delete[] h->h_stats; return fail(st); }
   st = attach_components(h);
   if (st) { delete[] h->h_stats; return fail(st); }

@@ -52,3 +52,26 @@ def test_sweep_matches_oracle(tnlib, chi):
     for prec in ("tf32x3", "bf16x3"):
         same, z2 = one_sweep(tnlib, g, chi, tensors, msgs, prec)
         assert all(np.array_equal(same[k], got[k]) for k in got) and np.array_equal(z, z2)
+
+
+@pytest.mark.parametrize("chi", [1, 2, 3, 7, 8, 9, 13, 16])
+def test_small_chi_sweep_in_a_union(tnlib, chi):
+    """At chi <= 16 a sweep's contractions run as one launch over (site, open leg,
+    open-leg block) jobs: every message is the same bit for bit alone and as one
+    of three components."""
+    g = OG.star3_tree()
+    tensors, msgs = random_state([g.degree(v) for v in range(g.n)], g.edges, chi, seed=100 + chi)
+    alone, _ = one_sweep(tnlib, g, chi, tensors, msgs, "fp32")
+    n, e, c, offs = tnlib.batch_union([(g.n, g.edges, g.colours)] * 3)
+    with tnlib.TNState(n, e, c, chi=chi) as s:
+        for off in offs:
+            for v in range(g.n):
+                s.set_site(off + v, tensors[v])
+        for i, off in enumerate(offs):
+            for (src, ed), m in msgs.items():
+                s.set_message(i * len(g.edges) + ed, off + src, m)
+        s.bp_converge(tol=1e30, max_iters=1)
+        for i, off in enumerate(offs):
+            for src, ed in msgs:
+                got = s.get_message(i * len(g.edges) + ed, off + src)
+                assert np.array_equal(got, alone[(src, ed)])
