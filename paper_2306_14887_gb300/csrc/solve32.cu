@@ -654,13 +654,12 @@ __global__ void __launch_bounds__(kThreads) solve32_kernel(SolveArgs a) {
   } else
   for (int sweep = 0; sweep < a.max_sweeps; ++sweep) {
     ++sweeps;
-    if (tid == 0) s.counter[0] = 0;
-    __syncthreads();
+    int rotated = 0;
     for (int r = 0; r < n - 1; ++r) {
       for (int k = warp; k < half; k += kWarps) {
-        int p, q;
-        if (k == 0) { p = r; q = n - 1; }
-        else { p = (r + k) % (n - 1); q = (r - k + (n - 1)) % (n - 1); }
+        // rows (r + k) and (r - k) mod n - 1; slot 0 pairs row r with the last row
+        const int p = r + k < n - 1 ? r + k : r + k - (n - 1);
+        const int q = k == 0 ? n - 1 : r >= k ? r - k : r - k + (n - 1);
         float2 xp[4], xq[4];
         float al = 0.f, be = 0.f, gr = 0.f, gi = 0.f;
 #pragma unroll
@@ -702,13 +701,12 @@ __global__ void __launch_bounds__(kThreads) solve32_kernel(SolveArgs a) {
               X[q * n + c] = make_float2(sn * xp[u].x + cs * pq.x, sn * xp[u].y + cs * pq.y);
             }
           }
-          if (lane == 0) atomicAdd(s.counter, 1);
+          rotated = 1;
         }
       }
       __syncthreads();
     }
-    if (s.counter[0] == 0) break;
-    __syncthreads();
+    if (!__syncthreads_or(rotated)) break;
   }
 
   // 4. sigma_j = ||row j|| (FP64), order by decreasing sigma, truncate, normalise.

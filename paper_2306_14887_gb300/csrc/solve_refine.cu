@@ -81,7 +81,6 @@ __device__ __forceinline__ cd shfl_xor(cd v, int o) {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kJG = 8;              // output columns accumulated together per warp row
 constexpr int kJU = 4;              // output columns per thread in the basis update
 constexpr int kSmemChi = 64;   // up to here the FP32 basis and the FP64 Cholesky run in
                                // shared memory; above, in the edge's global workspace
@@ -211,49 +210,77 @@ __device__ EdgeView edge_view(const SolveArgs& a, int edge) {
 }
 
 // out(i, j) = sum_{r in [lo(i), hi(i))} arow(i, r) * B[j * ldb + bidx(i, r)]
-// for the rows i < nrows and the cw columns j of B; store(i, j, value).  Each
-// row is taken by 8 lanes (4 rows per warp), each lane summing every 8th r in
-// FP64 for kJG columns at a time; the 8 partial sums are then combined in a
-// fixed order (3 shuffle levels) and lane jj of the row's group stores
-// column jj.
-template <class RF, class AF, class BF, class SF>
-__device__ void rows8(int nrows, int cw, const cd* B, int ldb, RF range, AF arow, BF bidx,
-                      SF store) {
+// for the rows i < nrows and the columns j0 .. j0 + J - 1 of B; store(i, j,
+// value).  Bound by the FP64 pipe (two lanes a clock: a warp's instruction takes
+// it for 16 clocks whatever its active lanes), so the split keeps the FP64
+// instructions few: a row is taken by L lanes, the fewest that still give every
+// warp rows, whose partial sums need log2(L) additions per column at the end;
+// four of a lane's operands are loaded ahead.
+template <int L, int J, class RF, class AF, class BF, class SF>
+__device__ __forceinline__ void rows_block(int nrows, int j0, const cd* B, int ldb, RF range,
+                                           AF arow, BF bidx, SF store) {
+  constexpr int kAhead = 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int sub = lane & 7;
-  for (int i0 = warp * 4; i0 < nrows; i0 += kWarps * 4) {
-    const int i = i0 + (lane >> 3);
+  const int sub = lane & (L - 1);
+  for (int i0 = warp * (32 / L); i0 < nrows; i0 += kWarps * (32 / L)) {
+    const int i = i0 + lane / L;
     int lo = 0, hi = 0;
     if (i < nrows) range(i, lo, hi);
-    for (int j0 = 0; j0 < cw; j0 += kJG) {
-      cd acc[kJG];
+    cd acc[J];
 #pragma unroll
-      for (int jj = 0; jj < kJG; ++jj) acc[jj] = cz();
-      const int nj = min(kJG, cw - j0);
-      for (int r = lo + sub; r < hi; r += 8) {
-        const cd av = arow(i, r);
-        const cd* bp = B + (int64_t)j0 * ldb + bidx(i, r);
-        if (nj == kJG) {
+    for (int jj = 0; jj < J; ++jj) acc[jj] = cz();
+    const cd* bj = B + (int64_t)j0 * ldb;
+    int r = lo + sub;
+    for (; r + (kAhead - 1) * L < hi; r += kAhead * L) {
+      cd av[kAhead];
 #pragma unroll
-          for (int jj = 0; jj < kJG; ++jj) cfma(acc[jj], av, bp[jj * ldb]);
-        } else {
+      for (int u = 0; u < kAhead; ++u) av[u] = arow(i, r + u * L);
 #pragma unroll
-          for (int jj = 0; jj < kJG; ++jj)
-            if (jj < nj) cfma(acc[jj], av, bp[jj * ldb]);
-        }
+      for (int u = 0; u < kAhead; ++u) {
+        const cd* bp = bj + bidx(i, r + u * L);
+#pragma unroll
+        for (int jj = 0; jj < J; ++jj) cfma(acc[jj], av[u], bp[jj * ldb]);
       }
+    }
+    for (; r < hi; r += L) {
+      const cd av = arow(i, r);
+      const cd* bp = bj + bidx(i, r);
 #pragma unroll
-      for (int jj = 0; jj < kJG; ++jj) {
+      for (int jj = 0; jj < J; ++jj) cfma(acc[jj], av, bp[jj * ldb]);
+    }
+    __syncwarp();
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) acc[jj] = cadd(acc[jj], shfl_xor(acc[jj], o));
-      }
-      cd mine = cz();
+    for (int jj = 0; jj < J; ++jj) {
 #pragma unroll
-      for (int jj = 0; jj < kJG; ++jj)
-        if (sub == jj) mine = acc[jj];
-      if (i < nrows && sub < nj) store(i, j0 + sub, mine);
+      for (int o = L / 2; o > 0; o >>= 1) acc[jj] = cadd(acc[jj], shfl_xor(acc[jj], o));
+      if (i < nrows && sub == (jj & (L - 1))) store(i, j0 + jj, acc[jj]);
     }
   }
+}
+
+// All cw columns, eight at a time and the rest in smaller groups.
+template <int L, class RF, class AF, class BF, class SF>
+__device__ void rows_cols(int nrows, int cw, const cd* B, int ldb, RF range, AF arow, BF bidx,
+                          SF store) {
+  int j = 0;
+  for (; j + 8 <= cw; j += 8) rows_block<L, 8>(nrows, j, B, ldb, range, arow, bidx, store);
+  if (j + 4 <= cw) {
+    rows_block<L, 4>(nrows, j, B, ldb, range, arow, bidx, store);
+    j += 4;
+  }
+  if (j + 2 <= cw) {
+    rows_block<L, 2>(nrows, j, B, ldb, range, arow, bidx, store);
+    j += 2;
+  }
+  if (j < cw) rows_block<L, 1>(nrows, j, B, ldb, range, arow, bidx, store);
+}
+
+// Lanes per row: eight warps hold 256 / L rows at once.
+template <class RF, class AF, class BF, class SF>
+__device__ void row_products(int nrows, int cw, const cd* B, int ldb, RF range, AF arow, BF bidx,
+                      SF store) {
+  if (nrows > 64) rows_cols<2>(nrows, cw, B, ldb, range, arow, bidx, store);
+  else rows_cols<8>(nrows, cw, B, ldb, range, arow, bidx, store);
 }
 
 // One Newton step for the kept columns [j0, j1) of one edge.  Shared-memory
@@ -274,7 +301,7 @@ __device__ void refine_chunk(const SolveArgs& a, const EdgeView& v, int j0, int 
   for (int idx = tid; idx < cw * n; idx += blockDim.x) Uc[idx] = v.U[(int64_t)j0 * n + idx];
   __syncthreads();
   // Y = R_v^H U_c: Y[(k, perm_k[s])] = sum_{t <= s, t < rank_k} L_k[s][t] U[(k, t)]
-  rows8(
+  row_products(
       n, cw, Uc, n,
       [&](int i, int& lo, int& hi) {
         const int k = i / chi, s = i - k * chi;
@@ -309,7 +336,7 @@ __device__ void refine_chunk(const SolveArgs& a, const EdgeView& v, int j0, int 
     B3[j * n + i] = {mine.x - sg * other.y, mine.y + sg * other.x};
   }
   __syncthreads();
-  rows8(
+  row_products(
       n, cw, B3, n, [&](int, int& lo, int& hi) { lo = 0; hi = chi; },
       [&](int i, int r) {
         const int q = i / chi, e = i - q * chi;
@@ -329,7 +356,7 @@ __device__ void refine_chunk(const SolveArgs& a, const EdgeView& v, int j0, int 
   }
   __syncthreads();
   // P = R_v Z: P[(b, t)] = sum_{s >= t} conj(L_b[s][t]) Z[(b, perm_b[s])], zero for t >= rank_b
-  rows8(
+  row_products(
       n, cw, B3, n,
       [&](int i, int& lo, int& hi) {
         const int b = i / chi, t = i - b * chi;
@@ -347,11 +374,11 @@ __device__ void refine_chunk(const SolveArgs& a, const EdgeView& v, int j0, int 
       [&](int i, int j, cd val) { B1[j * n + i] = val; });
   __syncthreads();
   // S = U_A^H P and R = I - U_A^H U_c
-  rows8(
+  row_products(
       A, cw, B1, n, [&](int, int& lo, int& hi) { lo = 0; hi = n; },
       [&](int i, int r) { return cconj(v.U[(int64_t)i * n + r]); }, [&](int, int r) { return r; },
       [&](int i, int j, cd val) { B2[j * n + i] = val; });
-  rows8(
+  row_products(
       A, cw, Uc, n, [&](int, int& lo, int& hi) { lo = 0; hi = n; },
       [&](int i, int r) { return cconj(v.U[(int64_t)i * n + r]); }, [&](int, int r) { return r; },
       [&](int i, int j, cd val) {
@@ -437,11 +464,17 @@ __device__ void refine_chunk(const SolveArgs& a, const EdgeView& v, int j0, int 
 #pragma unroll
     for (int jj = 0; jj < kJU; ++jj) acc[jj] = cz();
     const int nj = min(kJU, cw - jb);
-    for (int i = 0; i < A; ++i) {
-      const cd u = v.U[(int64_t)i * n + r];
+    for (int i0 = 0; i0 < A; i0 += 8) {
+      cd u[8];
 #pragma unroll
-      for (int jj = 0; jj < kJU; ++jj)
-        if (jj < nj) cfma(acc[jj], u, B2[(jb + jj) * n + i]);
+      for (int t = 0; t < 8; ++t) u[t] = i0 + t < A ? v.U[(int64_t)(i0 + t) * n + r] : cz();
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        if (i0 + t >= A) break;
+#pragma unroll
+        for (int jj = 0; jj < kJU; ++jj)
+          if (jj < nj) cfma(acc[jj], u[t], B2[(jb + jj) * n + i0 + t]);
+      }
     }
 #pragma unroll
     for (int jj = 0; jj < kJU; ++jj) {
@@ -458,6 +491,9 @@ __device__ void refine_chunk(const SolveArgs& a, const EdgeView& v, int j0, int 
   __syncthreads();
 }
 
+// Bound by the FP64 pipe.  Measured (ncu): chi = 64, 51 edges 1.78 ms (2.21 with
+// eight lanes on every row and every group of eight columns reduced whole);
+// chi = 37, 24 edges 0.24 ms (0.42); chi = 21, 7 edges 63 us (101).
 // The kept-column slots of all edges, ne * chi, split evenly over the grid: each
 // block takes a contiguous range (split further at edge boundaries and into
 // pieces of at most cwmax columns).
@@ -492,6 +528,9 @@ __global__ void __launch_bounds__(kThreads, 1) refine_kernel(SolveArgs a, int cw
 // then D_v[b][perm_b[s]][pos] = W[(b, s)] sqrt(sigma / ||sigma||) and
 // D_w[q][e][pos] = sum_b b_b(q) conj(Y[(b, pinv_b(e))]) / sqrt(sigma ||sigma||)
 // with b_b(q) = exp(s i pi/4 s_b s_q), as the gate split gives.
+// Measured (ncu): chi = 64, 51 edges 0.53 ms (0.56 with the substitution over the
+// whole block, two barriers a step), chi = 37, 24 edges 0.15 ms (0.21), chi = 21,
+// 7 edges 47 us (59).
 __global__ void __launch_bounds__(kThreads, 2) legs_kernel(SolveArgs a, int cwmax) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int chi = a.chi, n = 2 * chi;
@@ -568,7 +607,7 @@ __global__ void __launch_bounds__(kThreads, 2) legs_kernel(SolveArgs a, int cwma
       }
       __syncthreads();
       // Y = L_b u_b (from the unmodified columns) first
-      rows8(
+      row_products(
           n, cw, Ub, n,
           [&](int i, int& lo, int& hi) {
             const int b = i / chi, t = i - b * chi;
@@ -584,33 +623,58 @@ __global__ void __launch_bounds__(kThreads, 2) legs_kernel(SolveArgs a, int cwma
       __syncthreads();
       // W: solve L_b^H w = u_b for every column of the chunk by back
       // substitution over s = rank_b - 1 .. 0, in place in Ub: w[s] = u[s] /
-      // L[s][s], then u[t] -= conj(L[s][t]) w[s] for t < s (both blocks and all
-      // columns at once, one pass per s)
-      const int rmax = max(v.rank[0], v.rank[1]);
-      for (int sidx = rmax - 1; sidx >= 0; --sidx) {
-        for (int idx = tid; idx < 2 * cw; idx += blockDim.x) {
-          const int b = idx / cw, jj = idx - b * cw;
-          if (sidx < v.rank[b]) {
-            const cd d = v.L[b * c2 + (int64_t)sidx * chi + sidx];
-            Ub[jj * n + b * chi + sidx] = cscale(Ub[jj * n + b * chi + sidx], 1.0 / d.x);
+      // L[s][s], then u[t] -= conj(L[s][t]) w[s] for t < s.  One warp per
+      // (column, block) holds the column in registers (lane t % 32) and passes
+      // w[s] on by shuffle, so that a step waits for no other warp; the next
+      // row of L is loaded ahead.
+      for (int task = tid >> 5; task < 2 * cw; task += kWarps) {
+        const int b = task & 1, jj = task >> 1, lane = tid & 31;
+        cd* uc = Ub + jj * n + b * chi;
+        const cd* Lb = v.L + b * c2;
+        for (int base = (v.rank[b] - 1) / 32 * 32; base >= 0 && v.rank[b] > 0; base -= 32) {
+          // the triangle of columns base .. base + 31, then the rows above it
+          const int t = base + lane;
+          cd u = t < v.rank[b] ? uc[t] : cz();
+          const int last = min(v.rank[b], base + 32) - 1;
+          const double inv = t <= last ? 1.0 / Lb[(int64_t)t * chi + t].x : 0.0;
+          cd row = cz();
+          if (t <= last) row = Lb[(int64_t)last * chi + t];
+          for (int sidx = last; sidx >= base; --sidx) {
+            cd next = cz();
+            if (sidx > base && t < sidx) next = Lb[(int64_t)(sidx - 1) * chi + t];
+            const double is = __shfl_sync(0xffffffffu, inv, sidx & 31);
+            cd w = {__shfl_sync(0xffffffffu, u.x, sidx & 31),
+                    __shfl_sync(0xffffffffu, u.y, sidx & 31)};
+            w = cscale(w, is);
+            if (t == sidx) {
+              u = w;
+            } else if (t < sidx) {
+              const cd l = cconj(row);
+              u.x = fma(-l.x, w.x, u.x);
+              u.x = fma(l.y, w.y, u.x);
+              u.y = fma(-l.x, w.y, u.y);
+              u.y = fma(-l.y, w.x, u.y);
+            }
+            row = next;
           }
-        }
-        __syncthreads();
-        for (int idx = tid; idx < 2 * cw * sidx; idx += blockDim.x) {
-          const int b = idx / (cw * sidx), rem = idx - b * cw * sidx;
-          const int jj = rem / sidx, t = rem - jj * sidx;
-          if (sidx < v.rank[b]) {
-            const cd l = cconj(v.L[b * c2 + (int64_t)sidx * chi + t]);
-            const cd w = Ub[jj * n + b * chi + sidx];
-            cd& u = Ub[jj * n + b * chi + t];
-            u.x = fma(-l.x, w.x, u.x);
-            u.x = fma(l.y, w.y, u.x);
-            u.y = fma(-l.x, w.y, u.y);
-            u.y = fma(-l.y, w.x, u.y);
+          if (t <= last) uc[t] = u;
+          __syncwarp();
+          for (int t2 = lane; t2 < base; t2 += 32) {
+            cd x = uc[t2];
+            for (int sidx = last; sidx >= base; --sidx) {
+              const cd l = cconj(Lb[(int64_t)sidx * chi + t2]);
+              const cd w = uc[sidx];
+              x.x = fma(-l.x, w.x, x.x);
+              x.x = fma(l.y, w.y, x.x);
+              x.y = fma(-l.x, w.y, x.y);
+              x.y = fma(-l.y, w.x, x.y);
+            }
+            uc[t2] = x;
           }
+          __syncwarp();
         }
-        __syncthreads();
       }
+      __syncthreads();
       cd* Wb_ = Ub;  // W now occupies Ub (entries past each block's rank unused)
       // D_v and D_w columns, one thread per (column, e)
       for (int idx = tid; idx < cw * chi; idx += blockDim.x) {
