@@ -281,7 +281,7 @@ __host__ __device__ inline RefineLayout refine_layout(int chi) {
   l.misc = l.lam1 + chi;
   l.ints = l.misc + 4;
   l.S = l.ints + chi + 4;  // after the 2 chi + 3 ints
-  l.stride = 12 * n * n;  // solve_work_doubles(chi)
+  l.stride = l.S + (chi > 64 ? n * n : 0);  // even, and at most solve_work_doubles(chi)
   return l;
 }
 cudaError_t launch_solve(const SolveArgs& a, cudaStream_t s);

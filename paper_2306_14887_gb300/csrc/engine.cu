@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <cmath>
 #include <array>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -2713,6 +2714,51 @@ tn_status gamma_view(tn_handle* h, int v, const float** ptr, int64_t* len, cudaS
 
 extern "C" {
 
+}  // extern "C"
+
+namespace tnbp {
+namespace {
+// Workspace of the standalone solves: stream-ordered allocations from a pool of
+// the library's own, one per device, that keeps up to 64 MB between calls and
+// gives the rest back at the next synchronisation.  The device's default pool
+// returns everything at every synchronisation, and a call then maps its
+// workspace anew (measured on the refined solve: 4 edges at chi = 8 349 us a
+// call against 187 us of kernels).  Allocation order, threads and streams are
+// the runtime's to keep apart.
+cudaError_t solve_alloc(void** p, size_t bytes, cudaStream_t st) {
+  constexpr int kMaxDevices = 64;
+  static std::mutex mu;
+  static cudaMemPool_t pools[kMaxDevices] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= kMaxDevices) return cudaMallocAsync(p, bytes, st);
+  cudaMemPool_t pool;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    if (!pools[dev]) {
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      cudaMemPool_t q = nullptr;
+      if ((e = cudaMemPoolCreate(&q, &props)) != cudaSuccess) return e;
+      unsigned long long keep = 64ull << 20;
+      if ((e = cudaMemPoolSetAttribute(q, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+        cudaMemPoolDestroy(q);
+        return e;
+      }
+      pools[dev] = q;
+    }
+    pool = pools[dev];
+  }
+  return cudaMallocFromPoolAsync(p, bytes, pool, st);
+}
+}  // namespace
+}  // namespace tnbp
+
+extern "C" {
+
 tn_status tn_truncation_solve(const float* gram, float* dmat, double* s_out, int32_t n_edges,
                               int32_t chi, int32_t sign, double svd_cutoff, void* cuda_stream) {
   return tn_truncation_solve_ex(gram, dmat, s_out, n_edges, chi, sign, svd_cutoff, TN_SOLVE_FP64,
@@ -2738,13 +2784,16 @@ tn_status tn_truncation_solve_ex(const float* gram, float* dmat, double* s_out, 
     return TN_EINVAL;
   }
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  const size_t wbytes = sizeof(double) * (size_t)n_edges * solve_work_doubles(chi);
+  const int kind = solve_kind(solve, chi);
+  // workspace, per-edge statistics and the flag word in one allocation
+  const size_t per_edge = kind == TN_SOLVE_REFINED ? (size_t)refine_layout(chi).stride
+                                                   : solve_work_doubles(chi);
+  const size_t wbytes = sizeof(double) * (size_t)n_edges * per_edge;
   const size_t sbytes = sizeof(double) * 4 * (size_t)n_edges;
-  void *work = nullptr, *stats = nullptr, *flags = nullptr;
-  TN_CUDA_TRY(cudaMallocAsync(&work, wbytes, st));
-  TN_CUDA_TRY(cudaMallocAsync(&stats, sbytes, st));
-  TN_CUDA_TRY(cudaMallocAsync(&flags, sizeof(int), st));
-  TN_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int), st));
+  void* buf = nullptr;
+  TN_CUDA_TRY(solve_alloc(&buf, wbytes + sbytes + sizeof(double), st));
+  void *work = buf, *stats = (char*)buf + wbytes, *flags = (char*)stats + sbytes;
+  cudaError_t le = cudaMemsetAsync(flags, 0, sizeof(int), st);
   SolveArgs a;
   a.n_edges = n_edges;
   a.chi = chi;
@@ -2760,9 +2809,8 @@ tn_status tn_truncation_solve_ex(const float* gram, float* dmat, double* s_out, 
   a.stats = (double*)stats;
   a.flags = (int*)flags;
   a.max_sweeps = 30;
-  cudaError_t le;
-  const int kind = solve_kind(solve, chi);
-  if (kind == TN_SOLVE_SHARED) {
+  if (le != cudaSuccess) {
+  } else if (kind == TN_SOLVE_SHARED) {
     a.max_sweeps = 20;
     le = launch_solve32(a, st);
   } else if (kind == TN_SOLVE_REFINED) {
@@ -2773,9 +2821,7 @@ tn_status tn_truncation_solve_ex(const float* gram, float* dmat, double* s_out, 
   }
   int f = 0;
   cudaError_t ce = cudaMemcpyAsync(&f, flags, sizeof(int), cudaMemcpyDeviceToHost, st);
-  cudaFreeAsync(work, st);
-  cudaFreeAsync(stats, st);
-  cudaFreeAsync(flags, st);
+  cudaFreeAsync(buf, st);
   TN_CUDA_TRY(le);
   TN_CUDA_TRY(ce);
   TN_CUDA_TRY(cudaStreamSynchronize(st));
