@@ -498,7 +498,8 @@ __global__ void __launch_bounds__(kThreads) solve32_kernel(SolveArgs a) {
   const float orth_tol2 = orth_tol * orth_tol, abs_floor2 = abs_floor * abs_floor;
   const int half = n / 2;
   int sweeps = 0;
-  if (n % 32 == 0) {
+  if (n % 32 == 0 && (n & (n - 1)) == 0) {
+    // n a power of two (the halving below meets every pair only then).
     // Rows of 2 x 16-byte vectors, each pair owned by 16 lanes (two pairs per
     // warp, so the rotation arithmetic serves two pairs), lane l holding the
     // vectors l, l + 16, ... of a row (consecutive lanes, consecutive
