@@ -64,6 +64,10 @@ struct GemmDesc {
   const double* comp_state;
   // fused mode products only: store the output rounded to TF32 (nearest)
   int32_t round_c;
+  // CUDA-core GEMM only, B operand: with K0 > 0 its k1 = (i, j), j < K0, lies at
+  // i * b_k0 + j * b_k1
+  int32_t K0;
+  int64_t b_k0;
 };
 // true when the outer entry's component has met the BP stop rule
 __device__ __forceinline__ bool outer_frozen(const GemmDesc& d, int outer) {

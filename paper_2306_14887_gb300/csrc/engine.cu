@@ -468,8 +468,8 @@ bool use_tensor_cores(const tn_handle* h) {
 //  - The split modes stage both parts of every operand through registers there,
 //    three products each: the CUDA-core GEMM gives FP32-accurate products in
 //    less time at every chi measured (ms a sweep, tile against CUDA cores:
-//    union of 338 sites chi = 16 1.04 / 0.22, 65 sites chi = 23 0.77 / 0.19,
-//    127 sites chi = 32 1.02 / 0.33, chi = 64 6.99 / 2.61).
+//    union of 338 sites chi = 16 1.04 / 0.08, 65 sites chi = 23 0.77 / 0.16,
+//    127 sites chi = 32 1.02 / 0.24, chi = 64 6.99 / 2.10).
 // TN_KERNELS_TILE keeps every contraction that is large enough on the tile kernel.
 bool on_tile_kernel(const tn_handle* h, const GemmDesc& d) {
   if (!use_tensor_cores(h)) return false;
@@ -570,6 +570,8 @@ struct Spec {
   int n_inner = 1;
   int64_t a_in = 0, b_in = 0, c_in = 0;
   int conj_b = 0, b_pre = 0;
+  int K0 = 0;
+  int64_t b_k0 = 0;
 };
 
 void add_spec(Plan& P, const Spec& sp, int prec, const std::vector<Ent>& ent) {
@@ -583,7 +585,7 @@ void add_spec(Plan& P, const Spec& sp, int prec, const std::vector<Ent>& ent) {
   d.c_m = sp.c_m; d.c_m2 = sp.c_m2; d.c_m3 = sp.c_m3; d.c_n = sp.c_n;
   d.plane_a = sp.plane_a; d.plane_b = sp.plane_b; d.plane_c = sp.plane_c;
   d.n_inner = sp.n_inner; d.a_in = sp.a_in; d.b_in = sp.b_in; d.c_in = sp.c_in;
-  d.conj_b = sp.conj_b; d.b_pre = sp.b_pre;
+  d.conj_b = sp.conj_b; d.b_pre = sp.b_pre; d.K0 = sp.K0; d.b_k0 = sp.b_k0;
   for (auto& e : ent) { L.A.push_back(e[0]); L.B.push_back(e[1]); L.C.push_back((float*)e[2]); }
   d.n_outer = (int)ent.size();
   P.L.push_back(std::move(L));
@@ -742,6 +744,85 @@ void deg2_chain(tn_handle* h, Plan& P, int which, const std::vector<int>& sites,
   deg2_chain_sites(h, P, which, cs, open_p);
 }
 
+// Whether every contraction of the handle runs on the CUDA cores (FP32, and the
+// split modes, see on_tile_kernel).
+bool cuda_core_mode(const tn_config& c) {
+  return c.prec == TN_FP32 ||
+         (c.kernels == TN_KERNELS_AUTO && (c.prec == TN_TF32X3 || c.prec == TN_BF16X3));
+}
+
+// Mode product on the CUDA cores with its rows contiguous: A rows m at a_m, a_m2,
+// the contracted index at stride a_k; the message itself (columns contiguous)
+// as B; the output's rows contiguous, column n at stride c_n.
+Spec rows_spec(int chi, int64_t plane, int M, int M2, int M3, int64_t a_m, int64_t a_m2,
+               int64_t a_m3, int64_t a_k, int64_t c_m, int64_t c_m2, int64_t c_m3, int64_t c_n) {
+  Spec sp = mode_spec(chi, plane, M, M2, M3, a_m, a_m2, a_m3, c_m, c_m2, c_m3, c_n);
+  sp.a_k2 = a_k;
+  sp.b_pre = 0;
+  sp.b_n = 1; sp.b_k1 = 0; sp.b_k2 = chi; sp.plane_b = (int64_t)chi * chi;
+  return sp;
+}
+
+// The degree-3 chains of a sweep on the CUDA cores.  The same contractions in
+// the same order as deg3_chain, laid out so that almost every operand has its
+// rows (columns) contiguous, which the GEMM copies in 16-byte pieces, and with
+// the product T x_c Mc that the first two chains share taken once:
+//   A1  Y1[p][c'][b][a] = TA x_c Mc   A2  Y2[p][b'][c'][a] = Y1 x_b Mb   close on a, TA
+//   B2  Y2[p][a'][c'][b] = Y1 x_a Ma                                     close on b, T
+//   C1  Y1[p][a'][b][c] = T x_a Ma    C2  Y2[p][b'][a'][c] = Y1 x_b Mb   close on c, T
+// At chi = 64 on 127 qubits a sweep takes 2.10 ms, with K-contiguous operands
+// copied value by value and six products 2.61 ms; at chi = 23 on 65 qubits (no
+// 16-byte pieces) 0.16 and 0.165 ms.
+void deg3_chains_rows(tn_handle* h, Plan& P, const std::vector<int>& sites) {
+  if (sites.empty()) return;
+  const HostGraph& g = h->g;
+  const int x = h->chi, prec = h->cfg.prec;
+  const int64_t x2 = (int64_t)x * x, x3 = x2 * x, plane = 2 * x3;
+  const int M = (int)(2 * x2);
+  auto entries = [&](auto a, auto b, auto c) {
+    std::vector<Ent> e;
+    for (int v : sites) e.push_back({a(v), b(v), c(v)});
+    return e;
+  };
+  auto T = [&](int v) { return site_ptr(h, h->T, v); };
+  auto TA = [&](int v) { return site_ptr(h, h->TA, v); };
+  auto Y1 = [&](int v) { return site_ptr(h, h->Y1, v); };
+  auto Y2 = [&](int v) { return site_ptr(h, h->Y2, v); };
+  auto msg = [&](int j) { return [h, &g, j](int v) { return in_msg(h, v, g.legs[v][j]); }; };
+  auto raw = [&](int j) {
+    return [h, &g, j](int v) { return msg_ptr(h, h->raw, dir_id(g, v, g.legs[v][j])); };
+  };
+  // close: A = Y2 with the open leg contiguous, K = (k1, k2) at (a_k1, x)
+  auto close = [&](int K1, int K2, int64_t a_k1) {
+    Spec sp = close_spec(x, plane, K1, K2, 1, a_k1, 1, a_k1);
+    sp.a_k2 = x;
+    sp.b_k2 = x;
+    return sp;
+  };
+  // A1: rows (p, b, a) of TA; A2: rows (p, c', a); K = (p, (b', c'))
+  add_spec(P, rows_spec(x, plane, M, x, x, x3, x2, 1, x, x3, x, 1, x2), prec, entries(TA, msg(2), Y1));
+  add_spec(P, rows_spec(x, plane, M, x, x, x3, x2, 1, x, x3, x, 1, x2), prec, entries(Y1, msg(1), Y2));
+  add_spec(P, close(2, (int)x2, x3), prec, entries(Y2, TA, raw(0)));
+  // B2: rows (p, c', b) of Y1, a contiguous and contracted; K = ((p, a'), c')
+  add_spec(P, rows_spec(x, plane, M, (int)x2, 1, x3, x, 0, 1, x3, 1, 0, x2), prec,
+           entries(Y1, msg(0), Y2));
+  Spec sb = close(2 * x, x, x2);
+  sb.b_n = x;
+  sb.b_k1 = x2;
+  sb.b_k2 = 1;
+  add_spec(P, sb, prec, entries(Y2, T, raw(1)));
+  // C1: rows (p, (b, c)) of T; C2: rows (p, a', c); K = ((p, b'), a')
+  add_spec(P, rows_spec(x, plane, M, (int)x2, 1, x3, 1, 0, x2, x3, 1, 0, x2), prec,
+           entries(T, msg(0), Y1));
+  add_spec(P, rows_spec(x, plane, M, x, x, x3, x2, 1, x, x3, x, 1, x2), prec, entries(Y1, msg(1), Y2));
+  Spec sc = close(2 * x, x, x2);
+  sc.K0 = x;
+  sc.b_k0 = x3;
+  sc.b_k1 = x;
+  sc.b_k2 = x2;
+  add_spec(P, sc, prec, entries(Y2, T, raw(2)));
+}
+
 void build_sweep_plan(tn_handle* h) {
   const HostGraph& g = h->g;
   Plan& P = h->sweep;
@@ -753,7 +834,12 @@ void build_sweep_plan(tn_handle* h) {
     for (size_t i = from; i < P.L.size(); ++i) P.L[i].outer_site = sites;
   };
   const std::vector<int>& s3 = h->sites_by_deg[3];
-  for (int which = 0; which < 3; ++which) {
+  const bool rows = cuda_core_mode(h->cfg);
+  if (rows) {
+    deg3_chains_rows(h, P, s3);
+    tag(0, s3);
+  }
+  for (int which = 0; which < 3 && !rows; ++which) {
     std::vector<float*> outs;
     for (int v : s3) outs.push_back((float*)msg_ptr(h, h->raw, dir_id(g, v, g.legs[v][which])));
     const size_t from = P.L.size();
@@ -777,13 +863,6 @@ void build_sweep_plan(tn_handle* h) {
   const size_t from = P.L.size();
   add_close(P, 1, 0, h->chi, false, h->cfg.prec, d1);
   tag(from, h->sites_by_deg[1]);
-}
-
-// Whether every contraction of the handle runs on the CUDA cores (FP32, and the
-// split modes, see on_tile_kernel).
-bool cuda_core_mode(const tn_config& c) {
-  return c.prec == TN_FP32 ||
-         (c.kernels == TN_KERNELS_AUTO && (c.prec == TN_TF32X3 || c.prec == TN_BF16X3));
 }
 
 // The sweep as one launch (site_sweep.cu): the degree-3 chains first, the
@@ -828,12 +907,12 @@ tn_status build_site_jobs(tn_handle* h) {
 }
 
 // The sweep's contractions at small chi, with the split-K counts the plan's
-// degree-3 closes (every third launch) have.
+// degree-3 closes (launches 2, 4 and 7) have.
 tn_status run_site_sweep(tn_handle* h) {
   int splits[3] = {1, 1, 1};
   if (!h->sites_by_deg[3].empty())
     for (int j = 0; j < 3; ++j) {
-      const HostLaunch& L = h->sweep.L[3 * j + 2];
+      const HostLaunch& L = h->sweep.L[j == 0 ? 2 : j == 1 ? 4 : 7];
       size_t pf = 0;
       const int s = cgemm_plan(L.d, &pf, L.tuned);
       splits[j] = pf > h->part_floats ? 1 : s;

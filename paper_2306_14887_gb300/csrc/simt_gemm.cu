@@ -12,14 +12,18 @@
 // 16-byte shared reads per 64 FMAs, issued as packed pairs (the pair rate per
 // lane is the scalar one, but it leaves issue slots for the reads and copies:
 // 2.61 against 2.81 ms a sweep).  The two-sums take another 18 % of the pipe.
-// Measured on the 127-qubit sweep at chi = 64 (88.6 GFLOP as executed): 2.61 ms
-// a sweep, 34 TFLOP/s of the 77 the pipe reaches; with scalar global loads into
-// a single shared buffer and 16 scalar shared reads per step it took 8.08 ms.
-// Slices reach shared memory through a
-// 3-stage ring of 4-byte asynchronous copies laid out [k][row], which serves
-// every stride and alignment a descriptor may have (odd chi, K- or
-// row-contiguous operands) without staging registers; the copies of slice
-// s + 2 are in flight while slice s is multiplied.
+// Slices reach shared memory through a 3-stage ring of asynchronous copies laid
+// out [k][row]: 16-byte copies where four rows are one block of memory, else
+// 4-byte ones, which serve every stride and alignment a descriptor may have (odd
+// chi, K-contiguous operands) without staging registers; the copies of slice
+// s + 2 are in flight while slice s is multiplied.  The copies are the second
+// cost: an operand held twice in shared memory (to spare the register copies of
+// packed pairs) lost 15 %, 16-byte copies gained 10 %.
+// Measured on the 127-qubit sweep at chi = 64: 2.10 ms a sweep (78.8 GFLOP, 37
+// of the pipe's 77 TFLOP/s; a probe with this inner loop alone reaches 56).  With
+// scalar global loads into a single shared buffer and 16 scalar shared reads per
+// step it took 8.08 ms.  A persistent form, its copies running ahead across
+// tiles, spilled registers and took 2.95 against 2.61 ms.
 #include <algorithm>
 #include <mutex>
 
@@ -49,12 +53,34 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const float* src, bool o
                : "memory");
 }
 
-// Offset of contraction index k of an operand; k1 is zero for one-level K.
-__device__ __forceinline__ int k_off(int k, int K1, int K2, int s1, int s2) {
-  if (K1 == 1) return k * s2;
-  const int k1 = k / K2;
-  return k1 * s1 + (k - k1 * K2) * s2;
+// 16-byte asynchronous copy global -> shared, zero fill when !ok.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const float* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
+               "r"(ok ? 16 : 0)
+               : "memory");
 }
+
+// Quotients by n as products: x / n = x inv >> 40 with inv = ceil(2^40 / n), exact
+// for x n < 2^40 (here x <= 2^17, n <= 2^16).
+inline uint64_t inverse40(int n) { return n > 0 ? ((1ull << 40) + n - 1) / n : 0; }
+__device__ __forceinline__ int quotient(int x, uint64_t inv) {
+  return (int)(((uint64_t)(uint32_t)x * inv) >> 40);
+}
+
+// How an operand's contraction index runs: k = (k1, k2), with K0 > 0
+// k1 = (i, j), j < K0, at i s0 + j s1.
+struct KIndex {
+  int K1, K2, K0, s0, s1, s2;
+  uint64_t inv2, inv0;  // inverse40 of K2 and K0
+  __device__ __forceinline__ int off(int k) const {
+    if (K1 == 1) return k * s2;
+    const int k1 = quotient(k, inv2);
+    const int k2 = k - k1 * K2;
+    if (K0 == 0) return k1 * s1 + k2 * s2;
+    const int i = quotient(k1, inv0);
+    return i * s0 + (k1 - i * K0) * s1 + k2 * s2;
+  }
+};
 
 // BM x BN outputs, TM x TM of them per thread.
 template <int BM, int BN, int TM>
@@ -70,44 +96,65 @@ template <int TM> struct Vec;
 template <> struct Vec<4> { using type = float4; };
 template <> struct Vec<2> { using type = float2; };
 
-// What one thread copies of one operand per slice: for a K-contiguous operand
-// the K offset tid % 16 of every kThreads / 16-th row, else row tid % ROWS at
-// every kThreads / ROWS-th K offset.
+// How a slice of an operand is copied: by single values along K or along the
+// rows, whichever is contiguous, or by 16-byte pieces of four rows.
+enum CopyMode { kAlongK = 0, kAlongRows = 1, kFourRows = 2 };
+
+// What one thread copies of one operand per slice.  kAlongK: the K offset
+// tid % 16 of every THREADS / 16-th row; kAlongRows: row tid % ROWS at every
+// THREADS / ROWS-th K offset; kFourRows: rows 4 (tid % (ROWS / 4)) .. + 3 at
+// every 4 THREADS / ROWS-th K offset.
 template <int ROWS, int LD, int THREADS>
 struct Loader {
   static constexpr int kCount = ROWS * BK / THREADS;
   static_assert(kCount * THREADS == ROWS * BK && THREADS % ROWS == 0, "whole copies per thread");
+  static constexpr int kStep4 = THREADS / (ROWS / 4);  // K offsets one pass of 16-byte copies has
   const float* base;
-  int off[kCount];   // row offsets (K-contiguous) or off[0]
-  bool kfast;
+  int off[kCount];   // row offsets (kAlongK) or off[0]
   unsigned ok;       // valid rows, one bit per copy
-  int K1, K2, s1, s2, plane;
+  int mode, plane;
+  KIndex ki;
 
   template <class RowOff>
-  __device__ void init(const float* p, bool kf, int row0, int rows, int K1_, int K2_, int64_t s1_,
-                       int64_t s2_, int64_t plane_, RowOff row_off) {
+  __device__ void init(const float* p, int mode_, int row0, int rows, const KIndex& ki_,
+                       int64_t plane_, RowOff row_off) {
     base = p;
-    kfast = kf;
-    K1 = K1_;
-    K2 = K2_;
-    s1 = (int)s1_;
-    s2 = (int)s2_;
+    mode = mode_;
+    ki = ki_;
     plane = (int)plane_;
     ok = 0;
     const int tid = threadIdx.x;
+    if (mode == kAlongK) {
 #pragma unroll
-    for (int i = 0; i < kCount; ++i) {
-      const int r = row0 + (kfast ? (tid >> 4) + i * (THREADS / BK) : tid % ROWS);
-      off[i] = r < rows ? (int)row_off(r) : 0;
-      ok |= (r < rows ? 1u : 0u) << i;
+      for (int i = 0; i < kCount; ++i) {
+        const int r = row0 + (tid >> 4) + i * (THREADS / BK);
+        off[i] = r < rows ? (int)row_off(r) : 0;
+        ok |= (r < rows ? 1u : 0u) << i;
+      }
+    } else {
+      const int r = row0 + (mode == kFourRows ? 4 * (tid % (ROWS / 4)) : tid % ROWS);
+      off[0] = r < rows ? (int)row_off(r) : 0;
+      ok = r < rows ? 1u : 0u;
     }
   }
   __device__ __forceinline__ void load(uint32_t dst, int k0, int kend) const {
     const int tid = threadIdx.x;
-    if (kfast) {
+    if (mode == kFourRows) {
+      const int r = 4 * (tid % (ROWS / 4));
+#pragma unroll
+      for (int i = 0; i < (BK + kStep4 - 1) / kStep4; ++i) {
+        const int kk = tid / (ROWS / 4) + i * kStep4, k = k0 + kk;
+        if (kStep4 > BK && kk >= BK) break;
+        const bool v = k < kend && ok;
+        const float* q = base + off[0] + (v ? ki.off(k) : 0);
+        const uint32_t d0 = dst + 4 * (kk * LD + r);
+        cp_async16(d0, q, v);
+        cp_async16(d0 + 4 * BK * LD, q + plane, v);
+      }
+    } else if (mode == kAlongK) {
       const int kk = tid & (BK - 1), k = k0 + kk;
       const bool kok = k < kend;
-      const int ko = kok ? k_off(k, K1, K2, s1, s2) : 0;
+      const int ko = kok ? ki.off(k) : 0;
       const uint32_t d0 = dst + 4 * (kk * LD + (tid >> 4));
 #pragma unroll
       for (int i = 0; i < kCount; ++i) {
@@ -121,8 +168,8 @@ struct Loader {
 #pragma unroll
       for (int i = 0; i < kCount; ++i) {
         const int kk = tid / ROWS + i * (THREADS / ROWS), k = k0 + kk;
-        const bool v = k < kend && (ok & 1);
-        const float* q = base + off[0] + (v ? k_off(k, K1, K2, s1, s2) : 0);
+        const bool v = k < kend && ok;
+        const float* q = base + off[0] + (v ? ki.off(k) : 0);
         const uint32_t d0 = dst + 4 * (kk * LD + r);
         cp_async4(d0, q, v);
         cp_async4(d0 + 4 * BK * LD, q + plane, v);
@@ -131,9 +178,29 @@ struct Loader {
   }
 };
 
+// The copies of a slice follow the operand's contiguous index; rows in pieces of
+// four when every piece is a whole 16-byte block of memory.
+__device__ __forceinline__ int copy_mode_a(const GemmDesc& d, const float* A) {
+  const bool three = d.M3 > 1, two = !three && d.M2 > 1;
+  const int64_t row = three ? d.a_m3 : two ? d.a_m2 : d.a_m;  // stride of the innermost level
+  if (row != 1 || (d.a_k2 == 1 && !three && !two)) return d.a_k2 == 1 ? kAlongK : kAlongRows;
+  const int level = three ? d.M3 : two ? d.M2 : d.M;
+  const int64_t strides = (three || two ? d.a_m : 0) | (three ? d.a_m2 : 0) | d.a_k1 | d.a_k2 |
+                          d.plane_a;
+  const bool whole = level % 4 == 0 && strides % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+  return whole ? kFourRows : kAlongRows;
+}
+__device__ __forceinline__ int copy_mode_b(const GemmDesc& d, const float* B) {
+  if (d.b_n != 1) return kAlongK;
+  const int64_t strides = d.b_k0 | d.b_k1 | d.b_k2 | d.plane_b;
+  const bool whole = d.N % 4 == 0 && strides % 4 == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
+  return whole ? kFourRows : kAlongRows;
+}
+
 template <int BM, int BN, int TM, bool CONJ_B>
 __global__ void __launch_bounds__(Tile<BM, BN, TM>::kThreads, 512 / Tile<BM, BN, TM>::kThreads)
-    cgemm_simt_kernel(GemmDesc d, float* part, int splits, int k_per_split) {
+    cgemm_simt_kernel(GemmDesc d, float* part, int splits, int k_per_split, uint64_t inv2,
+                      uint64_t inv0) {
   using T = Tile<BM, BN, TM>;
   using V = typename Vec<TM>::type;
   constexpr int NT = T::kThreads, LDA = T::kLda, LDB = T::kLdb;
@@ -156,11 +223,11 @@ __global__ void __launch_bounds__(Tile<BM, BN, TM>::kThreads, 512 / Tile<BM, BN,
 
   Loader<BM, LDA, NT> la;
   Loader<BN, LDB, NT> lb;
-  // the copies of a slice follow the operand's contiguous index
-  la.init(A,
-          (d.a_k2 == 1) && !(d.M2 > 1 && d.M3 <= 1 && d.a_m2 == 1) && !(d.M3 > 1 && d.a_m3 == 1),
-          m0, d.M, d.K1, d.K2, d.a_k1, d.a_k2, d.plane_a, [&](int m) { return ROW_A(d, m); });
-  lb.init(B, d.b_n != 1, n0, d.N, d.K1, d.K2, d.b_k1, d.b_k2, d.plane_b,
+  la.init(A, copy_mode_a(d, A), m0, d.M,
+          KIndex{d.K1, d.K2, 0, 0, (int)d.a_k1, (int)d.a_k2, inv2, 0}, d.plane_a,
+          [&](int m) { return ROW_A(d, m); });
+  lb.init(B, copy_mode_b(d, B), n0, d.N,
+          KIndex{d.K1, d.K2, d.K0, (int)d.b_k0, (int)d.b_k1, (int)d.b_k2, inv2, inv0}, d.plane_b,
           [&](int n) { return (int64_t)n * d.b_n; });
   const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(sm);
   auto issue = [&](int s) {
@@ -334,10 +401,13 @@ template <int BM, int BN, int TM>
 void launch_tile(const GemmDesc& d, float* part, int splits, int kps, cudaStream_t s) {
   using T = Tile<BM, BN, TM>;
   const dim3 grid((d.M + BM - 1) / BM, (d.N + BN - 1) / BN, d.n_outer * d.n_inner * splits);
+  const uint64_t inv2 = inverse40(d.K2), inv0 = inverse40(d.K0);
   if (d.conj_b)
-    cgemm_simt_kernel<BM, BN, TM, true><<<grid, T::kThreads, T::kBytes, s>>>(d, part, splits, kps);
+    cgemm_simt_kernel<BM, BN, TM, true><<<grid, T::kThreads, T::kBytes, s>>>(d, part, splits, kps, inv2,
+                                                                            inv0);
   else
-    cgemm_simt_kernel<BM, BN, TM, false><<<grid, T::kThreads, T::kBytes, s>>>(d, part, splits, kps);
+    cgemm_simt_kernel<BM, BN, TM, false><<<grid, T::kThreads, T::kBytes, s>>>(d, part, splits, kps, inv2,
+                                                                            inv0);
 }
 
 }  // namespace
