@@ -216,10 +216,9 @@ __device__ EdgeView edge_view(const SolveArgs& a, int edge) {
 // instructions few: a row is taken by L lanes, the fewest that still give every
 // warp rows, whose partial sums need log2(L) additions per column at the end;
 // four of a lane's operands are loaded ahead.
-template <int L, int J, class RF, class AF, class BF, class SF>
+template <int L, int J, int kAhead, class RF, class AF, class BF, class SF>
 __device__ __forceinline__ void rows_block(int nrows, int j0, const cd* B, int ldb, RF range,
                                            AF arow, BF bidx, SF store) {
-  constexpr int kAhead = 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int sub = lane & (L - 1);
   for (int i0 = warp * (32 / L); i0 < nrows; i0 += kWarps * (32 / L)) {
@@ -258,29 +257,38 @@ __device__ __forceinline__ void rows_block(int nrows, int j0, const cd* B, int l
   }
 }
 
-// All cw columns, eight at a time and the rest in smaller groups.
+// All cw columns.  SMALL (n <= 64): every CTA runs each product about once, and
+// what it costs is fetching its instructions, so the loops stay short: eight
+// lanes a row, two columns at a time.  Otherwise two lanes a row (eight up to 64
+// rows), eight columns at a time and the rest in smaller groups.
 template <int L, class RF, class AF, class BF, class SF>
-__device__ void rows_cols(int nrows, int cw, const cd* B, int ldb, RF range, AF arow, BF bidx,
-                          SF store) {
+__device__ __forceinline__ void rows_cols(int nrows, int cw, const cd* B, int ldb, RF range,
+                                          AF arow, BF bidx, SF store) {
   int j = 0;
-  for (; j + 8 <= cw; j += 8) rows_block<L, 8>(nrows, j, B, ldb, range, arow, bidx, store);
+  for (; j + 8 <= cw; j += 8) rows_block<L, 8, 4>(nrows, j, B, ldb, range, arow, bidx, store);
   if (j + 4 <= cw) {
-    rows_block<L, 4>(nrows, j, B, ldb, range, arow, bidx, store);
+    rows_block<L, 4, 4>(nrows, j, B, ldb, range, arow, bidx, store);
     j += 4;
   }
   if (j + 2 <= cw) {
-    rows_block<L, 2>(nrows, j, B, ldb, range, arow, bidx, store);
+    rows_block<L, 2, 4>(nrows, j, B, ldb, range, arow, bidx, store);
     j += 2;
   }
-  if (j < cw) rows_block<L, 1>(nrows, j, B, ldb, range, arow, bidx, store);
+  if (j < cw) rows_block<L, 1, 4>(nrows, j, B, ldb, range, arow, bidx, store);
 }
 
-// Lanes per row: eight warps hold 256 / L rows at once.
-template <class RF, class AF, class BF, class SF>
-__device__ void row_products(int nrows, int cw, const cd* B, int ldb, RF range, AF arow, BF bidx,
-                      SF store) {
-  if (nrows > 64) rows_cols<2>(nrows, cw, B, ldb, range, arow, bidx, store);
-  else rows_cols<8>(nrows, cw, B, ldb, range, arow, bidx, store);
+template <bool SMALL, class RF, class AF, class BF, class SF>
+__device__ __forceinline__ void row_products(int nrows, int cw, const cd* B, int ldb, RF range,
+                                             AF arow, BF bidx, SF store) {
+  if (SMALL) {
+    int j = 0;
+    for (; j + 2 <= cw; j += 2) rows_block<8, 2, 1>(nrows, j, B, ldb, range, arow, bidx, store);
+    if (j < cw) rows_block<8, 1, 1>(nrows, j, B, ldb, range, arow, bidx, store);
+  } else if (nrows > 64) {
+    rows_cols<2>(nrows, cw, B, ldb, range, arow, bidx, store);
+  } else {
+    rows_cols<8>(nrows, cw, B, ldb, range, arow, bidx, store);
+  }
 }
 
 // One Newton step for the kept columns [j0, j1) of one edge.  Shared-memory
@@ -289,6 +297,7 @@ __device__ void row_products(int nrows, int cw, const cd* B, int ldb, RF range, 
 // update coefficients), B3 (Y'_q, then Z = conj(G_w) Y, then R); lamc the
 // columns' Rayleigh quotients (negated start eigenvalue for tail columns),
 // lamf the final eigenvalues.
+template <bool SMALL>
 __device__ void refine_chunk(const SolveArgs& a, const EdgeView& v, int j0, int j1, cd* Uc, cd* B1,
                              cd* B2, cd* B3, double* lamc, double* lamf) {
   const int chi = v.chi, n = v.n, A = v.act;
@@ -301,7 +310,7 @@ __device__ void refine_chunk(const SolveArgs& a, const EdgeView& v, int j0, int 
   for (int idx = tid; idx < cw * n; idx += blockDim.x) Uc[idx] = v.U[(int64_t)j0 * n + idx];
   __syncthreads();
   // Y = R_v^H U_c: Y[(k, perm_k[s])] = sum_{t <= s, t < rank_k} L_k[s][t] U[(k, t)]
-  row_products(
+  row_products<SMALL>(
       n, cw, Uc, n,
       [&](int i, int& lo, int& hi) {
         const int k = i / chi, s = i - k * chi;
@@ -336,7 +345,7 @@ __device__ void refine_chunk(const SolveArgs& a, const EdgeView& v, int j0, int 
     B3[j * n + i] = {mine.x - sg * other.y, mine.y + sg * other.x};
   }
   __syncthreads();
-  row_products(
+  row_products<SMALL>(
       n, cw, B3, n, [&](int, int& lo, int& hi) { lo = 0; hi = chi; },
       [&](int i, int r) {
         const int q = i / chi, e = i - q * chi;
@@ -356,7 +365,7 @@ __device__ void refine_chunk(const SolveArgs& a, const EdgeView& v, int j0, int 
   }
   __syncthreads();
   // P = R_v Z: P[(b, t)] = sum_{s >= t} conj(L_b[s][t]) Z[(b, perm_b[s])], zero for t >= rank_b
-  row_products(
+  row_products<SMALL>(
       n, cw, B3, n,
       [&](int i, int& lo, int& hi) {
         const int b = i / chi, t = i - b * chi;
@@ -374,11 +383,11 @@ __device__ void refine_chunk(const SolveArgs& a, const EdgeView& v, int j0, int 
       [&](int i, int j, cd val) { B1[j * n + i] = val; });
   __syncthreads();
   // S = U_A^H P and R = I - U_A^H U_c
-  row_products(
+  row_products<SMALL>(
       A, cw, B1, n, [&](int, int& lo, int& hi) { lo = 0; hi = n; },
       [&](int i, int r) { return cconj(v.U[(int64_t)i * n + r]); }, [&](int, int r) { return r; },
       [&](int i, int j, cd val) { B2[j * n + i] = val; });
-  row_products(
+  row_products<SMALL>(
       A, cw, Uc, n, [&](int, int& lo, int& hi) { lo = 0; hi = n; },
       [&](int i, int r) { return cconj(v.U[(int64_t)i * n + r]); }, [&](int, int r) { return r; },
       [&](int i, int j, cd val) {
@@ -457,27 +466,28 @@ __device__ void refine_chunk(const SolveArgs& a, const EdgeView& v, int j0, int 
   // u_j' = u_j + P_j / lambda_j + sum_{i < A} u_i c_ij for head columns,
   // u_j + sum_i u_i c_ij for tail columns; a head column without a positive
   // Rayleigh quotient keeps its start
-  const int ng = (cw + kJU - 1) / kJU;
+  constexpr int JU = SMALL ? 1 : kJU, AHEAD = SMALL ? 2 : 8;
+  const int ng = (cw + JU - 1) / JU;
   for (int idx = tid; idx < n * ng; idx += blockDim.x) {
-    const int r = idx % n, jb = (idx / n) * kJU;
-    cd acc[kJU];
+    const int r = idx % n, jb = (idx / n) * JU;
+    cd acc[JU];
 #pragma unroll
-    for (int jj = 0; jj < kJU; ++jj) acc[jj] = cz();
-    const int nj = min(kJU, cw - jb);
-    for (int i0 = 0; i0 < A; i0 += 8) {
-      cd u[8];
+    for (int jj = 0; jj < JU; ++jj) acc[jj] = cz();
+    const int nj = min(JU, cw - jb);
+    for (int i0 = 0; i0 < A; i0 += AHEAD) {
+      cd u[AHEAD];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) u[t] = i0 + t < A ? v.U[(int64_t)(i0 + t) * n + r] : cz();
+      for (int t = 0; t < AHEAD; ++t) u[t] = i0 + t < A ? v.U[(int64_t)(i0 + t) * n + r] : cz();
 #pragma unroll
-      for (int t = 0; t < 8; ++t) {
+      for (int t = 0; t < AHEAD; ++t) {
         if (i0 + t >= A) break;
 #pragma unroll
-        for (int jj = 0; jj < kJU; ++jj)
+        for (int jj = 0; jj < JU; ++jj)
           if (jj < nj) cfma(acc[jj], u[t], B2[(jb + jj) * n + i0 + t]);
       }
     }
 #pragma unroll
-    for (int jj = 0; jj < kJU; ++jj) {
+    for (int jj = 0; jj < JU; ++jj) {
       const int j = jb + jj;
       if (jj >= nj) continue;
       const double lj = lamc[j];
@@ -493,10 +503,13 @@ __device__ void refine_chunk(const SolveArgs& a, const EdgeView& v, int j0, int 
 
 // Bound by the FP64 pipe.  Measured (ncu): chi = 64, 51 edges 1.78 ms (2.21 with
 // eight lanes on every row and every group of eight columns reduced whole);
-// chi = 37, 24 edges 0.24 ms (0.42); chi = 21, 7 edges 63 us (101).
+// chi = 37, 24 edges 0.24 ms (0.42); with the short loops of SMALL chi = 21, 7
+// edges 38 us (63 with the unrolled ones, 101 at first), chi = 16, 48 edges 66 us
+// (100, 127).
 // The kept-column slots of all edges, ne * chi, split evenly over the grid: each
 // block takes a contiguous range (split further at edge boundaries and into
 // pieces of at most cwmax columns).
+template <bool SMALL>
 __global__ void __launch_bounds__(kThreads, 1) refine_kernel(SolveArgs a, int cwmax) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int chi = a.chi, n = 2 * chi;
@@ -513,7 +526,7 @@ __global__ void __launch_bounds__(kThreads, 1) refine_kernel(SolveArgs a, int cw
     const int e = (int)(g / chi), j0 = (int)(g % chi);
     const int jend = (int)min((int64_t)chi, j0 + (g1 - g));
     const EdgeView v = edge_view(a, e);
-    for (int s = j0; s < jend; s += cwmax) refine_chunk(a, v, s, min(jend, s + cwmax), Uc, B1, B2, B3, lamc, lamf);
+    for (int s = j0; s < jend; s += cwmax) refine_chunk<SMALL>(a, v, s, min(jend, s + cwmax), Uc, B1, B2, B3, lamc, lamf);
     g += jend - j0;
   }
 }
@@ -530,7 +543,8 @@ __global__ void __launch_bounds__(kThreads, 1) refine_kernel(SolveArgs a, int cw
 // with b_b(q) = exp(s i pi/4 s_b s_q), as the gate split gives.
 // Measured (ncu): chi = 64, 51 edges 0.53 ms (0.56 with the substitution over the
 // whole block, two barriers a step), chi = 37, 24 edges 0.15 ms (0.21), chi = 21,
-// 7 edges 47 us (59).
+// 7 edges 45 us (59).
+template <bool SMALL>
 __global__ void __launch_bounds__(kThreads, 2) legs_kernel(SolveArgs a, int cwmax) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int chi = a.chi, n = 2 * chi;
@@ -607,7 +621,7 @@ __global__ void __launch_bounds__(kThreads, 2) legs_kernel(SolveArgs a, int cwma
       }
       __syncthreads();
       // Y = L_b u_b (from the unmodified columns) first
-      row_products(
+      row_products<SMALL>(
           n, cw, Ub, n,
           [&](int i, int& lo, int& hi) {
             const int b = i / chi, t = i - b * chi;
@@ -737,11 +751,14 @@ cudaError_t refine_prepare() {
     result = cudaFuncSetAttribute(chol64_kernel<2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)kCholSmemMax);
     if (result == cudaSuccess)
-      result = cudaFuncSetAttribute(refine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)kRefineSmemMax);
-    if (result == cudaSuccess)
-      result = cudaFuncSetAttribute(legs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)kLegsSmemMax);
+      for (auto k : {refine_kernel<false>, refine_kernel<true>})
+        if (result == cudaSuccess)
+          result = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)kRefineSmemMax);
+    for (auto k : {legs_kernel<false>, legs_kernel<true>})
+      if (result == cudaSuccess)
+        result = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)kLegsSmemMax);
   });
   return result;
 }
@@ -777,6 +794,7 @@ cudaError_t launch_solve_refined_newton(const SolveArgs& a, cudaStream_t st) {
   if (a.n_edges <= 0) return cudaSuccess;
   if (!solve_refined_supported(a.chi)) return cudaErrorInvalidValue;
   const int chi = a.chi, n = 2 * chi;
+  const bool small = n <= 64;
   // 3. FP64 Newton step, the kept-column slots balanced over the SMs
   const int64_t T = (int64_t)a.n_edges * chi;
   const int cw_fit = (int)(kSmemBudget / (sizeof(cd) * 4 * (size_t)n + 2 * sizeof(double)));
@@ -787,7 +805,8 @@ cudaError_t launch_solve_refined_newton(const SolveArgs& a, cudaStream_t st) {
   cudaError_t e = refine_prepare();
   if (e != cudaSuccess) return e;
   if (sm_ref > kRefineSmemMax) return cudaErrorInvalidValue;
-  refine_kernel<<<grid, kThreads, sm_ref, st>>>(a, cwmax);
+  if (small) refine_kernel<true><<<grid, kThreads, sm_ref, st>>>(a, cwmax);
+  else refine_kernel<false><<<grid, kThreads, sm_ref, st>>>(a, cwmax);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // 4. FP64 leg matrices, spectrum and messages.  The back substitution is a
   // chain of chi dependent passes: two CTAs per SM (half the columns each)
@@ -799,7 +818,8 @@ cudaError_t launch_solve_refined_newton(const SolveArgs& a, cudaStream_t st) {
   const size_t sm_legs = sizeof(cd) * 2 * (size_t)cw_l * n + sizeof(double) * chi +
                          sizeof(int) * 3 * chi + chi + 16;
   if (sm_legs > kLegsSmemMax) return cudaErrorInvalidValue;
-  legs_kernel<<<grid_l, kThreads, sm_legs, st>>>(a, cw_l);
+  if (small) legs_kernel<true><<<grid_l, kThreads, sm_legs, st>>>(a, cw_l);
+  else legs_kernel<false><<<grid_l, kThreads, sm_legs, st>>>(a, cw_l);
   return cudaGetLastError();
 }
 
