@@ -218,18 +218,21 @@ cudaError_t launch_bp_stop(int n_comp, double* state, unsigned long long* res,
 
 // Realified transposed copies of n planar complex chi x chi matrices (each at
 // src + i*src_stride): dst + i*4chi^2 holds Bt[(t,n)][(s,k)] as in GemmDesc::b_pre.
-// tf32: every value rounded to TF32 (nearest).
 cudaError_t launch_realify(const float* src, int64_t src_stride, float* dst, int n, int chi,
-                           cudaStream_t s, bool tf32 = false);
+                           cudaStream_t s);
+// dst = src rounded to TF32 (nearest); n floats, a multiple of 4, 16-byte aligned.
+cudaError_t launch_round_tf32(const float* src, float* dst, int64_t n, cudaStream_t s);
 
 // TA copies of site tensors with the first leg moved last:
 // TA[pl][p][l1..l_{d-1}][l0] = T[pl][p][l0][l1..l_{d-1}] (planar).
+// tf32: the copies rounded to TF32 (nearest).
 cudaError_t launch_first_leg_last(const float* T, float* TA, const int64_t* site_off, int n_sites,
-                                  int d, int chi, cudaStream_t s);
+                                  int d, int chi, cudaStream_t s, bool tf32 = false);
 
 // rho[site][p][p'] = sum_r X[p][r] conj(T[p'][r]) in FP64 (complex, 8 doubles
 // per site).  x_off / t_off: real-plane offsets; len = chi^d; plane = 2*len.
-// rho of n_sites sites; part: scratch of n_sites * 16 * 8 doubles.
+// rho of n_sites sites; part: scratch of n_sites * kRhoBlocks * 8 doubles.
+constexpr int kRhoBlocks = 32;
 cudaError_t launch_rho(const float* X, const float* T, const int64_t* x_off,
                        const int64_t* t_off, int n_sites, int64_t len, int64_t plane,
                        double* rho, double* part, cudaStream_t s);

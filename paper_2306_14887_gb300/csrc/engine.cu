@@ -51,7 +51,6 @@ struct HostLaunch {
   TcStreamPlan sp;         // maps set: the launch runs in a TMA kernel
   bool fuse_next = false;  // the next launch contracts this one's output (chain stages)
   bool skip = false;       // carried out by the previous launch's fused kernel
-  bool cuda_cores = false; // runs in the CUDA-core GEMM whatever the precision
   int tuned = 0;           // split-K count chosen by tn_autotune (0: the heuristic)
   std::vector<int> outer_site;  // sweep launches: the site of each outer entry
 };
@@ -353,7 +352,7 @@ tn_status upload_plans(tn_handle* h) {
       for (size_t li = 0; li < p->L.size(); ++li) {
         HostLaunch& L = p->L[li];
         TcStreamPlan sp;
-        if (L.skip || L.cuda_cores) continue;
+        if (L.skip) continue;
         // two chain stages in one pass: the intermediate never reaches HBM
         if (L.fuse_next && li + 1 < p->L.size()) {
           HostLaunch& L2 = p->L[li + 1];
@@ -509,7 +508,7 @@ tn_status run_plan(tn_handle* h, const Plan& P, int cls, size_t begin = 0,
     } else if (L.sp.maps) {
       TN_CUDA_TRY(launch_tc_stream(L.d, L.sp, h->flags, stream));
       h->stats.tma_launches++;
-    } else if (!L.cuda_cores && on_tile_kernel(h, L.d)) {
+    } else if (on_tile_kernel(h, L.d)) {
       TN_CUDA_TRY(launch_cgemm_tc(L.d, h->part, h->flags, stream, &nk, L.tuned, h->part_floats));
     } else {
       // a tiny-grid launch on the main stream may split K into the partial buffer
@@ -1032,13 +1031,14 @@ void build_rho_plan(tn_handle* h) {
   Plan& P = h->rho_prep;
   std::vector<Ent> a, b, c;
   if (h->mrt_tf32) {
-    // Y2 = T x_2 M2 x_1 M1 in the fused tensor-core kernel, Y1 = Y2 x_0 M0 on
-    // the CUDA cores.  Every operand is rounded to TF32 as the tile kernel
-    // rounds it (messages and intermediates to nearest before they are
-    // stored, T by the tensor core), so the products are the same.  At chi =
-    // 64 on 127 qubits the three products took 2.0 ms as strided tile GEMMs
-    // (operands staged element by element); fused they take 0.06 ms and the
-    // third one 0.3 ms (9.7 GFLOP at the FP32 rate, the larger part now).
+    // Degree 3: Y2 = T x_2 M2 x_1 M1 in the fused tensor-core kernel, Y1 = Y2
+    // with its first leg last, Y2 = Y1 x_0 M0 in the streaming kernel.  Degree 2:
+    // Y1 = T with its first leg last, Y2 = Y1 x_0 M0, Y1 = Y2 x_1 M1.  Every
+    // operand is rounded to TF32 as the tile kernel rounds it in the plain plan
+    // (messages, intermediates and transposed tensors to nearest before they are
+    // stored, T by the tensor core), so the products are the same.  At chi = 64 on
+    // 127 qubits the products took 2.0 ms as strided tile GEMMs (operands staged
+    // element by element) and take 0.20 ms so, two transposes included.
     const int64_t x = chi, x2 = x * x, x3 = x2 * x, plane = 2 * x3;
     auto m_in = [&](int v, int j) {
       const int e = g.legs[v][j];
@@ -1047,18 +1047,24 @@ void build_rho_plan(tn_handle* h) {
     for (int v : h->sites_by_deg[3]) {
       a.push_back({site_ptr(h, h->T, v), m_in(v, 2), site_ptr(h, h->Y1, v)});
       b.push_back({site_ptr(h, h->Y1, v), m_in(v, 1), site_ptr(h, h->Y2, v)});
-      c.push_back({site_ptr(h, h->Y2, v), m_in(v, 0), site_ptr(h, h->Y1, v)});
+      c.push_back({site_ptr(h, h->Y1, v), m_in(v, 0), site_ptr(h, h->Y2, v)});
     }
-    // the first two as in the first degree-3 chain: Y2 at a 2x^2 + p x^2 + b' x + c'
+    // the first two as in the first degree-3 chain, Y2 at p x^3 + a x^2 + b' x + c'
     add_spec(P, mode_spec(chi, plane, (int)(2 * x2), chi, 1, x2, x, 0, x2, 1, 0, x), prec, a);
-    if (!a.empty()) P.L.back().fuse_next = true;
-    add_spec(P, mode_spec(chi, plane, (int)(2 * x2), chi, chi, x3, x2, x, x2, 2 * x2, 1, x), prec, b);
-    if (!a.empty()) P.L.back().d.round_c = 1;
-    // rows (p, bc) contiguous on both sides, the contracted leg a at stride 2x^2
-    Spec sp = mode_spec(chi, plane, (int)(2 * x2), (int)x2, 1, x2, 1, 0, x3, 1, 0, x2);
-    sp.a_k2 = 2 * x2;
-    add_spec(P, sp, prec, c);
-    if (!a.empty()) P.L.back().cuda_cores = true;
+    P.L.back().fuse_next = true;
+    add_spec(P, mode_spec(chi, plane, (int)(2 * x2), chi, chi, x3, x2, x, x3, x2, 1, x), prec, b);
+    P.L.back().d.round_c = 1;
+    // rows (p, bc) of Y1[p][bc][a], the output at p x^3 + a' x^2 + bc
+    add_spec(P, mode_spec(chi, plane, (int)(2 * x2), (int)x2, 1, x3, x, 0, x3, 1, 0, x2), prec, c);
+    a.clear(); b.clear(); c.clear();
+    for (int v : h->sites_by_deg[2]) {
+      a.push_back({site_ptr(h, h->Y1, v), m_in(v, 0), site_ptr(h, h->Y2, v)});
+      b.push_back({site_ptr(h, h->Y2, v), m_in(v, 1), site_ptr(h, h->Y1, v)});
+    }
+    // rows (p, b) of Y1[p][b][a], then (p, a') of Y2[p][a'][b]
+    add_spec(P, mode_spec(chi, 2 * x2, 2 * chi, chi, 1, x2, x, 0, x2, 1, 0, x), prec, a);
+    add_spec(P, mode_spec(chi, 2 * x2, 2 * chi, chi, 1, x2, x, 0, x2, x, 0, 1), prec, b);
+    a.clear(); b.clear();
   } else {
     // degree 3: Y1 = T x_2 M2 ; Y2 = Y1 x_1 M1 ; Y1 = Y2 x_0 M0
     for (int v : h->sites_by_deg[3]) {
@@ -1074,6 +1080,7 @@ void build_rho_plan(tn_handle* h) {
   a.clear(); b.clear();
   // degree 2: Y1 = T x_0 M0 ; Y2 = Y1 x_1 M1 -> result in Y2, copy pointer for rho
   for (int v : h->sites_by_deg[2]) {
+    if (h->mrt_tf32) break;
     const auto& lg = g.legs[v];
     a.push_back({site_ptr(h, h->T, v), in_msg(h, v, lg[0]), site_ptr(h, h->Y2, v)});
     b.push_back({site_ptr(h, h->Y2, v), in_msg(h, v, lg[1]), site_ptr(h, h->Y1, v)});
@@ -1084,7 +1091,7 @@ void build_rho_plan(tn_handle* h) {
   for (int v : h->sites_by_deg[1])
     a.push_back({site_ptr(h, h->T, v), in_msg(h, v, g.legs[v][0]), site_ptr(h, h->Y1, v)});
   add_mode_product(P, 1, 0, chi, prec, a);
-  // every degree ends with X in Y1
+  // every degree ends with X in Y1 (degree 3 of the fused products: in Y2)
   for (int d = 1; d <= 3; ++d) {
     if (h->sites_by_deg[d].empty()) continue;
     RhoLaunch r;
@@ -1578,12 +1585,23 @@ tn_status bp_converge_impl(tn_handle* h, double tol, int max_iters, int* iters, 
 }
 
 tn_status compute_rho(tn_handle* h, std::vector<double>* rho_out) {
+  tn_status st;
   if (h->mrt_tf32) {
-    TN_CUDA_TRY(launch_realify(h->msg, 2LL * h->chi * h->chi, h->mrt_tf32,
-                               2 * (int)h->g.eu.size(), h->chi, h->stream, true));
-    h->stats.kernel_launches++;
+    st = ensure_mrt(h);
+    if (st) return st;
+    const int64_t n_mrt = 2LL * h->g.eu.size() * 4 * h->chi * h->chi;
+    TN_CUDA_TRY(launch_round_tf32(h->mrt, h->mrt_tf32, n_mrt, h->stream));
+    st = run_plan(h, h->rho_prep, P_RHO, 0, 2);
+    if (st) return st;
+    TN_CUDA_TRY(launch_first_leg_last(h->Y2, h->Y1, h->site_offs_by_deg[3], h->n_by_deg[3], 3,
+                                      h->chi, h->stream));
+    TN_CUDA_TRY(launch_first_leg_last(h->T, h->Y1, h->site_offs_by_deg[2], h->n_by_deg[2], 2,
+                                      h->chi, h->stream, true));
+    h->stats.kernel_launches += 2 + (h->n_by_deg[2] > 0);
+    st = run_plan(h, h->rho_prep, P_RHO, 2);
+  } else {
+    st = run_plan(h, h->rho_prep, P_RHO);
   }
-  tn_status st = run_plan(h, h->rho_prep, P_RHO);
   if (st) return st;
   const int n = h->g.n;
   int base = 0;
@@ -1591,8 +1609,9 @@ tn_status compute_rho(tn_handle* h, std::vector<double>* rho_out) {
   for (auto& r : h->rho_l) {
     const int64_t len = ipow(h->chi, r.deg);
     const int pi = prof_begin(h, P_RHO);
-    TN_CUDA_TRY(launch_rho(h->Y1, h->T, r.d_x, r.d_t, (int)r.sites.size(), len, 2 * len,
-                           h->rho + 8 * base, h->rho_part, h->stream));
+    TN_CUDA_TRY(launch_rho(h->mrt_tf32 && r.deg == 3 ? h->Y2 : h->Y1, h->T, r.d_x, r.d_t,
+                           (int)r.sites.size(), len, 2 * len, h->rho + 8 * base, h->rho_part,
+                           h->stream));
     prof_end(h, pi, 32.0 * len * r.sites.size(), 2.0 * 16.0 * len * r.sites.size());
     h->stats.kernel_launches += 2;
     for (int v : r.sites) order.push_back(v);
@@ -1850,7 +1869,7 @@ tn_status tn_create(const tn_graph* graph, const tn_config* cfg, const tn_alloca
   h->loop_par = (double*)dev_alloc(h, sizeof(double) * 4);
   h->loop_out = (unsigned long long*)dev_alloc(h, sizeof(unsigned long long) * 8);
   h->rho = (double*)dev_alloc(h, sizeof(double) * 8 * g.n);
-  h->rho_part = (double*)dev_alloc(h, sizeof(double) * 16 * 8 * std::max(1, g.n));
+  h->rho_part = (double*)dev_alloc(h, sizeof(double) * kRhoBlocks * 8 * std::max(1, g.n));
   for (int d = 1, base = 0; d <= 3; ++d) {
     h->n_by_deg[d] = (int)h->sites_by_deg[d].size();
     h->site_offs_by_deg[d] = (int64_t*)dev_alloc(h, sizeof(int64_t) * (h->n_by_deg[d] + 1));

@@ -368,7 +368,6 @@ __global__ void dot_msgs_kernel(const float* R, const float* M, int chi, double*
 }
 
 // Realified transposed copies (see GemmDesc::b_pre).
-template <bool TF32>
 __global__ void realify_kernel(const float* src, int64_t stride, float* dst, int chi) {
   const int64_t n2 = (int64_t)chi * chi;
   const float* a = src + blockIdx.y * stride;
@@ -377,11 +376,7 @@ __global__ void realify_kernel(const float* src, int64_t stride, float* dst, int
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n2;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(idx / chi), j = (int)(idx - (int64_t)i * chi);  // element [k = i][n = j]
-    float re = a[idx], im = a[n2 + idx];
-    if (TF32) {
-      re = __uint_as_float(tc::to_tf32(re));
-      im = __uint_as_float(tc::to_tf32(im));
-    }
+    const float re = a[idx], im = a[n2 + idx];
     q[(int64_t)j * w + i] = re;
     q[(int64_t)(chi + j) * w + chi + i] = re;
     q[(int64_t)(chi + j) * w + i] = im;
@@ -392,6 +387,7 @@ __global__ void realify_kernel(const float* src, int64_t stride, float* dst, int
 // TA[pl][p][rest][l0] = T[pl][p][l0][rest]: per (site, plane, p) a chi x rest
 // matrix transposed through a padded 32 x 33 shared tile, so that both the
 // reads (along rest) and the writes (along l0) are row-contiguous.
+template <bool TF32>
 __global__ void first_leg_last_kernel(const float* T, float* TA, const int64_t* site_off,
                                       int chi, int64_t rest) {
   __shared__ float tile[32][33];
@@ -411,7 +407,17 @@ __global__ void first_leg_last_kernel(const float* T, float* TA, const int64_t* 
   for (int i = ty; i < 32; i += 8) {
     const int64_t r = r0 + i;
     const int l0 = l00 + tx;
-    if (r < rest && l0 < chi) dst[r * chi + l0] = tile[tx][i];
+    if (r < rest && l0 < chi)
+      dst[r * chi + l0] = TF32 ? __uint_as_float(tc::to_tf32(tile[tx][i])) : tile[tx][i];
+  }
+}
+
+__global__ void round_tf32_kernel(const float4* src, float4* dst, int64_t n4) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n4;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const float4 v = src[i];
+    dst[i] = make_float4(__uint_as_float(tc::to_tf32(v.x)), __uint_as_float(tc::to_tf32(v.y)),
+                         __uint_as_float(tc::to_tf32(v.z)), __uint_as_float(tc::to_tf32(v.w)));
   }
 }
 
@@ -457,26 +463,34 @@ cudaError_t launch_dot_msgs(const float* R, const float* M, int chi, double* out
 }
 
 cudaError_t launch_realify(const float* src, int64_t src_stride, float* dst, int n, int chi,
-                           cudaStream_t s, bool tf32) {
+                           cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int64_t n2 = (int64_t)chi * chi;
   int64_t bx = (n2 + 255) / 256;
   if (bx > 64) bx = 64;
   dim3 grid((unsigned)bx, n);
-  if (tf32) realify_kernel<true><<<grid, 256, 0, s>>>(src, src_stride, dst, chi);
-  else realify_kernel<false><<<grid, 256, 0, s>>>(src, src_stride, dst, chi);
+  realify_kernel<<<grid, 256, 0, s>>>(src, src_stride, dst, chi);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_round_tf32(const float* src, float* dst, int64_t n, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  if (n % 4) return cudaErrorInvalidValue;
+  const int64_t blocks = std::min<int64_t>((n / 4 + 255) / 256, 8 * 152);
+  round_tf32_kernel<<<(unsigned)blocks, 256, 0, s>>>(reinterpret_cast<const float4*>(src),
+                                                     reinterpret_cast<float4*>(dst), n / 4);
   return cudaGetLastError();
 }
 
 cudaError_t launch_first_leg_last(const float* T, float* TA, const int64_t* site_off, int n_sites,
-                                  int d, int chi, cudaStream_t s) {
+                                  int d, int chi, cudaStream_t s, bool tf32) {
   if (n_sites <= 0 || d < 2) return cudaSuccess;
   int64_t rest = 1;
   for (int i = 1; i < d; ++i) rest *= chi;
   if (4LL * n_sites > 65535) return cudaErrorInvalidValue;
   // site offsets are multiples of 4 floats (whole planes of chi^d values, chi
   // even) when chi % 32 == 0; the base pointers come from 256-byte allocations
-  const bool wide = rest % 128 == 0 && chi % 32 == 0 &&
+  const bool wide = !tf32 && rest % 128 == 0 && chi % 32 == 0 &&
                     ((reinterpret_cast<uintptr_t>(T) | reinterpret_cast<uintptr_t>(TA)) & 15) == 0;
   if (wide) {
     dim3 grid((unsigned)(rest / 128), (unsigned)(chi / 32), (unsigned)(4 * n_sites));
@@ -484,7 +498,8 @@ cudaError_t launch_first_leg_last(const float* T, float* TA, const int64_t* site
     return cudaGetLastError();
   }
   dim3 grid((unsigned)((rest + 31) / 32), (unsigned)((chi + 31) / 32), (unsigned)(4 * n_sites));
-  first_leg_last_kernel<<<grid, dim3(32, 8), 0, s>>>(T, TA, site_off, chi, rest);
+  if (tf32) first_leg_last_kernel<true><<<grid, dim3(32, 8), 0, s>>>(T, TA, site_off, chi, rest);
+  else first_leg_last_kernel<false><<<grid, dim3(32, 8), 0, s>>>(T, TA, site_off, chi, rest);
   return cudaGetLastError();
 }
 
@@ -556,14 +571,12 @@ __device__ __forceinline__ void pair_add_prod(float& s, float& c, float a, float
 // second kernel adds the blocks in a fixed order in FP64.
 __global__ void rho_part_kernel(const float* X, const float* T, const int64_t* x_off,
                                 const int64_t* t_off, int64_t len, int64_t plane, double* part) {
-  __shared__ double sh[32];
+  __shared__ double sh[8 * 8];  // [warp][component], at most 8 warps
   const float* x = X + x_off[blockIdx.y];
   const float* t = T + t_off[blockIdx.y];
   float s[8] = {0, 0, 0, 0, 0, 0, 0, 0}, c[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const float x0r = x[i], x0i = x[plane + i], x1r = x[len + i], x1i = x[plane + len + i];
-    const float t0r = t[i], t0i = t[plane + i], t1r = t[len + i], t1i = t[plane + len + i];
+  auto add = [&](float x0r, float x0i, float x1r, float x1i, float t0r, float t0i, float t1r,
+                 float t1i) {
     // x_p conj(t_q) = (xr tr + xi ti) + i (xi tr - xr ti)
     pair_add_prod(s[0], c[0], x0r, t0r); pair_add_prod(s[0], c[0], x0i, t0i);
     pair_add_prod(s[1], c[1], x0i, t0r); pair_add_prod(s[1], c[1], -x0r, t0i);
@@ -573,28 +586,75 @@ __global__ void rho_part_kernel(const float* X, const float* T, const int64_t* x
     pair_add_prod(s[5], c[5], x1i, t0r); pair_add_prod(s[5], c[5], -x1r, t0i);
     pair_add_prod(s[6], c[6], x1r, t1r); pair_add_prod(s[6], c[6], x1i, t1i);
     pair_add_prod(s[7], c[7], x1i, t1r); pair_add_prod(s[7], c[7], -x1r, t1i);
+  };
+  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  if (len % 4 == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(t)) & 15) == 0) {
+    // sixteen bytes of each of the eight planes in flight per thread
+    const int64_t l4 = len / 4, p4 = plane / 4;
+    const float4* x4 = reinterpret_cast<const float4*>(x);
+    const float4* t4 = reinterpret_cast<const float4*>(t);
+    for (int64_t i = first; i < l4; i += step) {
+      const float4 a0 = x4[i], a1 = x4[p4 + i], a2 = x4[l4 + i], a3 = x4[p4 + l4 + i];
+      const float4 b0 = t4[i], b1 = t4[p4 + i], b2 = t4[l4 + i], b3 = t4[p4 + l4 + i];
+      add(a0.x, a1.x, a2.x, a3.x, b0.x, b1.x, b2.x, b3.x);
+      add(a0.y, a1.y, a2.y, a3.y, b0.y, b1.y, b2.y, b3.y);
+      add(a0.z, a1.z, a2.z, a3.z, b0.z, b1.z, b2.z, b3.z);
+      add(a0.w, a1.w, a2.w, a3.w, b0.w, b1.w, b2.w, b3.w);
+    }
+  } else {
+    for (int64_t i = first; i < len; i += step)
+      add(x[i], x[plane + i], x[len + i], x[plane + len + i], t[i], t[plane + i], t[len + i],
+          t[plane + len + i]);
   }
-  for (int k = 0; k < 8; ++k) {
-    const double v = block_sum((double)s[k] + (double)c[k], sh);
-    if (threadIdx.x == 0) part[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * 8 + k] = v;
+  // The eight sums over the block in FP64, in a fixed order.  Within a warp the
+  // values are shared out over the lanes while they are added (component lane &
+  // 7 after three steps), nine additions instead of forty: the FP64 pipe takes a
+  // warp's addition for 16 clocks.
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double v[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = (double)s[k] + (double)c[k];
+#pragma unroll
+  for (int half = 4; half > 0; half >>= 1)
+#pragma unroll
+    for (int k = 0; k < half; ++k) {
+      const bool up = lane & half;
+      const double keep = up ? v[k + half] : v[k], give = up ? v[k] : v[k + half];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, give, half);
+    }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 8);
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
+  if (lane < 8) sh[warp * 8 + lane] = v[0];
+  __syncthreads();
+  if (threadIdx.x < 8) {
+    double t = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w * 8 + threadIdx.x];
+    part[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * 8 + threadIdx.x] = t;
   }
 }
 
+// One warp per (site, component): lane b sums blocks b, b + 32, ..; a fixed order.
 __global__ void rho_sum_kernel(const double* part, int nblk, int n_sites, double* rho) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;  // (site, component)
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (i >= 8 * n_sites) return;
   const int site = i / 8, k = i % 8;
   double v = 0.0;
-  for (int b = 0; b < nblk; ++b) v += part[((int64_t)site * nblk + b) * 8 + k];
-  rho[i] = v;
+  for (int b = lane; b < nblk; b += 32) v += part[((int64_t)site * nblk + b) * 8 + k];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) rho[i] = v;
 }
 }  // namespace
 
+// Blocks per site: the reads of both tensors are bound by what is in flight, so
+// the sites together get about eight blocks an SM, at most kRhoBlocks each.  At
+// chi = 64 on 127 qubits 2 x 151 MB take 66 us, 70 % of the issue slots (155 us with
+// 4-byte reads, 256 us with two blocks an SM and the sums reduced one by one).
 int rho_blocks(int n_sites, int64_t len) {
-  int nblk = (2 * 152 + n_sites - 1) / n_sites;
+  int nblk = (8 * 152 + n_sites - 1) / n_sites;
   const int64_t most = (len + 255) / 256;
   if (nblk > most) nblk = (int)most;
-  if (nblk > 16) nblk = 16;
+  if (nblk > kRhoBlocks) nblk = kRhoBlocks;
   return nblk < 1 ? 1 : nblk;
 }
 
@@ -606,7 +666,7 @@ cudaError_t launch_rho(const float* X, const float* T, const int64_t* x_off,
   rho_part_kernel<<<dim3(nblk, n_sites), 256, 0, s>>>(X, T, x_off, t_off, len, plane, part);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  rho_sum_kernel<<<(8 * n_sites + 255) / 256, 256, 0, s>>>(part, nblk, n_sites, rho);
+  rho_sum_kernel<<<(8 * n_sites + 7) / 8, 256, 0, s>>>(part, nblk, n_sites, rho);
   return cudaGetLastError();
 }
 
