@@ -1473,6 +1473,7 @@ bool splits_valid(const tn_handle* h, const HostLaunch& L, int kind, int s) {
   if (pf > h->part_floats) return false;
   if (kind == TUNE_CLOSE) {
     const int chunks = L.d.K1 * L.d.K2 / 32;
+    if (L.d.N == 32) return s >= 2 && s <= 64 && s % 2 == 0 && chunks % s == 0;
     const int per = (chunks + s - 1) / s;
     return s >= 1 && s <= 64 && (chunks + per - 1) / per == s;  // no empty split
   }

@@ -294,10 +294,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_stream_kernel(GemmDesc d, Stre
 }
 
 // ---------------------------------------------------------------- closes
-// out[m][n] = sum_K A[m][K] op(B[n][K]) with M = N = 64 (the message's two
+// out[m][n] = sum_K A[m][K] op(B[n][K]) with M = N = chi (the message's two
 // indices), both operands K-contiguous site tensors: per K chunk of 32 the
 // tile is [(s, m)][32] of A and [(t, n)][32] of B (s, t the re/im planes, so
-// the 128 x 128 product holds all four real products P_st), streamed by TMA
+// the 128 x 128 product at chi = 64 holds all four real products P_st; at chi =
+// 32 a CTA stacks the chunks of two K splits, cut as the tile kernel cuts them,
+// and only their own blocks are read: the same partial sums as there), streamed by TMA
 // through a 3-stage ring; K is split over CTAs, two CTAs per SM.  The
 // epilogue stages P in shared memory, combines C_re = P_rr - sa sb P_ii,
 // C_im = sb P_ri + sa P_ir and writes the CTA's partial; a second kernel sums
@@ -317,7 +319,9 @@ struct CloseArgs {
   int* err;
 };
 
+template <int CHI>
 __global__ void __launch_bounds__(kCThreads, 2) tc_close_kernel(GemmDesc d, CloseArgs a) {
+  constexpr int H = 64 / CHI, C2 = CHI * CHI;  // K splits a CTA carries; outputs
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -332,8 +336,9 @@ __global__ void __launch_bounds__(kCThreads, 2) tc_close_kernel(GemmDesc d, Clos
   // a converged component of a union: nothing is initialised yet, the whole
   // CTA leaves together (its partial is never read: the reduce skips it too)
   if (outer_frozen(d, e / d.n_inner)) return;
-  const int c0 = split * a.per_split;
-  const int c1 = min(a.chunks, c0 + a.per_split);
+  // chunks of the CTA's first split; with two splits both are whole
+  const int c0 = split * H * a.per_split;
+  const int c1 = H == 1 ? min(a.chunks, c0 + a.per_split) : c0 + a.per_split;
   const int nt = c1 > c0 ? c1 - c0 : 0;  // >= 1 by the host's choice of splits
 
   if (tid == 0) {
@@ -366,11 +371,14 @@ __global__ void __launch_bounds__(kCThreads, 2) tc_close_kernel(GemmDesc d, Clos
         const int slot = i % kCStages;
         if (!mbar_wait(&empty[slot], ((i / kCStages) & 1) ^ 1, a.err)) { *abort_flag = 1; break; }
         mbar_expect_tx(&full[slot], (uint32_t)(2 * kChunk));
-        const int k = (c0 + i) * 32;
-        const int k1 = k / a.K2, k2 = k - k1 * a.K2;
         const uint32_t dst = smem_u32(smem + slot * kCStage);
-        tma_load_4d(dst, amap, k2, 0, k1, 0, &full[slot]);
-        tma_load_4d(dst + kChunk, bmap, k2, 0, k1, 0, &full[slot]);
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const int k = (c0 + h * a.per_split + i) * 32;
+          const int k1 = k / a.K2, k2 = k - k1 * a.K2;
+          tma_load_4d(dst + h * (kChunk / H), amap, k2, 0, k1, 0, &full[slot]);
+          tma_load_4d(dst + kChunk + h * (kChunk / H), bmap, k2, 0, k1, 0, &full[slot]);
+        }
         ++issued[slot];
       }
       for (int s = 0; s < kCStages; ++s)
@@ -404,24 +412,25 @@ __global__ void __launch_bounds__(kCThreads, 2) tc_close_kernel(GemmDesc d, Clos
     // P staged in the (now idle) pipeline buffers: [128 rows][129]
     float* P = reinterpret_cast<float*>(smem);
     const int q = warp & 3, row = q * 32 + lane;
+    const int cb = H == 1 ? 0 : row / 64 * 64;  // a chunk's rows meet its own columns only
 #pragma unroll
-    for (int c = 0; c < 128; c += 32) {
+    for (int c = 0; c < 128 / H; c += 32) {
       float v[32];
-      tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c, v);
+      tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(cb + c), v);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) P[row * 129 + c + j] = v[j];
+      for (int j = 0; j < 32; ++j) P[row * 129 + cb + c + j] = v[j];
     }
     asm volatile("bar.sync 1, 128;" ::: "memory");
     const float sa = d.conj_a ? -1.f : 1.f, sb = d.conj_b ? -1.f : 1.f;
-    float* out = a.part + ((int64_t)split * a.n_outer + e) * 2 * 4096;
     const int outer = e / d.n_inner, inner = e - outer * d.n_inner;
     float* C = d.C[outer] + inner * d.c_in;
-    for (int idx = tid - 64; idx < 4096; idx += 128) {
-      const int m = idx >> 6, n = idx & 63;
+    for (int idx = tid - 64; idx < H * C2; idx += 128) {
+      const int h = idx / C2, o = idx - h * C2, m = o / CHI, n = o % CHI;
       float cr = 0.f, ci = 0.f;
       if (ok) {
-        const float prr = P[m * 129 + n], pii = P[(64 + m) * 129 + 64 + n];
-        const float pri = P[m * 129 + 64 + n], pir = P[(64 + m) * 129 + n];
+        const float* q0 = P + (h * 64 + m) * 129 + h * 64 + n;
+        const float prr = q0[0], pii = q0[CHI * 129 + CHI];
+        const float pri = q0[CHI], pir = q0[CHI * 129];
         cr = prr - sa * sb * pii;
         ci = sb * pri + sa * pir;
       }
@@ -430,8 +439,9 @@ __global__ void __launch_bounds__(kCThreads, 2) tc_close_kernel(GemmDesc d, Clos
         pc[0] = cr;
         pc[d.plane_c] = ci;
       } else {
-        out[idx] = cr;
-        out[4096 + idx] = ci;
+        float* out = a.part + ((int64_t)(split * H + h) * a.n_outer + e) * 2 * C2;
+        out[o] = cr;
+        out[C2 + o] = ci;
       }
     }
   }
@@ -931,12 +941,12 @@ cudaError_t tc_stream_prepare() {
     if (result == cudaSuccess)
       result = cudaFuncSetAttribute(tc_chain_kernel<64>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, kFSmemBytes);
-    if (result == cudaSuccess)
-      result = cudaFuncSetAttribute(tc_close_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    kCSmemBytes);
-    if (result == cudaSuccess)
-      result = cudaFuncSetAttribute(tc_close_kernel,
-                                    cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    for (auto k : {tc_close_kernel<32>, tc_close_kernel<64>}) {
+      if (result == cudaSuccess)
+        result = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kCSmemBytes);
+      if (result == cudaSuccess)
+        result = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    }
     int dev = 0, sms = 0;
     if (result == cudaSuccess) result = cudaGetDevice(&dev);
     if (result == cudaSuccess)
@@ -969,7 +979,8 @@ cudaError_t launch_tc_stream(const GemmDesc& d, const TcStreamPlan& p, int* err,
 
 bool tc_close_encode(const GemmDesc& d, const float* const* A, const float* const* B, int n_outer,
                      size_t part_floats, void* host_maps, TcStreamPlan* p) {
-  if (d.prec != TN_TF32 || d.b_pre || d.M != 64 || d.N != 64 || d.a_k2 != 1 || d.b_k2 != 1 ||
+  const int chi = d.N;
+  if (d.prec != TN_TF32 || d.b_pre || (chi != 64 && chi != 32) || d.M != chi || d.a_k2 != 1 || d.b_k2 != 1 ||
       d.n_inner < 1 || d.K2 % 32 || d.M2 > 1 || d.M3 > 1 || d.accumulate || n_outer < 1)
     return false;
   // entries (outer, inner) in the order the partial buffer and the reduce use
@@ -983,13 +994,24 @@ bool tc_close_encode(const GemmDesc& d, const float* const* A, const float* cons
     if (s_a[i] <= 0 || s_b[i] <= 0 || (s_a[i] * 4) % 16 || (s_b[i] * 4) % 16) return false;
   const int chunks = d.K1 * d.K2 / 32;
   int S = 1;
-  while ((int64_t)n_ent * S * 2 <= 2LL * g_num_sms && chunks / (S * 2) >= 4) S *= 2;
-  const int per = (chunks + S - 1) / S;
-  S = (chunks + per - 1) / per;  // every split holds at least one chunk
-  if ((size_t)S * n_ent * 2 * 4096 > part_floats) return false;
+  if (chi == 32) {
+    // an even number of equal splits, two to a CTA.  The accumulation order is
+    // the tile kernel's: the tensor core truncates its running sums, so another
+    // cut of K moves a message by about 1e-5.  433 sites: 27 us a launch, 70 us
+    // in the tile kernel.
+    int quad = 0;
+    size_t pf = 0;
+    tc_plan(d, &quad, &S, &pf);
+    if (S % 2 || chunks % S) return false;
+  } else {
+    while ((int64_t)n_ent * S * 2 <= 2LL * g_num_sms && chunks / (S * 2) >= 4) S *= 2;
+    const int per = (chunks + S - 1) / S;
+    S = (chunks + per - 1) / per;  // every split holds at least one chunk
+  }
+  if ((size_t)S * n_ent * 2 * chi * chi > part_floats) return false;
   CUtensorMap* maps = reinterpret_cast<CUtensorMap*>(host_maps);
   const cuuint32_t estr[4] = {1, 1, 1, 1};
-  const cuuint32_t box[4] = {32, 64, 1, 2};
+  const cuuint32_t box[4] = {32, (cuuint32_t)chi, 1, 2};
   if ((d.a_in * 4) % 16 || (d.b_in * 4) % 16) return false;
   for (int e = 0; e < n_ent; ++e) {
     const int o = e / d.n_inner, in = e - o * d.n_inner;
@@ -997,7 +1019,7 @@ bool tc_close_encode(const GemmDesc& d, const float* const* A, const float* cons
     const float* Be = B[o] + (int64_t)in * d.b_in;
     if ((reinterpret_cast<uintptr_t>(Ae) & 15) || (reinterpret_cast<uintptr_t>(Be) & 15))
       return false;
-    cuuint64_t dims[4] = {(cuuint64_t)d.K2, 64, (cuuint64_t)d.K1, 2};
+    cuuint64_t dims[4] = {(cuuint64_t)d.K2, (cuuint64_t)chi, (cuuint64_t)d.K1, 2};
     cuuint64_t sa[3] = {(cuuint64_t)(s_a[0] * 4), (cuuint64_t)(s_a[1] * 4),
                         (cuuint64_t)(s_a[2] * 4)};
     cuuint64_t sb[3] = {(cuuint64_t)(s_b[0] * 4), (cuuint64_t)(s_b[1] * 4),
@@ -1033,8 +1055,9 @@ cudaError_t launch_tc_close(const GemmDesc& d, const TcStreamPlan& p, float* par
   a.direct = p.splits == 1 ? 1 : 0;
   a.part = part;
   a.err = err;
-  dim3 grid(p.splits, p.n_outer);
-  tc_close_kernel<<<grid, kCThreads, kCSmemBytes, st>>>(d, a);
+  dim3 grid(d.N == 64 ? p.splits : p.splits / 2, p.n_outer);
+  if (d.N == 64) tc_close_kernel<64><<<grid, kCThreads, kCSmemBytes, st>>>(d, a);
+  else tc_close_kernel<32><<<grid, kCThreads, kCSmemBytes, st>>>(d, a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || a.direct) return e;
   return launch_tc_reduce(d, part, p.splits, st);
