@@ -104,11 +104,11 @@ cudaError_t simt_prepare();  // kernel attributes, once, before any stream captu
 cudaError_t launch_cgemm(const GemmDesc& d, cudaStream_t s, float* part = nullptr,
                          size_t part_cap = 0, int* n_kernels = nullptr, int force_splits = 0);
 // One site's chain to one open leg (site_sweep.cu): the message contractions of
-// a BP sweep at chi <= 16 in one launch, FP32, the same sums as the CUDA-core
-// GEMM.  Degree 3: open-leg values o0 .. o0 + on - 1 (at most
+// a BP sweep at chi <= 24 in one launch, FP32, summed as the CUDA-core GEMM sums
+// them.  Degree 3: open-leg values o0 .. o0 + on - 1 (at most
 // site_sweep_open(chi)); mf, mg the incoming messages (planar chi x chi) on the
 // first and second contracted legs.  splits: the split-K counts of the three
-// degree-3 closes; comp_state: as in GemmDesc (null: no skipping).
+// degree-3 closes (used up to chi = 16); comp_state: as in GemmDesc (null: no skipping).
 struct SiteJob {
   const float *T, *mf, *mg;
   float* out;

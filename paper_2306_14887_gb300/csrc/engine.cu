@@ -134,7 +134,7 @@ struct tn_handle {
   // degree-2 chains and degree-1 closes, which share no scratch with the
   // degree-3 chains) runs beside sweep.L[..sweep_split].
   size_t sweep_split = 0;
-  // chi <= 16 on the CUDA cores: the sweep's contractions as one launch (one job
+  // chi <= 24 on the CUDA cores: the sweep's contractions as one launch (one job
   // per site, open leg and block of open-leg values) instead of sweep.L
   tnbp::SiteJob* site_jobs = nullptr;
   int n_site_jobs = 0;

@@ -1,4 +1,4 @@
-// One BP sweep's message contractions for small bond dimensions (chi <= 16) in
+// One BP sweep's message contractions for small bond dimensions (chi <= 24) in
 // one launch, FP32: every CTA carries one site's chain to one open leg (two mode
 // products and the close) through shared memory.
 //
@@ -10,7 +10,7 @@
 // 16 46 us (147 us as separate GEMM launches), 338 sites at chi = 16 79 us (201),
 // 65 sites at chi = 9 24 us (173 with the GEMM before its rewrite).
 //
-// Every sum is taken exactly as the CUDA-core GEMM takes it (16-deep slices of
+// Up to chi = 16 every sum is taken exactly as the CUDA-core GEMM takes it (16-deep slices of
 // the contraction in the same order, slice sums added by compensated two-sums,
 // split-K parts added in FP64), so the messages are the same bit for bit.
 //
@@ -31,7 +31,8 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kMaxChi = 16;
+constexpr int kMaxChi = 16;        // the site tensor fits twice into an SM
+constexpr int kStreamMaxChi = 24;  // rows of a slab a warp holds
 constexpr int kOpen = 8;      // open-leg values per degree-3 CTA: two CTAs per site and leg at
                               // chi = 16, two of them on an SM
 constexpr int kSlice = 16;    // slice depth of the CUDA-core GEMM
@@ -296,17 +297,378 @@ size_t smem_floats(int chi) {
   return 2 * 2 * (size_t)chi * chi * ld + 4 * (size_t)chi * chi + 2 * 2 * (size_t)kOpen * chi * ld;
 }
 
+// --- chi = 17 .. 24 ---------------------------------------------------------
+// T and the messages no longer fit an SM beside a block of slabs: a CTA of 16 warps
+// holds its slabs (one per warp, interleaved complex, 77 KB at chi = 24), and the
+// close streams T through two stages of 256 contraction indices, one 16-deep slice
+// per warp and stage.  Bound by the issue of the products' operand reads and of the
+// transposing 4-byte copies.  A whole sweep with normalisation and stop rule, before
+// (eight GEMM launches) and now: 65 sites at chi = 17 181 and 63 us, 22 224 and 74,
+// 23 184 and 83; 127 qubits at chi = 23 255 and 134; 338 sites at chi = 24 490 and
+// 391.  Two CTAs of eight warps per SM took 71, 96, 97, 133 and 454.
+// Every product is summed as above.  The close is one chain of compensated sums:
+// split-K parts, each rounded to FP32 and added in FP64, kept the FP64 units busy
+// for as long as the products took.
+// Above chi = 24 the GEMM launches have work enough: the same scheme with one slab
+// pair per warp took 157 us against 194 at chi = 28 but 259 against 267 at chi = 32.
+constexpr int kStreamThreads = 512, kStreamWarps = kStreamThreads / 32;
+constexpr int kStageK = kStreamWarps * kSlice;
+constexpr int kStageLd = kStageK + 1;  // float2 per o' row of a stage
+
+// kRI x kCJ values of a slab per lane (4 x 8 lanes), kOI x kPJ of a close (kOL lanes
+// along the open leg, 8 along o').
+constexpr int kRI = 6, kCJ = 3, kOL = 4, kOI = 2, kPJ = 3;
+
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_wait_all() {
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+// y <- (y M)^T of one slab (rows x contracted, interleaved complex, in place):
+// two 16-deep slices at most, whose compensated sum is their rounded sum.
+// M's entries are (re, im, -im, re).
+__device__ __forceinline__ void slab_product(float2* y, const float4* M, int chi, int ld) {
+  const int lane = threadIdx.x & 31, rg = lane >> 3, cg = lane & 7;
+  int row[kRI], col[kCJ];
+#pragma unroll
+  for (int i = 0; i < kRI; ++i) row[i] = min(rg + 4 * i, chi - 1) * ld;
+#pragma unroll
+  for (int j = 0; j < kCJ; ++j) col[j] = min(cg + 8 * j, chi - 1);
+  float2 acc[kRI][kCJ], head[kRI][kCJ];
+#pragma unroll
+  for (int i = 0; i < kRI; ++i)
+#pragma unroll
+    for (int j = 0; j < kCJ; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  for (int k0 = 0; k0 < chi; k0 += kSlice) {
+    if (k0 == kSlice)
+#pragma unroll
+      for (int i = 0; i < kRI; ++i)
+#pragma unroll
+        for (int j = 0; j < kCJ; ++j) {
+          head[i][j] = acc[i][j];
+          acc[i][j] = make_float2(0.f, 0.f);
+        }
+    const int kend = min(chi, k0 + kSlice);
+    for (int k = k0; k < kend; ++k) {
+      float2 a[kRI];
+#pragma unroll
+      for (int i = 0; i < kRI; ++i) a[i] = y[row[i] + k];
+#pragma unroll
+      for (int j = 0; j < kCJ; ++j) {
+        const float4 b = M[k * chi + col[j]];
+#pragma unroll
+        for (int i = 0; i < kRI; ++i)
+          acc[i][j] = __ffma2_rn(make_float2(a[i].x, a[i].x), make_float2(b.x, b.y), acc[i][j]);
+#pragma unroll
+        for (int i = 0; i < kRI; ++i)
+          acc[i][j] = __ffma2_rn(make_float2(a[i].y, a[i].y), make_float2(b.z, b.w), acc[i][j]);
+      }
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < kRI; ++i)
+#pragma unroll
+    for (int j = 0; j < kCJ; ++j) {
+      const int r = rg + 4 * i, c = cg + 8 * j;
+      if (r < chi && c < chi)
+        y[c * ld + r] = make_float2(__fadd_rn(head[i][j].x, acc[i][j].x),
+                                    __fadd_rn(head[i][j].y, acc[i][j].y));
+    }
+  __syncwarp();
+}
+
+// One site of degree 1 or 2 (T[p, o, f]), the chains of site_sweep_kernel with a
+// 2 x 4 tile of the product and a 2 x 2 tile of the close per thread.
+__device__ void stream_low_degree(const SiteJob& job, float* sm, int chi) {
+  const int ld = chi | 1, c2 = chi * chi, tid = threadIdx.x;
+  float2* sT = (float2*)sm;
+  float2* sY = sT + 2 * chi * ld;
+  float2* sM = sY + 2 * chi * ld;
+  const int trows = job.deg == 2 ? 2 * chi : 2;
+  for (int i = tid; i < trows * chi; i += kStreamThreads) {
+    const int r = i / chi;
+    sT[r * ld + i - r * chi] = make_float2(job.T[i], job.T[trows * chi + i]);
+  }
+  if (job.deg == 2)
+    for (int i = tid; i < c2; i += kStreamThreads) sM[i] = make_float2(job.mf[i], job.mf[c2 + i]);
+  __syncthreads();
+  const int so = job.deg == 1 || job.open == 1 ? 1 : ld;
+  const int sf = job.deg == 1 ? 0 : job.open == 1 ? ld : 1;
+  const int sp = job.deg == 1 ? ld : chi * ld;
+  const int nf = job.deg == 2 ? chi : 1;
+  if (job.deg == 2) {
+    const int tr = chi, tc = (chi + 3) / 4;  // rows (p, o) in pairs o, o + half; columns by fours
+    for (int i = tid; i < tr * tc; i += kStreamThreads) {
+      const int r = i / tc, n0 = 4 * (i - r * tc);
+      // rows r and r + chi of the 2 chi rows (p, o): the two spins
+      const float2* a0 = sT + r * so;
+      float2 acc[2][4], head[2][4];
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[u][j] = head[u][j] = make_float2(0.f, 0.f);
+      for (int k = 0; k < chi; ++k) {
+        if (k == kSlice)
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              head[u][j] = acc[u][j];
+              acc[u][j] = make_float2(0.f, 0.f);
+            }
+        const float2 a[2] = {a0[k * sf], a0[sp + k * sf]};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float2 b = sM[k * chi + min(n0 + j, chi - 1)];
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+            cmac(acc[u][j].x, acc[u][j].y, a[u].x, a[u].y, b.x, b.y);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (n0 + j < chi)
+            sY[(u * chi + r) * ld + n0 + j] = make_float2(__fadd_rn(head[u][j].x, acc[u][j].x),
+                                                          __fadd_rn(head[u][j].y, acc[u][j].y));
+    }
+    __syncthreads();
+  }
+  const float2* Y = job.deg == 2 ? sY : sT;
+  const int yo = job.deg == 2 ? ld : so, yf = job.deg == 2 ? 1 : 0;
+  const int half = (chi + 1) / 2;
+  for (int i = tid; i < half * half; i += kStreamThreads) {
+    const int o0 = i / half, n0 = i - o0 * half;
+    const int o[2] = {o0, min(o0 + half, chi - 1)}, n[2] = {n0, min(n0 + half, chi - 1)};
+    float2 acc[2][2], sum[2][2], err[2][2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int w = 0; w < 2; ++w) acc[u][w] = sum[u][w] = err[u][w] = make_float2(0.f, 0.f);
+    const int K = 2 * nf;
+    int p = 0, f = 0;
+    for (int k0 = 0; k0 < K; k0 += kSlice) {
+      for (int k = k0; k < min(K, k0 + kSlice); ++k) {
+        float2 y[2], t[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          y[u] = Y[p * sp + o[u] * yo + f * yf];
+          t[u] = sT[p * sp + n[u] * so + f * sf];
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int w = 0; w < 2; ++w)
+            cmac(acc[u][w].x, acc[u][w].y, y[u].x, y[u].y, t[w].x, -t[w].y);
+        if (++f == nf) { f = 0; ++p; }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+          two_sum_acc(sum[u][w].x, err[u][w].x, acc[u][w].x);
+          two_sum_acc(sum[u][w].y, err[u][w].y, acc[u][w].y);
+          acc[u][w] = make_float2(0.f, 0.f);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int w = 0; w < 2; ++w) {  // a repeated edge value is written twice, the same
+        job.out[o[u] * chi + n[w]] = __fadd_rn(sum[u][w].x, err[u][w].x);
+        job.out[c2 + o[u] * chi + n[w]] = __fadd_rn(sum[u][w].y, err[u][w].y);
+      }
+  }
+}
+
+__global__ void __launch_bounds__(kStreamThreads, 1)
+    site_stream_kernel(const SiteJob* jobs, int chi, int open_max, uint32_t inv_chi,
+                       const double* comp_state) {
+  extern __shared__ __align__(16) float sm[];
+  const SiteJob job = jobs[blockIdx.x];
+  if (comp_state && comp_state[4 * job.comp + 3] != 0.0) return;
+  if (job.deg < 3) {
+    stream_low_degree(job, sm, chi);
+    return;
+  }
+  const int ld = chi | 1, c2 = chi * chi, K = 2 * c2;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // both stages first (16-byte aligned), the slice sums, the slabs
+  const int stage_len = (chi * kStageLd + 1) / 2 * 2;
+  float2* sStage = (float2*)sm;
+  float* sums = (float*)(sStage + 2 * stage_len);
+  float2* sY = (float2*)(sums + kStreamWarps * 2 * open_max * chi);
+  float4* sMf = (float4*)(sStage + stage_len);  // the messages lie there until the second stage is needed
+  float4* sMg = sMf + c2;
+  // strides of the legs in T
+  const int so = job.open == 0 ? c2 : job.open == 1 ? chi : 1;
+  const int sf = job.open == 2 ? c2 : 1;
+  const int sg = job.open == 1 ? c2 : chi;
+  const int sp = c2 * chi;
+  const float* T = job.T;
+  const int plane = 2 * sp;
+  // stage st: k = 128 st .. + 127 of (p, g, f), as [o'][k]
+  auto load_stage = [&](int st) {
+    float2* dst = sStage + (st & 1) * stage_len;
+    const int k0 = st * kStageK;
+    if (job.open < 2) {  // contiguous along f
+      const int kk = tid & (kStageK - 1), k = k0 + kk;
+      if (k < K) {
+        const int r = (int)((uint32_t)k * inv_chi >> 20), p = r >= chi;
+        const float* src = T + p * sp + (r - p * chi) * sg + (k - r * chi) * sf;
+        for (int o = tid / kStageK; o < chi; o += kStreamThreads / kStageK) {
+          cp_async4(&dst[o * kStageLd + kk].x, src + o * so);
+          cp_async4(&dst[o * kStageLd + kk].y, src + o * so + plane);
+        }
+      }
+    } else if (lane < chi) {  // contiguous along o'
+      for (int kk = warp; kk < min(kStageK, K - k0); kk += kStreamWarps) {
+        const int k = k0 + kk;
+        const int r = (int)((uint32_t)k * inv_chi >> 20), p = r >= chi;
+        const float* src = T + p * sp + (r - p * chi) * sg + (k - r * chi) * sf + lane;
+        cp_async4(&dst[lane * kStageLd + kk].x, src);
+        cp_async4(&dst[lane * kStageLd + kk].y, src + plane);
+      }
+    }
+    cp_commit();
+  };
+  // the slabs [2 o + p][g][f]
+  if (job.open < 2) {
+    if (lane < chi)
+      for (int r = warp; r < 2 * job.on * chi; r += kStreamWarps) {
+        const int s = (int)((uint32_t)r * inv_chi >> 20), g = r - s * chi;
+        const float* src = T + (s & 1) * sp + (job.o0 + (s >> 1)) * so + g * sg + lane;
+        cp_async4(&sY[r * ld + lane].x, src);
+        cp_async4(&sY[r * ld + lane].y, src + plane);
+      }
+  } else if ((lane & 7) < job.on) {
+    const int ol = lane & 7;
+    for (int r = tid >> 3; r < K; r += kStreamThreads / 8) {  // (p, f, g)
+      const int q = (int)((uint32_t)r * inv_chi >> 20), p = q >= chi;
+      float2* dst = sY + ((2 * ol + p) * chi + r - q * chi) * ld + q - p * chi;
+      const float* src = T + r * chi + job.o0 + ol;
+      cp_async4(&dst->x, src);
+      cp_async4(&dst->y, src + plane);
+    }
+  }
+  load_stage(0);
+  for (int i = tid; i < c2; i += kStreamThreads) {
+    float re = job.mf[i], im = job.mf[c2 + i];
+    sMf[i] = make_float4(re, im, -im, re);
+    re = job.mg[i];
+    im = job.mg[c2 + i];
+    sMg[i] = make_float4(re, im, -im, re);
+  }
+  cp_wait_all();
+  __syncthreads();
+  for (int s = warp; s < 2 * job.on; s += kStreamWarps) {
+    slab_product(sY + s * chi * ld, sMf, chi, ld);  // [f'][g]
+    slab_product(sY + s * chi * ld, sMg, chi, ld);  // [g'][f']
+  }
+  const int ns = (K + kSlice - 1) / kSlice, nst = (ns + kStreamWarps - 1) / kStreamWarps;
+  const int nout = job.on * chi;
+  const int ol = lane % kOL, cl = lane / kOL;
+  int yo[kOI], to[kPJ];
+#pragma unroll
+  for (int i = 0; i < kOI; ++i) yo[i] = min(ol + kOL * i, job.on - 1) * 2 * chi * ld;
+#pragma unroll
+  for (int j = 0; j < kPJ; ++j) to[j] = min(cl + 32 / kOL * j, chi - 1) * kStageLd;
+  // thread tid < 2 nout sums the slices of output part tid
+  float total = 0.f, lost = 0.f;
+  for (int st = 0; st < nst; ++st) {
+    cp_wait_all();
+    __syncthreads();  // stage st is there; the other stage and the sums are done with
+    if (st + 1 < nst) load_stage(st + 1);
+    const int t = st * kStreamWarps + warp;
+    if (t < ns) {
+      float2 acc[kOI][kPJ];
+#pragma unroll
+      for (int i = 0; i < kOI; ++i)
+#pragma unroll
+        for (int j = 0; j < kPJ; ++j) acc[i][j] = make_float2(0.f, 0.f);
+      const int k0 = t * kSlice, kend = min(K, k0 + kSlice);
+      int r = (int)((uint32_t)k0 * inv_chi >> 20), f = k0 - r * chi;
+      const float2* yb = sY + r * ld + f;
+      const float2* tb = sStage + (st & 1) * stage_len + warp * kSlice;
+#pragma unroll 4
+      for (int k = k0; k < kend; ++k) {
+        float2 y[kOI];
+#pragma unroll
+        for (int i = 0; i < kOI; ++i) y[i] = yb[yo[i]];
+#pragma unroll
+        for (int j = 0; j < kPJ; ++j) {
+          const float2 b = tb[to[j]];
+#pragma unroll
+          for (int i = 0; i < kOI; ++i) {
+            acc[i][j] = __ffma2_rn(make_float2(y[i].x, y[i].x), make_float2(b.x, -b.y), acc[i][j]);
+            acc[i][j] = __ffma2_rn(make_float2(y[i].y, y[i].y), make_float2(b.y, b.x), acc[i][j]);
+          }
+        }
+        ++tb;
+        ++yb;
+        if (++f == chi) {
+          f = 0;
+          yb += ld - chi;
+        }
+      }
+      float* d = sums + warp * 2 * nout;
+#pragma unroll
+      for (int i = 0; i < kOI; ++i)
+#pragma unroll
+        for (int j = 0; j < kPJ; ++j) {
+          const int o = ol + kOL * i, c = cl + 32 / kOL * j;
+          if (o < job.on && c < chi) {
+            d[o * chi + c] = acc[i][j].x;
+            d[nout + o * chi + c] = acc[i][j].y;
+          }
+        }
+    }
+    __syncthreads();
+    if (tid < 2 * nout)
+#pragma unroll
+      for (int w = 0; w < kStreamWarps; ++w)
+        if (st * kStreamWarps + w < ns) two_sum_acc(total, lost, sums[w * 2 * nout + tid]);
+  }
+  if (tid < 2 * nout) {
+    const int pl = tid >= nout;
+    job.out[pl * c2 + job.o0 * chi + tid - pl * nout] = __fadd_rn(total, lost);
+  }
+}
+
+size_t stream_bytes(int chi, int open) {
+  const size_t ld = chi | 1;
+  return 2 * sizeof(float2) * (((size_t)chi * kStageLd + 1) / 2 * 2) +
+         sizeof(float) * kStreamWarps * 2 * open * chi + sizeof(float2) * 2 * open * chi * ld;
+}
+// Open-leg values per degree-3 CTA, in even blocks of at most kOpen.
+int stream_open(int chi) {
+  const int blocks = (chi + kOpen - 1) / kOpen;
+  return (chi + blocks - 1) / blocks;
+}
+
 }  // namespace
 
-bool site_sweep_supported(int chi) { return chi >= 1 && chi <= kMaxChi; }
-int site_sweep_open(int chi) { return std::min(chi, kOpen); }
+bool site_sweep_supported(int chi) { return chi >= 1 && chi <= kStreamMaxChi; }
+int site_sweep_open(int chi) { return chi <= kMaxChi ? std::min(chi, kOpen) : stream_open(chi); }
 
 cudaError_t site_sweep_prepare() {
   static std::once_flag once;
   static cudaError_t result = cudaSuccess;
   std::call_once(once, [] {
-    result = cudaFuncSetAttribute(site_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    result = cudaFuncSetAttribute(site_sweep_kernel, at,
                                   (int)(sizeof(float) * smem_floats(kMaxChi)));
+    if (result == cudaSuccess)
+      result = cudaFuncSetAttribute(site_stream_kernel, at,
+                                    (int)stream_bytes(kStreamMaxChi, stream_open(kStreamMaxChi)));
   });
   return result;
 }
@@ -315,8 +677,16 @@ cudaError_t launch_site_sweep(const SiteJob* jobs, int n_jobs, int chi, const in
                               const double* comp_state, cudaStream_t s) {
   if (n_jobs <= 0) return cudaSuccess;
   if (!site_sweep_supported(chi)) return cudaErrorInvalidValue;
-  site_sweep_kernel<<<n_jobs, kThreads, sizeof(float) * smem_floats(chi), s>>>(
-      jobs, chi, make_int3(splits[0], splits[1], splits[2]), comp_state);
+  const int3 sp = make_int3(splits[0], splits[1], splits[2]);
+  if (chi <= kMaxChi) {
+    site_sweep_kernel<<<n_jobs, kThreads, sizeof(float) * smem_floats(chi), s>>>(jobs, chi, sp,
+                                                                                 comp_state);
+    return cudaGetLastError();
+  }
+  const uint32_t inv = ((1u << 20) + chi - 1) / chi;  // x / chi = x inv >> 20 for x <= 2 chi^2
+  const int open = stream_open(chi);
+  site_stream_kernel<<<n_jobs, kStreamThreads, stream_bytes(chi, open), s>>>(jobs, chi, open, inv,
+                                                                       comp_state);
   return cudaGetLastError();
 }
 

@@ -75,3 +75,31 @@ def test_small_chi_sweep_in_a_union(tnlib, chi):
             for src, ed in msgs:
                 got = s.get_message(i * len(g.edges) + ed, off + src)
                 assert np.array_equal(got, alone[(src, ed)])
+
+
+@pytest.mark.parametrize("chi", [17, 18, 19, 20, 21, 22, 23, 24, 25])
+def test_streamed_sweep(tnlib, chi):
+    """At chi = 17 .. 24 a CTA holds the slabs of a block of open-leg values and
+    streams the site tensor for the close (25: back to GEMM launches): against the
+    oracle, and the same bit for bit as one of two components.  Tolerance as above."""
+    g = OG.star3_tree()
+    tensors, msgs = random_state([g.degree(v) for v in range(g.n)], g.edges, chi, seed=300 + chi)
+    alone, _ = one_sweep(tnlib, g, chi, tensors, msgs, "fp32")
+    o = OB.BPState(g, chi)
+    o.T = [t.astype(np.complex64).astype(complex) for t in tensors]
+    o.M = {k: m.astype(np.complex64).astype(complex) for k, m in msgs.items()}
+    o.bp_sweep()
+    assert max(float(np.linalg.norm(alone[k] - o.M[k])) for k in o.M) < 6e-6
+    n, e, c, offs = tnlib.batch_union([(g.n, g.edges, g.colours)] * 2)
+    with tnlib.TNState(n, e, c, chi=chi) as s:
+        for i, off in enumerate(offs):
+            for v in range(g.n):
+                s.set_site(off + v, tensors[v])
+            for (src, ed), m in msgs.items():
+                s.set_message(i * len(g.edges) + ed, off + src, m)
+        s.bp_converge(tol=1e30, max_iters=1)
+        if chi <= 24:
+            for i, off in enumerate(offs):
+                for src, ed in msgs:
+                    got = s.get_message(i * len(g.edges) + ed, off + src)
+                    assert np.array_equal(got, alone[(src, ed)])
