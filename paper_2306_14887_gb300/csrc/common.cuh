@@ -104,7 +104,7 @@ cudaError_t simt_prepare();  // kernel attributes, once, before any stream captu
 cudaError_t launch_cgemm(const GemmDesc& d, cudaStream_t s, float* part = nullptr,
                          size_t part_cap = 0, int* n_kernels = nullptr, int force_splits = 0);
 // One site's chain to one open leg (site_sweep.cu): the message contractions of
-// a BP sweep at chi <= 24 in one launch, FP32, summed as the CUDA-core GEMM sums
+// a BP sweep at chi <= 32 in one launch, FP32, summed as the CUDA-core GEMM sums
 // them.  Degree 3: open-leg values o0 .. o0 + on - 1 (at most
 // site_sweep_open(chi)); mf, mg the incoming messages (planar chi x chi) on the
 // first and second contracted legs.  splits: the split-K counts of the three
@@ -115,6 +115,8 @@ struct SiteJob {
   int32_t deg, open, o0, on, comp, pad;
 };
 bool site_sweep_supported(int chi);
+// whether one launch is the faster sweep, with this many degree-3 jobs
+bool site_sweep_preferred(int chi, int n_deg3_jobs);
 int site_sweep_open(int chi);
 cudaError_t site_sweep_prepare();
 cudaError_t launch_site_sweep(const SiteJob* jobs, int n_jobs, int chi, const int splits[3],

@@ -134,7 +134,7 @@ struct tn_handle {
   // degree-2 chains and degree-1 closes, which share no scratch with the
   // degree-3 chains) runs beside sweep.L[..sweep_split].
   size_t sweep_split = 0;
-  // chi <= 24 on the CUDA cores: the sweep's contractions as one launch (one job
+  // chi <= 32 on the CUDA cores: the sweep's contractions as one launch (one job
   // per site, open leg and block of open-leg values) instead of sweep.L
   tnbp::SiteJob* site_jobs = nullptr;
   int n_site_jobs = 0;
@@ -869,6 +869,10 @@ void build_sweep_plan(tn_handle* h) {
 tn_status build_site_jobs(tn_handle* h) {
   if (!cuda_core_mode(h->cfg) || !site_sweep_supported(h->chi)) return TN_OK;
   const HostGraph& g = h->g;
+  const int step3 = site_sweep_open(h->chi);
+  if (!site_sweep_preferred(h->chi, 3 * (int)h->sites_by_deg[3].size() *
+                                        ((h->chi + step3 - 1) / step3)))
+    return TN_OK;
   std::vector<SiteJob> jobs;
   for (int d = 3; d >= 1; --d)
     for (int v : h->sites_by_deg[d])
@@ -885,7 +889,7 @@ tn_status build_site_jobs(tn_handle* h) {
         } else if (d == 2) {
           q.mf = in_msg(h, v, g.legs[v][1 - j]);
         }
-        const int step = d == 3 ? site_sweep_open(h->chi) : h->chi;
+        const int step = d == 3 ? step3 : h->chi;
         for (int o = 0; o < h->chi; o += step) {
           q.o0 = o;
           q.on = std::min(step, h->chi - o);

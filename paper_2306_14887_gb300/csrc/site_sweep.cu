@@ -1,4 +1,4 @@
-// One BP sweep's message contractions for small bond dimensions (chi <= 24) in
+// One BP sweep's message contractions for small bond dimensions (chi <= 32) in
 // one launch, FP32: every CTA carries one site's chain to one open leg (two mode
 // products and the close) through shared memory.
 //
@@ -32,7 +32,9 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxChi = 16;        // the site tensor fits twice into an SM
-constexpr int kStreamMaxChi = 24;  // rows of a slab a warp holds
+constexpr int kSms = 152;
+constexpr int kNarrowMaxChi = 24;  // three column groups of eight to a slab
+constexpr int kStreamMaxChi = 32;  // rows of a slab a warp holds
 constexpr int kOpen = 8;      // open-leg values per degree-3 CTA: two CTAs per site and leg at
                               // chi = 16, two of them on an SM
 constexpr int kSlice = 16;    // slice depth of the CUDA-core GEMM
@@ -309,8 +311,6 @@ size_t smem_floats(int chi) {
 // Every product is summed as above.  The close is one chain of compensated sums:
 // split-K parts, each rounded to FP32 and added in FP64, kept the FP64 units busy
 // for as long as the products took.
-// Above chi = 24 the GEMM launches have work enough: the same scheme with one slab
-// pair per warp took 157 us against 194 at chi = 28 but 259 against 267 at chi = 32.
 constexpr int kStreamThreads = 512, kStreamWarps = kStreamThreads / 32;
 constexpr int kStageK = kStreamWarps * kSlice;
 constexpr int kStageLd = kStageK + 1;  // float2 per o' row of a stage
@@ -648,6 +648,304 @@ size_t stream_bytes(int chi, int open) {
   return 2 * sizeof(float2) * (((size_t)chi * kStageLd + 1) / 2 * 2) +
          sizeof(float) * kStreamWarps * 2 * open * chi + sizeof(float2) * 2 * open * chi * ld;
 }
+// --- chi = 25 .. 32 ---------------------------------------------------------
+// As above with 144 KB of slabs: two warps share a slab and a slice, and with fewer
+// registers to a warp the slabs lie planar, their contracted leg slow, so that every
+// operand of the packed products (two rows; two values o') is one aligned read.
+// Bound by the operand reads, the transposing copies and the last wave of one CTA
+// per SM (31 percent of the FP32 rate at chi = 32).  A whole sweep, before (GEMM
+// launches) and now: 65 sites at chi = 25 220 and 136 us, 31 257 and 185, 32 181 and
+// 171; 127 qubits at chi = 26 280 and 201, 28 255 and 206, 32 267 and 246; 338 sites
+// at chi = 31 1028 and 933, but 28 656 and 677, 32 795 and 860: with rows of whole
+// 16-byte pieces and enough sites the GEMM launches stay (site_sweep_preferred).
+constexpr int kWideSlices = kStreamWarps / 2, kWideK = kWideSlices * kSlice;
+constexpr int kWideFloats = 2 * kWideK * 32;  // planes of [k][o'], o' rotated by 2 k
+constexpr int kLd = 36;  // slab rows: conflict-free transposed copies and stores
+__host__ __device__ inline int slab_plane(int chi) { return chi * kLd; }
+// o -> o + 1: two spins of two planes; 4 mod 32 banks apart
+__host__ __device__ inline int slab_open(int chi) { return 4 * slab_plane(chi) + 4; }
+
+// Meets the other warp of the pair (both run the same slabs).
+__device__ __forceinline__ void pair_sync(int pair) {
+  asm volatile("bar.sync %0, 64;" ::"r"(pair + 1) : "memory");
+}
+
+// One slab's product in place.  y is planar [k][row] (k the contracted leg); the
+// result goes to [row][col], or with FLIP to [col][row].  M's entries are (re, re,
+// im, im).  Two warps share a slab, sixteen columns each; a lane holds the row pairs
+// 2 rg + 8 h and the columns cg + 8 j.  The sum is taken in two 16-deep slices,
+// whose compensated sum is their rounded sum.
+template <bool FLIP>
+__device__ __forceinline__ void pair_product(float* y, const float4* M, int chi) {
+  constexpr int RP = 4, CJ = 2;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rg = lane >> 3, cg = (lane & 7) + 16 * (warp & 1), plane = slab_plane(chi);
+  float2 pr[RP][CJ], pi[RP][CJ], hr[RP][CJ], hi[RP][CJ];
+#pragma unroll
+  for (int h = 0; h < RP; ++h)
+#pragma unroll
+    for (int j = 0; j < CJ; ++j) pr[h][j] = pi[h][j] = make_float2(0.f, 0.f);
+  int col[CJ];
+#pragma unroll
+  for (int j = 0; j < CJ; ++j) col[j] = min(cg + 8 * j, chi - 1);
+  const float* a = y + 2 * rg;
+  for (int k0 = 0; k0 < chi; k0 += kSlice) {
+    if (k0 == kSlice)
+#pragma unroll
+      for (int h = 0; h < RP; ++h)
+#pragma unroll
+        for (int j = 0; j < CJ; ++j) {
+          hr[h][j] = pr[h][j];
+          hi[h][j] = pi[h][j];
+          pr[h][j] = pi[h][j] = make_float2(0.f, 0.f);
+        }
+    const int kend = min(chi, k0 + kSlice);
+    for (int k = k0; k < kend; ++k) {
+      float2 ar[RP], ai[RP];
+#pragma unroll
+      for (int h = 0; h < RP; ++h) {
+        ar[h] = *(const float2*)(a + k * kLd + 8 * h);
+        ai[h] = *(const float2*)(a + plane + k * kLd + 8 * h);
+      }
+#pragma unroll
+      for (int j = 0; j < CJ; ++j) {
+        const float4 b = M[k * chi + col[j]];
+        const float2 br = make_float2(b.x, b.y), bi = make_float2(b.z, b.w);
+        const float2 bm = make_float2(-b.z, -b.w);
+#pragma unroll
+        for (int h = 0; h < RP; ++h) {
+          pr[h][j] = __ffma2_rn(ar[h], br, pr[h][j]);
+          pi[h][j] = __ffma2_rn(ar[h], bi, pi[h][j]);
+        }
+#pragma unroll
+        for (int h = 0; h < RP; ++h) {
+          pr[h][j] = __ffma2_rn(ai[h], bm, pr[h][j]);
+          pi[h][j] = __ffma2_rn(ai[h], br, pi[h][j]);
+        }
+      }
+    }
+  }
+  pair_sync(warp >> 1);
+#pragma unroll
+  for (int h = 0; h < RP; ++h)
+#pragma unroll
+    for (int j = 0; j < CJ; ++j) {
+      const int r = 2 * rg + 8 * h, c = cg + 8 * j;
+      const float2 re = make_float2(__fadd_rn(hr[h][j].x, pr[h][j].x),
+                                    __fadd_rn(hr[h][j].y, pr[h][j].y));
+      const float2 im = make_float2(__fadd_rn(hi[h][j].x, pi[h][j].x),
+                                    __fadd_rn(hi[h][j].y, pi[h][j].y));
+      if (c < chi && r < chi) {
+        if (FLIP) {  // a row beyond the last one falls into the padding
+          *(float2*)(y + c * kLd + r) = re;
+          *(float2*)(y + plane + c * kLd + r) = im;
+        } else {
+          y[r * kLd + c] = re.x;
+          y[plane + r * kLd + c] = im.x;
+          if (r + 1 < chi) {
+            y[(r + 1) * kLd + c] = re.y;
+            y[plane + (r + 1) * kLd + c] = im.y;
+          }
+        }
+      }
+    }
+  pair_sync(warp >> 1);
+}
+
+// VEC: chi is a multiple of four, and the close reads four contraction indices of a
+// slab at a time.
+template <bool VEC>
+__global__ void __launch_bounds__(kStreamThreads, 1)
+    site_wide_kernel(const SiteJob* jobs, int chi, int open_max, uint32_t inv_chi,
+                     const double* comp_state) {
+  extern __shared__ __align__(16) float sm[];
+  const SiteJob job = jobs[blockIdx.x];
+  if (comp_state && comp_state[4 * job.comp + 3] != 0.0) return;
+  if (job.deg < 3) {
+    stream_low_degree(job, sm, chi);
+    return;
+  }
+  const int c2 = chi * chi, K = 2 * c2, splane = slab_plane(chi), sopen = slab_open(chi);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float* sStage = sm;                     // two stages
+  float* sY = sStage + 2 * kWideFloats;   // the slabs [o][p][plane]
+  float* sums = sY + open_max * sopen;    // a stage's slice sums [slice][plane][o][o']
+  float4* sMf = (float4*)(sStage + kWideFloats);  // until the second stage is needed
+  float4* sMg = sMf + c2;
+  // strides of the legs in T
+  const int so = job.open == 0 ? c2 : job.open == 1 ? chi : 1;
+  const int sf = job.open == 2 ? c2 : 1;
+  const int sg = job.open == 1 ? c2 : chi;
+  const int sp = c2 * chi;
+  const float* T = job.T;
+  const int tplane = 2 * sp;
+  // stage st: k = 128 st .. + 127 of (p, g, f)
+  auto load_stage = [&](int st) {
+    float* dst = sStage + (st & 1) * kWideFloats;
+    const int k0 = st * kWideK;
+    if (job.open < 2) {  // contiguous along f
+      const int kk = tid & (kWideK - 1), k = k0 + kk;
+      if (k < K) {
+        const int r = (int)((uint32_t)k * inv_chi >> 20), p = r >= chi;
+        const float* src = T + p * sp + (r - p * chi) * sg + (k - r * chi) * sf;
+        for (int o = tid / kWideK; o < chi; o += kStreamThreads / kWideK) {
+          float* d = dst + kk * 32 + ((o + 2 * kk) & 31);
+          cp_async4(d, src + o * so);
+          cp_async4(d + kWideK * 32, src + o * so + tplane);
+        }
+      }
+    } else if (lane < chi) {  // contiguous along o'
+      for (int kk = warp; kk < min(kWideK, K - k0); kk += kStreamWarps) {
+        const int k = k0 + kk;
+        const int r = (int)((uint32_t)k * inv_chi >> 20), p = r >= chi;
+        const float* src = T + p * sp + (r - p * chi) * sg + (k - r * chi) * sf + lane;
+        float* d = dst + kk * 32 + ((lane + 2 * kk) & 31);
+        cp_async4(d, src);
+        cp_async4(d + kWideK * 32, src + tplane);
+      }
+    }
+    cp_commit();
+  };
+  // the slabs as [o][p][plane][f][g]
+  if (job.open < 2) {  // eight f by four g per warp
+    const int fb = (chi + 7) / 8, gb = (chi + 3) / 4, nb = fb * gb;
+    for (int i = warp; i < 2 * job.on * nb; i += kStreamWarps) {
+      const int s = i / nb, bl = i - s * nb, f = 8 * (bl % fb) + (lane & 7);
+      const int g = 4 * (bl / fb) + (lane >> 3);
+      if (f < chi && g < chi) {
+        const float* src = T + (s & 1) * sp + (job.o0 + (s >> 1)) * so + g * sg + f;
+        float* d = sY + (s >> 1) * sopen + (s & 1) * 2 * splane + f * kLd + g;
+        cp_async4(d, src);
+        cp_async4(d + splane, src + tplane);
+      }
+    }
+  } else if ((lane & 7) < job.on) {  // eight o by four g
+    const int ol = lane & 7;
+    for (int r = tid >> 3; r < K; r += kStreamThreads / 8) {  // (p, f, g)
+      const int q = (int)((uint32_t)r * inv_chi >> 20), p = q >= chi;
+      float* d = sY + ol * sopen + p * 2 * splane + (q - p * chi) * kLd + r - q * chi;
+      const float* src = T + r * chi + job.o0 + ol;
+      cp_async4(d, src);
+      cp_async4(d + splane, src + tplane);
+    }
+  }
+  load_stage(0);
+  for (int i = tid; i < c2; i += kStreamThreads) {
+    float re = job.mf[i], im = job.mf[c2 + i];
+    sMf[i] = make_float4(re, re, im, im);
+    re = job.mg[i];
+    im = job.mg[c2 + i];
+    sMg[i] = make_float4(re, re, im, im);
+  }
+  cp_wait_all();
+  __syncthreads();
+  for (int s = warp >> 1; s < 2 * job.on; s += kStreamWarps / 2) {
+    float* y = sY + (s >> 1) * sopen + (s & 1) * 2 * splane;
+    pair_product<false>(y, sMf, chi);  // [f][g] -> [g][f']
+    pair_product<true>(y, sMg, chi);   // [g][f'] -> [g'][f']
+  }
+  const int ns = (K + kSlice - 1) / kSlice, nst = (ns + kWideSlices - 1) / kWideSlices;
+  const int nout = job.on * chi;
+  // two warps share a slice, four open values each: a lane closes o = ol, ol + 2 with
+  // the pair o' = 2 cl, 2 cl + 1
+  const int slice = warp >> 1, ol = (lane >> 4) + 4 * (warp & 1), cl = lane & 15;
+  int yo[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) yo[i] = min(ol + 2 * i, job.on - 1) * sopen;
+  // thread tid < 2 nout sums the slices of output part tid
+  float total = 0.f, lost = 0.f;
+  for (int st = 0; st < nst; ++st) {
+    cp_wait_all();
+    __syncthreads();  // stage st is there; the other stage and the sums are done with
+    if (st + 1 < nst) load_stage(st + 1);
+    const int t = st * kWideSlices + slice;
+    if (t < ns) {
+      float2 pr[2], pi[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) pr[i] = pi[i] = make_float2(0.f, 0.f);
+      const int k0 = t * kSlice, n = min(K - k0, kSlice);
+      int r = (int)((uint32_t)k0 * inv_chi >> 20), f = k0 - r * chi;
+      // row r = (p, g') of a slab: spin 1 starts two planes after spin 0
+      const float* yb = sY + (r + (r >= chi ? chi : 0)) * kLd + f;
+      const float* tb = sStage + (st & 1) * kWideFloats + slice * kSlice * 32;
+      auto step = [&](int kk, const float (&yr)[2], const float (&yi)[2]) {
+        const float* q = tb + kk * 32 + ((2 * cl + 2 * kk) & 31);  // 32 | 2 kSlice
+        const float2 tr = *(const float2*)q, ti = *(const float2*)(q + kWideK * 32);
+        const float2 tm = make_float2(-ti.x, -ti.y);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const float2 y2 = make_float2(yr[i], yr[i]);
+          pr[i] = __ffma2_rn(y2, tr, pr[i]);
+          pi[i] = __ffma2_rn(y2, tm, pi[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const float2 y2 = make_float2(yi[i], yi[i]);
+          pr[i] = __ffma2_rn(y2, ti, pr[i]);
+          pi[i] = __ffma2_rn(y2, tr, pi[i]);
+        }
+      };
+      auto advance = [&](int by) {
+        yb += by;
+        f += by;
+        if (f == chi) {
+          f = 0;
+          yb += kLd - chi;
+          if (++r == chi) yb += splane;
+        }
+      };
+      if (VEC) {  // K is a multiple of 16, f of 4
+#pragma unroll
+        for (int kk = 0; kk < kSlice; kk += 4) {
+          float4 vr[2], vi[2];
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            vr[i] = *(const float4*)(yb + yo[i]);
+            vi[i] = *(const float4*)(yb + splane + yo[i]);
+          }
+          step(kk, {vr[0].x, vr[1].x}, {vi[0].x, vi[1].x});
+          step(kk + 1, {vr[0].y, vr[1].y}, {vi[0].y, vi[1].y});
+          step(kk + 2, {vr[0].z, vr[1].z}, {vi[0].z, vi[1].z});
+          step(kk + 3, {vr[0].w, vr[1].w}, {vi[0].w, vi[1].w});
+          advance(4);
+        }
+      } else {
+#pragma unroll 2
+        for (int kk = 0; kk < n; ++kk) {
+          step(kk, {yb[yo[0]], yb[yo[1]]}, {yb[splane + yo[0]], yb[splane + yo[1]]});
+          advance(1);
+        }
+      }
+      float* d = sums + slice * 2 * nout;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int o = ol + 2 * i, c = 2 * cl;
+        if (o < job.on && c < chi) {
+          d[o * chi + c] = pr[i].x;
+          d[nout + o * chi + c] = pi[i].x;
+          if (c + 1 < chi) {
+            d[o * chi + c + 1] = pr[i].y;
+            d[nout + o * chi + c + 1] = pi[i].y;
+          }
+        }
+      }
+    }
+    __syncthreads();
+    if (tid < 2 * nout)
+#pragma unroll
+      for (int w = 0; w < kWideSlices; ++w)
+        if (st * kWideSlices + w < ns) two_sum_acc(total, lost, sums[w * 2 * nout + tid]);
+  }
+  if (tid < 2 * nout) {
+    const int pl = tid >= nout;
+    job.out[pl * c2 + job.o0 * chi + tid - pl * nout] = __fadd_rn(total, lost);
+  }
+}
+
+size_t wide_bytes(int chi, int open) {
+  return sizeof(float) *
+         (2 * kWideFloats + (size_t)open * slab_open(chi) + kWideSlices * 2 * open * chi);
+}
+
 // Open-leg values per degree-3 CTA, in even blocks of at most kOpen.
 int stream_open(int chi) {
   const int blocks = (chi + kOpen - 1) / kOpen;
@@ -657,6 +955,9 @@ int stream_open(int chi) {
 }  // namespace
 
 bool site_sweep_supported(int chi) { return chi >= 1 && chi <= kStreamMaxChi; }
+bool site_sweep_preferred(int chi, int n_deg3_jobs) {
+  return chi <= kNarrowMaxChi || chi % 4 != 0 || n_deg3_jobs <= 4 * kSms;
+}
 int site_sweep_open(int chi) { return chi <= kMaxChi ? std::min(chi, kOpen) : stream_open(chi); }
 
 cudaError_t site_sweep_prepare() {
@@ -668,7 +969,11 @@ cudaError_t site_sweep_prepare() {
                                   (int)(sizeof(float) * smem_floats(kMaxChi)));
     if (result == cudaSuccess)
       result = cudaFuncSetAttribute(site_stream_kernel, at,
-                                    (int)stream_bytes(kStreamMaxChi, stream_open(kStreamMaxChi)));
+                                    (int)stream_bytes(kNarrowMaxChi, stream_open(kNarrowMaxChi)));
+    if (result == cudaSuccess)
+      result = cudaFuncSetAttribute(site_wide_kernel<true>, at, (int)wide_bytes(32, kOpen));
+    if (result == cudaSuccess)
+      result = cudaFuncSetAttribute(site_wide_kernel<false>, at, (int)wide_bytes(31, kOpen));
   });
   return result;
 }
@@ -685,8 +990,12 @@ cudaError_t launch_site_sweep(const SiteJob* jobs, int n_jobs, int chi, const in
   }
   const uint32_t inv = ((1u << 20) + chi - 1) / chi;  // x / chi = x inv >> 20 for x <= 2 chi^2
   const int open = stream_open(chi);
-  site_stream_kernel<<<n_jobs, kStreamThreads, stream_bytes(chi, open), s>>>(jobs, chi, open, inv,
-                                                                       comp_state);
+  if (chi <= kNarrowMaxChi)
+    site_stream_kernel<<<n_jobs, kStreamThreads, stream_bytes(chi, open), s>>>(jobs, chi, open, inv,
+                                                                               comp_state);
+  else
+    (chi % 4 ? site_wide_kernel<false> : site_wide_kernel<true>)<<<
+        n_jobs, kStreamThreads, wide_bytes(chi, open), s>>>(jobs, chi, open, inv, comp_state);
   return cudaGetLastError();
 }
 

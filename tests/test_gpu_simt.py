@@ -103,3 +103,34 @@ def test_streamed_sweep(tnlib, chi):
                 for src, ed in msgs:
                     got = s.get_message(i * len(g.edges) + ed, off + src)
                     assert np.array_equal(got, alone[(src, ed)])
+
+
+@pytest.mark.parametrize("chi", [25, 26, 27, 28, 29, 30, 31, 32])
+def test_wide_streamed_sweep(tnlib, chi):
+    """chi = 25 .. 32, two warps to a slab: against the oracle, as one of two
+    components bit for bit the same, and as one of 52 (over four CTAs per SM, where
+    multiples of four run as GEMM launches) against the oracle again.  Tolerance as
+    above."""
+    g = OG.star3_tree()
+    tensors, msgs = random_state([g.degree(v) for v in range(g.n)], g.edges, chi, seed=400 + chi)
+    alone, _ = one_sweep(tnlib, g, chi, tensors, msgs, "fp32")
+    o = OB.BPState(g, chi)
+    o.T = [t.astype(np.complex64).astype(complex) for t in tensors]
+    o.M = {k: m.astype(np.complex64).astype(complex) for k, m in msgs.items()}
+    o.bp_sweep()
+    assert max(float(np.linalg.norm(alone[k] - o.M[k])) for k in o.M) < 6e-6
+    for copies in (2, 52):
+        n, e, c, offs = tnlib.batch_union([(g.n, g.edges, g.colours)] * copies)
+        with tnlib.TNState(n, e, c, chi=chi) as s:
+            for i, off in enumerate(offs):
+                for v in range(g.n):
+                    s.set_site(off + v, tensors[v])
+                for (src, ed), m in msgs.items():
+                    s.set_message(i * len(g.edges) + ed, off + src, m)
+            s.bp_converge(tol=1e30, max_iters=1)
+            for i in (0, copies - 1):
+                for src, ed in msgs:
+                    got = s.get_message(i * len(g.edges) + ed, offs[i] + src)
+                    assert float(np.linalg.norm(got - o.M[(src, ed)])) < 6e-6
+                    if copies == 2:
+                        assert np.array_equal(got, alone[(src, ed)])
