@@ -138,6 +138,9 @@ struct tn_handle {
   // per site, open leg and block of open-leg values) instead of sweep.L
   tnbp::SiteJob* site_jobs = nullptr;
   int n_site_jobs = 0;
+  // chi <= 16: a gate layer's environments as one launch instead of gate_env
+  std::vector<tnbp::SiteJob*> env_jobs;
+  std::vector<int> n_env_jobs;
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 
@@ -864,49 +867,78 @@ void build_sweep_plan(tn_handle* h) {
   tag(from, h->sites_by_deg[1]);
 }
 
-// The sweep as one launch (site_sweep.cu): the degree-3 chains first, the
-// longest jobs.  Legs contracted in the order of the chains above.
-tn_status build_site_jobs(tn_handle* h) {
-  if (!cuda_core_mode(h->cfg) || !site_sweep_supported(h->chi)) return TN_OK;
+// The jobs of site v's chain to its leg j, cut into blocks of open-leg values;
+// the legs are contracted in the order of the chains above.
+void add_site_jobs(const tn_handle* h, int v, int j, float* out, std::vector<SiteJob>& jobs) {
   const HostGraph& g = h->g;
-  const int step3 = site_sweep_open(h->chi);
-  if (!site_sweep_preferred(h->chi, 3 * (int)h->sites_by_deg[3].size() *
-                                        ((h->chi + step3 - 1) / step3)))
-    return TN_OK;
-  std::vector<SiteJob> jobs;
-  for (int d = 3; d >= 1; --d)
-    for (int v : h->sites_by_deg[d])
-      for (int j = 0; j < d; ++j) {
-        SiteJob q{};
-        q.T = site_ptr(h, h->T, v);
-        q.out = (float*)msg_ptr(h, h->raw, dir_id(g, v, g.legs[v][j]));
-        q.deg = d;
-        q.open = j;
-        q.comp = h->comp_of_vertex[v];
-        if (d == 3) {
-          q.mf = in_msg(h, v, g.legs[v][j == 2 ? 0 : 2]);
-          q.mg = in_msg(h, v, g.legs[v][j == 1 ? 0 : 1]);
-        } else if (d == 2) {
-          q.mf = in_msg(h, v, g.legs[v][1 - j]);
-        }
-        const int step = d == 3 ? step3 : h->chi;
-        for (int o = 0; o < h->chi; o += step) {
-          q.o0 = o;
-          q.on = std::min(step, h->chi - o);
-          jobs.push_back(q);
-        }
-      }
+  const int d = g.degree(v);
+  SiteJob q{};
+  q.T = site_ptr(h, h->T, v);
+  q.out = out;
+  q.deg = d;
+  q.open = j;
+  q.comp = h->comp_of_vertex[v];
+  if (d == 3) {
+    q.mf = in_msg(h, v, g.legs[v][j == 2 ? 0 : 2]);
+    q.mg = in_msg(h, v, g.legs[v][j == 1 ? 0 : 1]);
+  } else if (d == 2) {
+    q.mf = in_msg(h, v, g.legs[v][1 - j]);
+  }
+  const int step = d == 3 ? site_sweep_open(h->chi) : h->chi;
+  for (int o = 0; o < h->chi; o += step) {
+    q.o0 = o;
+    q.on = std::min(step, h->chi - o);
+    jobs.push_back(q);
+  }
+}
+
+tn_status upload_site_jobs(tn_handle* h, const std::vector<SiteJob>& jobs, SiteJob** dev, int* n) {
   if (jobs.empty()) return TN_OK;
-  h->site_jobs = (SiteJob*)dev_alloc(h, sizeof(SiteJob) * jobs.size());
-  if (!h->site_jobs) { set_error("device allocation of the sweep jobs failed"); return TN_ENOMEM; }
-  if (cudaMemcpy(h->site_jobs, jobs.data(), sizeof(SiteJob) * jobs.size(),
-                 cudaMemcpyHostToDevice) != cudaSuccess ||
+  *dev = (SiteJob*)dev_alloc(h, sizeof(SiteJob) * jobs.size());
+  if (!*dev) { set_error("device allocation of the sweep jobs failed"); return TN_ENOMEM; }
+  if (cudaMemcpy(*dev, jobs.data(), sizeof(SiteJob) * jobs.size(), cudaMemcpyHostToDevice) !=
+          cudaSuccess ||
       site_sweep_prepare() != cudaSuccess) {
     set_error("preparing the sweep jobs failed");
     return TN_ECUDA;
   }
-  h->n_site_jobs = (int)jobs.size();
+  *n = (int)jobs.size();
   return TN_OK;
+}
+
+// The sweep and the gate layers' environments as one launch each (site_sweep.cu):
+// the degree-3 chains first, the longest jobs.
+tn_status build_site_jobs(tn_handle* h) {
+  const HostGraph& g = h->g;
+  h->env_jobs.assign(g.layers.size(), nullptr);
+  h->n_env_jobs.assign(g.layers.size(), 0);
+  if (!cuda_core_mode(h->cfg) || !site_sweep_supported(h->chi)) return TN_OK;
+  std::vector<SiteJob> jobs;
+  tn_status st;
+  if (site_env_supported(h->chi))
+    for (size_t li = 0; li < g.layers.size(); ++li) {
+      jobs.clear();
+      for (int d = 3; d >= 1; --d)
+        for (size_t s = 0; s < g.layers[li].size(); ++s)
+          for (int side = 0; side < 2; ++side) {
+            const int e = g.layers[li][s], v = side ? g.ew[e] : g.eu[e];
+            if (g.degree(v) == d)
+              add_site_jobs(h, v, g.leg_pos(v, e),
+                            h->gram + ((int64_t)s * 2 + side) * 4 * h->chi * h->chi, jobs);
+          }
+      st = upload_site_jobs(h, jobs, &h->env_jobs[li], &h->n_env_jobs[li]);
+      if (st) return st;
+    }
+  const int step3 = site_sweep_open(h->chi);
+  if (!site_sweep_preferred(h->chi, 3 * (int)h->sites_by_deg[3].size() *
+                                        ((h->chi + step3 - 1) / step3)))
+    return TN_OK;
+  jobs.clear();
+  for (int d = 3; d >= 1; --d)
+    for (int v : h->sites_by_deg[d])
+      for (int j = 0; j < d; ++j)
+        add_site_jobs(h, v, j, (float*)msg_ptr(h, h->raw, dir_id(g, v, g.legs[v][j])), jobs);
+  return upload_site_jobs(h, jobs, &h->site_jobs, &h->n_site_jobs);
 }
 
 // The sweep's contractions at small chi, with the split-K counts the plan's
@@ -1239,8 +1271,23 @@ tn_status gate_layer(tn_handle* h, int li, int sign) {
   if (st) return st;
   st = ensure_mrt(h);
   if (st) return st;
-  st = run_plan(h, h->gate_env[li], P_ENV);
-  if (st) return st;
+  if (h->n_env_jobs[li]) {
+    const int pe = prof_begin(h, P_ENV);
+    TN_CUDA_TRY(launch_site_env(h->env_jobs[li], h->n_env_jobs[li], h->chi, h->stream));
+    h->stats.kernel_launches++;
+    if (pe >= 0) {
+      double flops = 0.0, bytes = 0.0, f, b;
+      for (auto& L : h->gate_env[li].L) {
+        gemm_work(L.d, &f, &b);
+        flops += f;
+        bytes += b;
+      }
+      prof_end(h, pe, flops, bytes);
+    }
+  } else {
+    st = run_plan(h, h->gate_env[li], P_ENV);
+    if (st) return st;
+  }
   SolveArgs a;
   a.n_edges = (int)h->g.layers[li].size();
   a.chi = h->chi;

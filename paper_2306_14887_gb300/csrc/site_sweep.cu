@@ -20,6 +20,11 @@
 // in place in shared memory; then all warps close over k = (p, g', f'),
 //   out[o][o'] = sum_k Y2[o; k] conj(T[o'; k]),
 // each warp taking every eighth slice for all outputs.
+//
+// A gate layer's environments are the same chains with p left open: two parts, one
+// per p, each closed over (g', f') into out[p][o][o'].  Their K = chi^2 <= 256 is
+// never split.  A step's three layers: 127 qubits at chi = 16 0.465 ms as GEMM
+// launches, 0.071 ms; 65 sites at chi = 9 0.407 and 0.044.
 #include <algorithm>
 #include <mutex>
 
@@ -68,7 +73,8 @@ __device__ __forceinline__ void load_rows(float* dst, int ld, int64_t dst_plane,
 }
 
 __global__ void __launch_bounds__(kThreads, 2)
-    site_sweep_kernel(const SiteJob* jobs, int chi, int3 splits3, const double* comp_state) {
+    site_sweep_kernel(const SiteJob* jobs, int chi, int parts, int3 splits3,
+                      const double* comp_state) {
   extern __shared__ __align__(16) float sm[];
   const SiteJob job = jobs[blockIdx.x];
   // a converged component of a union keeps its messages
@@ -164,7 +170,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     __syncthreads();
     // close: slice t covers k = 16 t .. 16 t + 15 of (p, g', f')
     constexpr int kPer = 2 * kMaxChi * kMaxChi / kSlice / kWarps;  // slices per warp at most
-    const int K = 2 * c2, ns = (K + kSlice - 1) / kSlice;
+    const int K = 2 * c2 / parts, nsp = (K + kSlice - 1) / kSlice, ns = parts * nsp;
     float psr[kPer][2][2], psi[kPer][2][2];
     {
       int ro[2], co[2];
@@ -181,9 +187,9 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
           for (int j = 0; j < 2; ++j) psr[u][i][j] = psi[u][i][j] = 0.f;
         if (t >= ns) continue;
-        const int k0 = t * kSlice;
+        const int q = t >= nsp, k0 = q * K + (t - q * nsp) * kSlice;
         int p = k0 / c2, g = (k0 - p * c2) / chi, f = k0 - p * c2 - g * chi;
-        const int kend = min(K, k0 + kSlice);
+        const int kend = min((q + 1) * K, k0 + kSlice);
         for (int k = k0; k < kend; ++k) {
           const float* yb = sY + (p * chi + g) * ld + f;
           const float* tb = sT + p * sp + g * sg + f * sf;
@@ -225,19 +231,19 @@ __global__ void __launch_bounds__(kThreads, 2)
     __syncthreads();
     const int splits = job.open == 0 ? splits3.x : job.open == 1 ? splits3.y : splits3.z;
     // slices per split-K part, as the GEMM cuts K
-    const int per = splits > 1 ? ((K + splits - 1) / splits + kSlice - 1) / kSlice : ns;
-    if (tid < 2 * nout) {
-      const int pl = tid >= nout, o = tid - pl * nout;
+    const int per = splits > 1 ? ((K + splits - 1) / splits + kSlice - 1) / kSlice : nsp;
+    for (int i = tid; i < parts * 2 * nout; i += kThreads) {
+      const int r = i / nout, pl = r & 1, o = i - r * nout, t0 = (r >> 1) * nsp;
       double sum = 0.0;
       float val = 0.f;
       for (int q = 0; q < splits; ++q) {
         float s = 0.f, c = 0.f;
-        for (int t = q * per; t < min(ns, (q + 1) * per); ++t)
-          two_sum_acc(s, c, sY[(t * 2 + pl) * nout + o]);
+        for (int t = q * per; t < min(nsp, (q + 1) * per); ++t)
+          two_sum_acc(s, c, sY[((t0 + t) * 2 + pl) * nout + o]);
         val = __fadd_rn(s, c);
         sum += (double)val;
       }
-      job.out[pl * c2 + job.o0 * chi + o] = splits > 1 ? (float)sum : val;
+      job.out[r * c2 + job.o0 * chi + o] = splits > 1 ? (float)sum : val;
     }
     return;
   }
@@ -269,11 +275,11 @@ __global__ void __launch_bounds__(kThreads, 2)
   }
   const float* Y = job.deg == 2 ? sY : sT;
   const int yo = job.deg == 2 ? ld : so, yf = job.deg == 2 ? 1 : 0;
-  for (int i = tid; i < c2; i += kThreads) {
-    const int o = i / chi, n = i - o * chi;
+  for (int i = tid; i < parts * c2; i += kThreads) {
+    const int q = i / c2, o = (i - q * c2) / chi, n = i - q * c2 - o * chi;
     float sr = 0.f, cr = 0.f, si = 0.f, ci = 0.f, pr = 0.f, pi = 0.f;
     int left = kSlice;
-    for (int p = 0; p < 2; ++p)
+    for (int p = q; p < (parts == 2 ? q + 1 : 2); ++p)
       for (int f = 0; f < nf; ++f) {
         const float* y = Y + p * sp + o * yo + f * yf;
         const float* t = sT + p * sp + n * so + f * sf;
@@ -289,8 +295,8 @@ __global__ void __launch_bounds__(kThreads, 2)
       two_sum_acc(sr, cr, pr);
       two_sum_acc(si, ci, pi);
     }
-    job.out[i] = __fadd_rn(sr, cr);
-    job.out[c2 + i] = __fadd_rn(si, ci);
+    job.out[2 * q * c2 + o * chi + n] = __fadd_rn(sr, cr);
+    job.out[(2 * q + 1) * c2 + o * chi + n] = __fadd_rn(si, ci);
   }
 }
 
@@ -306,7 +312,7 @@ size_t smem_floats(int chi) {
 // per warp and stage.  Bound by the issue of the products' operand reads and of the
 // transposing 4-byte copies.  A whole sweep with normalisation and stop rule, before
 // (eight GEMM launches) and now: 65 sites at chi = 17 181 and 63 us, 22 224 and 74,
-// 23 184 and 83; 127 qubits at chi = 23 255 and 134; 338 sites at chi = 24 490 and
+// 23 184 and 83; 127 qubits at chi = 23 255 and 134; 433 sites at chi = 24 490 and
 // 391.  Two CTAs of eight warps per SM took 71, 96, 97, 133 and 454.
 // Every product is summed as above.  The close is one chain of compensated sums:
 // split-K parts, each rounded to FP32 and added in FP64, kept the FP64 units busy
@@ -655,7 +661,7 @@ size_t stream_bytes(int chi, int open) {
 // Bound by the operand reads, the transposing copies and the last wave of one CTA
 // per SM (31 percent of the FP32 rate at chi = 32).  A whole sweep, before (GEMM
 // launches) and now: 65 sites at chi = 25 220 and 136 us, 31 257 and 185, 32 181 and
-// 171; 127 qubits at chi = 26 280 and 201, 28 255 and 206, 32 267 and 246; 338 sites
+// 171; 127 qubits at chi = 26 280 and 201, 28 255 and 206, 32 267 and 246; 433 sites
 // at chi = 31 1028 and 933, but 28 656 and 677, 32 795 and 860: with rows of whole
 // 16-byte pieces and enough sites the GEMM launches stay (site_sweep_preferred).
 constexpr int kWideSlices = kStreamWarps / 2, kWideK = kWideSlices * kSlice;
@@ -984,7 +990,7 @@ cudaError_t launch_site_sweep(const SiteJob* jobs, int n_jobs, int chi, const in
   if (!site_sweep_supported(chi)) return cudaErrorInvalidValue;
   const int3 sp = make_int3(splits[0], splits[1], splits[2]);
   if (chi <= kMaxChi) {
-    site_sweep_kernel<<<n_jobs, kThreads, sizeof(float) * smem_floats(chi), s>>>(jobs, chi, sp,
+    site_sweep_kernel<<<n_jobs, kThreads, sizeof(float) * smem_floats(chi), s>>>(jobs, chi, 1, sp,
                                                                                  comp_state);
     return cudaGetLastError();
   }
@@ -996,6 +1002,16 @@ cudaError_t launch_site_sweep(const SiteJob* jobs, int n_jobs, int chi, const in
   else
     (chi % 4 ? site_wide_kernel<false> : site_wide_kernel<true>)<<<
         n_jobs, kStreamThreads, wide_bytes(chi, open), s>>>(jobs, chi, open, inv, comp_state);
+  return cudaGetLastError();
+}
+
+bool site_env_supported(int chi) { return chi >= 1 && chi <= kMaxChi; }
+
+cudaError_t launch_site_env(const SiteJob* jobs, int n_jobs, int chi, cudaStream_t s) {
+  if (n_jobs <= 0) return cudaSuccess;
+  if (!site_env_supported(chi)) return cudaErrorInvalidValue;
+  site_sweep_kernel<<<n_jobs, kThreads, sizeof(float) * smem_floats(chi), s>>>(
+      jobs, chi, 2, make_int3(1, 1, 1), nullptr);
   return cudaGetLastError();
 }
 

@@ -134,3 +134,17 @@ def test_wide_streamed_sweep(tnlib, chi):
                     assert float(np.linalg.norm(got - o.M[(src, ed)])) < 6e-6
                     if copies == 2:
                         assert np.array_equal(got, alone[(src, ed)])
+
+
+@pytest.mark.parametrize("chi", [4, 5, 7, 8, 9, 13, 15, 16, 17])
+def test_one_launch_environments(tnlib, chi):
+    """Up to chi = 16 a gate layer's environments run as one launch (17: GEMM
+    launches): four steps on the star, where bond dimension 4 is exact, against the
+    oracle, within the FP32 path's 1e-6 for exact evolutions.  Sites of degree 1, 2
+    and 3, every leg open."""
+    g = OG.star3_tree()
+    o = OB.run(g, chi, 0.6, 4)
+    for prec in ("fp32", "tf32x3"):
+        with tnlib.TNState(g.n, g.edges, g.colours, chi=chi, prec=prec) as s:
+            s.apply_floquet(0.6, 4)
+            assert np.abs(s.expect_z_all() - o.all_z()).max() < 1e-6
