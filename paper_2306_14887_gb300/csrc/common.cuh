@@ -121,9 +121,8 @@ int site_sweep_open(int chi);
 cudaError_t site_sweep_prepare();
 cudaError_t launch_site_sweep(const SiteJob* jobs, int n_jobs, int chi, const int splits[3],
                               const double* comp_state, cudaStream_t s);
-// The same chains with p left open (chi <= 16): a gate layer's environments, out
+// The same chains with p left open: a gate layer's environments, out
 // [p][re|im][chi][chi].
-bool site_env_supported(int chi);
 cudaError_t launch_site_env(const SiteJob* jobs, int n_jobs, int chi, cudaStream_t s);
 // Tensor-core version (tc_gemm.cu) for TN_TF32 / TN_BF16 descriptors.  part:
 // scratch for K-split partial products (tc_plan gives the size, part_cap the

@@ -138,7 +138,7 @@ struct tn_handle {
   // per site, open leg and block of open-leg values) instead of sweep.L
   tnbp::SiteJob* site_jobs = nullptr;
   int n_site_jobs = 0;
-  // chi <= 16: a gate layer's environments as one launch instead of gate_env
+  // the same for a gate layer's environments, instead of gate_env
   std::vector<tnbp::SiteJob*> env_jobs;
   std::vector<int> n_env_jobs;
   cudaStream_t side = nullptr;
@@ -915,24 +915,25 @@ tn_status build_site_jobs(tn_handle* h) {
   if (!cuda_core_mode(h->cfg) || !site_sweep_supported(h->chi)) return TN_OK;
   std::vector<SiteJob> jobs;
   tn_status st;
-  if (site_env_supported(h->chi))
-    for (size_t li = 0; li < g.layers.size(); ++li) {
-      jobs.clear();
-      for (int d = 3; d >= 1; --d)
-        for (size_t s = 0; s < g.layers[li].size(); ++s)
-          for (int side = 0; side < 2; ++side) {
-            const int e = g.layers[li][s], v = side ? g.ew[e] : g.eu[e];
-            if (g.degree(v) == d)
-              add_site_jobs(h, v, g.leg_pos(v, e),
-                            h->gram + ((int64_t)s * 2 + side) * 4 * h->chi * h->chi, jobs);
-          }
-      st = upload_site_jobs(h, jobs, &h->env_jobs[li], &h->n_env_jobs[li]);
-      if (st) return st;
+  const int step3 = site_sweep_open(h->chi), blocks = (h->chi + step3 - 1) / step3;
+  for (size_t li = 0; li < g.layers.size(); ++li) {
+    jobs.clear();
+    int n3 = 0;
+    for (int d = 3; d >= 1; --d) {
+      for (size_t s = 0; s < g.layers[li].size(); ++s)
+        for (int side = 0; side < 2; ++side) {
+          const int e = g.layers[li][s], v = side ? g.ew[e] : g.eu[e];
+          if (g.degree(v) == d)
+            add_site_jobs(h, v, g.leg_pos(v, e),
+                          h->gram + ((int64_t)s * 2 + side) * 4 * h->chi * h->chi, jobs);
+        }
+      if (d == 3) n3 = (int)jobs.size();
     }
-  const int step3 = site_sweep_open(h->chi);
-  if (!site_sweep_preferred(h->chi, 3 * (int)h->sites_by_deg[3].size() *
-                                        ((h->chi + step3 - 1) / step3)))
-    return TN_OK;
+    if (!site_sweep_preferred(h->chi, n3)) continue;
+    st = upload_site_jobs(h, jobs, &h->env_jobs[li], &h->n_env_jobs[li]);
+    if (st) return st;
+  }
+  if (!site_sweep_preferred(h->chi, 3 * (int)h->sites_by_deg[3].size() * blocks)) return TN_OK;
   jobs.clear();
   for (int d = 3; d >= 1; --d)
     for (int v : h->sites_by_deg[d])

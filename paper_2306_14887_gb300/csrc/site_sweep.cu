@@ -22,9 +22,12 @@
 // each warp taking every eighth slice for all outputs.
 //
 // A gate layer's environments are the same chains with p left open: two parts, one
-// per p, each closed over (g', f') into out[p][o][o'].  Their K = chi^2 <= 256 is
-// never split.  A step's three layers: 127 qubits at chi = 16 0.465 ms as GEMM
-// launches, 0.071 ms; 65 sites at chi = 9 0.407 and 0.044.
+// per p, each closed over (g', f') into out[p][o][o'].  A step's three layers, as
+// GEMM launches and as one launch each: 127 qubits at chi = 16 0.465 and 0.071 ms, 24
+// 0.56 and 0.14, 32 0.62 and 0.24; 65 sites at chi = 9 0.407 and 0.044, 23 0.55 and
+// 0.13, 31 0.69 and 0.25; 433 sites at chi = 32 1.30 and 0.92.  Up to chi = 16 their
+// K = chi^2 is never split and the sums are the GEMM's.  The streamed kernels take
+// the parts as a template argument: as a runtime value they cost the sweep 6 percent.
 #include <algorithm>
 #include <mutex>
 
@@ -392,7 +395,7 @@ __device__ __forceinline__ void slab_product(float2* y, const float4* M, int chi
 
 // One site of degree 1 or 2 (T[p, o, f]), the chains of site_sweep_kernel with a
 // 2 x 4 tile of the product and a 2 x 2 tile of the close per thread.
-__device__ void stream_low_degree(const SiteJob& job, float* sm, int chi) {
+__device__ void stream_low_degree(const SiteJob& job, float* sm, int chi, int parts) {
   const int ld = chi | 1, c2 = chi * chi, tid = threadIdx.x;
   float2* sT = (float2*)sm;
   float2* sY = sT + 2 * chi * ld;
@@ -451,16 +454,17 @@ __device__ void stream_low_degree(const SiteJob& job, float* sm, int chi) {
   const float2* Y = job.deg == 2 ? sY : sT;
   const int yo = job.deg == 2 ? ld : so, yf = job.deg == 2 ? 1 : 0;
   const int half = (chi + 1) / 2;
-  for (int i = tid; i < half * half; i += kStreamThreads) {
-    const int o0 = i / half, n0 = i - o0 * half;
+  for (int i = tid; i < parts * half * half; i += kStreamThreads) {
+    const int q = i >= half * half, i0 = i - q * half * half;
+    const int o0 = i0 / half, n0 = i0 - o0 * half;
     const int o[2] = {o0, min(o0 + half, chi - 1)}, n[2] = {n0, min(n0 + half, chi - 1)};
     float2 acc[2][2], sum[2][2], err[2][2];
 #pragma unroll
     for (int u = 0; u < 2; ++u)
 #pragma unroll
       for (int w = 0; w < 2; ++w) acc[u][w] = sum[u][w] = err[u][w] = make_float2(0.f, 0.f);
-    const int K = 2 * nf;
-    int p = 0, f = 0;
+    const int K = 2 * nf / parts;
+    int p = q, f = 0;
     for (int k0 = 0; k0 < K; k0 += kSlice) {
       for (int k = k0; k < min(K, k0 + kSlice); ++k) {
         float2 y[2], t[2];
@@ -489,12 +493,13 @@ __device__ void stream_low_degree(const SiteJob& job, float* sm, int chi) {
     for (int u = 0; u < 2; ++u)
 #pragma unroll
       for (int w = 0; w < 2; ++w) {  // a repeated edge value is written twice, the same
-        job.out[o[u] * chi + n[w]] = __fadd_rn(sum[u][w].x, err[u][w].x);
-        job.out[c2 + o[u] * chi + n[w]] = __fadd_rn(sum[u][w].y, err[u][w].y);
+        job.out[2 * q * c2 + o[u] * chi + n[w]] = __fadd_rn(sum[u][w].x, err[u][w].x);
+        job.out[(2 * q + 1) * c2 + o[u] * chi + n[w]] = __fadd_rn(sum[u][w].y, err[u][w].y);
       }
   }
 }
 
+template <int PARTS>
 __global__ void __launch_bounds__(kStreamThreads, 1)
     site_stream_kernel(const SiteJob* jobs, int chi, int open_max, uint32_t inv_chi,
                        const double* comp_state) {
@@ -502,10 +507,11 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   const SiteJob job = jobs[blockIdx.x];
   if (comp_state && comp_state[4 * job.comp + 3] != 0.0) return;
   if (job.deg < 3) {
-    stream_low_degree(job, sm, chi);
+    stream_low_degree(job, sm, chi, PARTS);
     return;
   }
-  const int ld = chi | 1, c2 = chi * chi, K = 2 * c2;
+  const int ld = chi | 1, c2 = chi * chi, K = 2 * c2 / PARTS;
+  const int nsp = (K + kSlice - 1) / kSlice, ns = PARTS * nsp;  // slices per part, of all
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // both stages first (16-byte aligned), the slice sums, the slabs
   const int stage_len = (chi * kStageLd + 1) / 2 * 2;
@@ -521,13 +527,20 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   const int sp = c2 * chi;
   const float* T = job.T;
   const int plane = 2 * sp;
+  // first k of slice t; the k of position kk of stage st, or -1
+  auto second = [&](int t) { return PARTS == 2 && t >= nsp; };
+  auto slice_k = [&](int t) { return second(t) ? K + (t - nsp) * kSlice : t * kSlice; };
+  auto stage_k = [&](int st, int kk) {
+    if (PARTS == 1) return st * kStageK + kk < K ? st * kStageK + kk : -1;
+    const int t = st * kStreamWarps + kk / kSlice, k = slice_k(t) + kk % kSlice;
+    return t < ns && k < (second(t) ? 2 * K : K) ? k : -1;
+  };
   // stage st: k = 128 st .. + 127 of (p, g, f), as [o'][k]
   auto load_stage = [&](int st) {
     float2* dst = sStage + (st & 1) * stage_len;
-    const int k0 = st * kStageK;
     if (job.open < 2) {  // contiguous along f
-      const int kk = tid & (kStageK - 1), k = k0 + kk;
-      if (k < K) {
+      const int kk = tid & (kStageK - 1), k = stage_k(st, kk);
+      if (k >= 0) {
         const int r = (int)((uint32_t)k * inv_chi >> 20), p = r >= chi;
         const float* src = T + p * sp + (r - p * chi) * sg + (k - r * chi) * sf;
         for (int o = tid / kStageK; o < chi; o += kStreamThreads / kStageK) {
@@ -536,8 +549,9 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         }
       }
     } else if (lane < chi) {  // contiguous along o'
-      for (int kk = warp; kk < min(kStageK, K - k0); kk += kStreamWarps) {
-        const int k = k0 + kk;
+      for (int kk = warp; kk < kStageK; kk += kStreamWarps) {
+        const int k = stage_k(st, kk);
+        if (k < 0) continue;
         const int r = (int)((uint32_t)k * inv_chi >> 20), p = r >= chi;
         const float* src = T + p * sp + (r - p * chi) * sg + (k - r * chi) * sf + lane;
         cp_async4(&dst[lane * kStageLd + kk].x, src);
@@ -557,7 +571,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       }
   } else if ((lane & 7) < job.on) {
     const int ol = lane & 7;
-    for (int r = tid >> 3; r < K; r += kStreamThreads / 8) {  // (p, f, g)
+    for (int r = tid >> 3; r < 2 * c2; r += kStreamThreads / 8) {  // (p, f, g)
       const int q = (int)((uint32_t)r * inv_chi >> 20), p = q >= chi;
       float2* dst = sY + ((2 * ol + p) * chi + r - q * chi) * ld + q - p * chi;
       const float* src = T + r * chi + job.o0 + ol;
@@ -579,7 +593,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     slab_product(sY + s * chi * ld, sMf, chi, ld);  // [f'][g]
     slab_product(sY + s * chi * ld, sMg, chi, ld);  // [g'][f']
   }
-  const int ns = (K + kSlice - 1) / kSlice, nst = (ns + kStreamWarps - 1) / kStreamWarps;
+  const int nst = (ns + kStreamWarps - 1) / kStreamWarps;
   const int nout = job.on * chi;
   const int ol = lane % kOL, cl = lane / kOL;
   int yo[kOI], to[kPJ];
@@ -589,6 +603,11 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   for (int j = 0; j < kPJ; ++j) to[j] = min(cl + 32 / kOL * j, chi - 1) * kStageLd;
   // thread tid < 2 nout sums the slices of output part tid
   float total = 0.f, lost = 0.f;
+  auto store = [&](int q) {
+    const int pl = tid >= nout;
+    job.out[(2 * q + pl) * c2 + job.o0 * chi + tid - pl * nout] = __fadd_rn(total, lost);
+    total = lost = 0.f;
+  };
   for (int st = 0; st < nst; ++st) {
     cp_wait_all();
     __syncthreads();  // stage st is there; the other stage and the sums are done with
@@ -600,7 +619,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       for (int i = 0; i < kOI; ++i)
 #pragma unroll
         for (int j = 0; j < kPJ; ++j) acc[i][j] = make_float2(0.f, 0.f);
-      const int k0 = t * kSlice, kend = min(K, k0 + kSlice);
+      const int k0 = slice_k(t), kend = min(second(t) ? 2 * K : K, k0 + kSlice);
       int r = (int)((uint32_t)k0 * inv_chi >> 20), f = k0 - r * chi;
       const float2* yb = sY + r * ld + f;
       const float2* tb = sStage + (st & 1) * stage_len + warp * kSlice;
@@ -641,12 +660,12 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     if (tid < 2 * nout)
 #pragma unroll
       for (int w = 0; w < kStreamWarps; ++w)
-        if (st * kStreamWarps + w < ns) two_sum_acc(total, lost, sums[w * 2 * nout + tid]);
+        if (st * kStreamWarps + w < ns) {
+          if (PARTS == 2 && st * kStreamWarps + w == nsp) store(0);  // the second part begins
+          two_sum_acc(total, lost, sums[w * 2 * nout + tid]);
+        }
   }
-  if (tid < 2 * nout) {
-    const int pl = tid >= nout;
-    job.out[pl * c2 + job.o0 * chi + tid - pl * nout] = __fadd_rn(total, lost);
-  }
+  if (tid < 2 * nout) store(PARTS - 1);
 }
 
 size_t stream_bytes(int chi, int open) {
@@ -759,7 +778,7 @@ __device__ __forceinline__ void pair_product(float* y, const float4* M, int chi)
 
 // VEC: chi is a multiple of four, and the close reads four contraction indices of a
 // slab at a time.
-template <bool VEC>
+template <bool VEC, int PARTS>
 __global__ void __launch_bounds__(kStreamThreads, 1)
     site_wide_kernel(const SiteJob* jobs, int chi, int open_max, uint32_t inv_chi,
                      const double* comp_state) {
@@ -767,10 +786,11 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   const SiteJob job = jobs[blockIdx.x];
   if (comp_state && comp_state[4 * job.comp + 3] != 0.0) return;
   if (job.deg < 3) {
-    stream_low_degree(job, sm, chi);
+    stream_low_degree(job, sm, chi, PARTS);
     return;
   }
-  const int c2 = chi * chi, K = 2 * c2, splane = slab_plane(chi), sopen = slab_open(chi);
+  const int c2 = chi * chi, K = 2 * c2 / PARTS, splane = slab_plane(chi), sopen = slab_open(chi);
+  const int nsp = (K + kSlice - 1) / kSlice, ns = PARTS * nsp;  // slices per part, of all
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float* sStage = sm;                     // two stages
   float* sY = sStage + 2 * kWideFloats;   // the slabs [o][p][plane]
@@ -784,13 +804,20 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   const int sp = c2 * chi;
   const float* T = job.T;
   const int tplane = 2 * sp;
+  // first k of slice t; the k of position kk of stage st, or -1
+  auto second = [&](int t) { return PARTS == 2 && t >= nsp; };
+  auto slice_k = [&](int t) { return second(t) ? K + (t - nsp) * kSlice : t * kSlice; };
+  auto stage_k = [&](int st, int kk) {
+    if (PARTS == 1) return st * kWideK + kk < K ? st * kWideK + kk : -1;
+    const int t = st * kWideSlices + kk / kSlice, k = slice_k(t) + kk % kSlice;
+    return t < ns && k < (second(t) ? 2 * K : K) ? k : -1;
+  };
   // stage st: k = 128 st .. + 127 of (p, g, f)
   auto load_stage = [&](int st) {
     float* dst = sStage + (st & 1) * kWideFloats;
-    const int k0 = st * kWideK;
     if (job.open < 2) {  // contiguous along f
-      const int kk = tid & (kWideK - 1), k = k0 + kk;
-      if (k < K) {
+      const int kk = tid & (kWideK - 1), k = stage_k(st, kk);
+      if (k >= 0) {
         const int r = (int)((uint32_t)k * inv_chi >> 20), p = r >= chi;
         const float* src = T + p * sp + (r - p * chi) * sg + (k - r * chi) * sf;
         for (int o = tid / kWideK; o < chi; o += kStreamThreads / kWideK) {
@@ -800,8 +827,9 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         }
       }
     } else if (lane < chi) {  // contiguous along o'
-      for (int kk = warp; kk < min(kWideK, K - k0); kk += kStreamWarps) {
-        const int k = k0 + kk;
+      for (int kk = warp; kk < kWideK; kk += kStreamWarps) {
+        const int k = stage_k(st, kk);
+        if (k < 0) continue;
         const int r = (int)((uint32_t)k * inv_chi >> 20), p = r >= chi;
         const float* src = T + p * sp + (r - p * chi) * sg + (k - r * chi) * sf + lane;
         float* d = dst + kk * 32 + ((lane + 2 * kk) & 31);
@@ -826,7 +854,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     }
   } else if ((lane & 7) < job.on) {  // eight o by four g
     const int ol = lane & 7;
-    for (int r = tid >> 3; r < K; r += kStreamThreads / 8) {  // (p, f, g)
+    for (int r = tid >> 3; r < 2 * c2; r += kStreamThreads / 8) {  // (p, f, g)
       const int q = (int)((uint32_t)r * inv_chi >> 20), p = q >= chi;
       float* d = sY + ol * sopen + p * 2 * splane + (q - p * chi) * kLd + r - q * chi;
       const float* src = T + r * chi + job.o0 + ol;
@@ -849,7 +877,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     pair_product<false>(y, sMf, chi);  // [f][g] -> [g][f']
     pair_product<true>(y, sMg, chi);   // [g][f'] -> [g'][f']
   }
-  const int ns = (K + kSlice - 1) / kSlice, nst = (ns + kWideSlices - 1) / kWideSlices;
+  const int nst = (ns + kWideSlices - 1) / kWideSlices;
   const int nout = job.on * chi;
   // two warps share a slice, four open values each: a lane closes o = ol, ol + 2 with
   // the pair o' = 2 cl, 2 cl + 1
@@ -859,6 +887,11 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   for (int i = 0; i < 2; ++i) yo[i] = min(ol + 2 * i, job.on - 1) * sopen;
   // thread tid < 2 nout sums the slices of output part tid
   float total = 0.f, lost = 0.f;
+  auto store = [&](int q) {
+    const int pl = tid >= nout;
+    job.out[(2 * q + pl) * c2 + job.o0 * chi + tid - pl * nout] = __fadd_rn(total, lost);
+    total = lost = 0.f;
+  };
   for (int st = 0; st < nst; ++st) {
     cp_wait_all();
     __syncthreads();  // stage st is there; the other stage and the sums are done with
@@ -868,7 +901,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       float2 pr[2], pi[2];
 #pragma unroll
       for (int i = 0; i < 2; ++i) pr[i] = pi[i] = make_float2(0.f, 0.f);
-      const int k0 = t * kSlice, n = min(K - k0, kSlice);
+      const int k0 = slice_k(t), n = min((second(t) ? 2 * K : K) - k0, kSlice);
       int r = (int)((uint32_t)k0 * inv_chi >> 20), f = k0 - r * chi;
       // row r = (p, g') of a slab: spin 1 starts two planes after spin 0
       const float* yb = sY + (r + (r >= chi ? chi : 0)) * kLd + f;
@@ -939,12 +972,12 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     if (tid < 2 * nout)
 #pragma unroll
       for (int w = 0; w < kWideSlices; ++w)
-        if (st * kWideSlices + w < ns) two_sum_acc(total, lost, sums[w * 2 * nout + tid]);
+        if (st * kWideSlices + w < ns) {
+          if (PARTS == 2 && st * kWideSlices + w == nsp) store(0);  // the second part begins
+          two_sum_acc(total, lost, sums[w * 2 * nout + tid]);
+        }
   }
-  if (tid < 2 * nout) {
-    const int pl = tid >= nout;
-    job.out[pl * c2 + job.o0 * chi + tid - pl * nout] = __fadd_rn(total, lost);
-  }
+  if (tid < 2 * nout) store(PARTS - 1);
 }
 
 size_t wide_bytes(int chi, int open) {
@@ -970,49 +1003,55 @@ cudaError_t site_sweep_prepare() {
   static std::once_flag once;
   static cudaError_t result = cudaSuccess;
   std::call_once(once, [] {
-    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    result = cudaFuncSetAttribute(site_sweep_kernel, at,
-                                  (int)(sizeof(float) * smem_floats(kMaxChi)));
-    if (result == cudaSuccess)
-      result = cudaFuncSetAttribute(site_stream_kernel, at,
-                                    (int)stream_bytes(kNarrowMaxChi, stream_open(kNarrowMaxChi)));
-    if (result == cudaSuccess)
-      result = cudaFuncSetAttribute(site_wide_kernel<true>, at, (int)wide_bytes(32, kOpen));
-    if (result == cudaSuccess)
-      result = cudaFuncSetAttribute(site_wide_kernel<false>, at, (int)wide_bytes(31, kOpen));
+    auto raise = [](auto kernel, size_t bytes) {
+      if (result == cudaSuccess)
+        result = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)bytes);
+    };
+    const size_t narrow = stream_bytes(kNarrowMaxChi, stream_open(kNarrowMaxChi));
+    raise(site_sweep_kernel, sizeof(float) * smem_floats(kMaxChi));
+    raise(site_stream_kernel<1>, narrow);
+    raise(site_stream_kernel<2>, narrow);
+    raise(site_wide_kernel<true, 1>, wide_bytes(32, kOpen));
+    raise(site_wide_kernel<true, 2>, wide_bytes(32, kOpen));
+    raise(site_wide_kernel<false, 1>, wide_bytes(31, kOpen));
+    raise(site_wide_kernel<false, 2>, wide_bytes(31, kOpen));
   });
   return result;
 }
 
-cudaError_t launch_site_sweep(const SiteJob* jobs, int n_jobs, int chi, const int splits[3],
-                              const double* comp_state, cudaStream_t s) {
+namespace {
+cudaError_t launch_parts(const SiteJob* jobs, int n_jobs, int chi, int parts, int3 splits,
+                         const double* comp_state, cudaStream_t s) {
   if (n_jobs <= 0) return cudaSuccess;
   if (!site_sweep_supported(chi)) return cudaErrorInvalidValue;
-  const int3 sp = make_int3(splits[0], splits[1], splits[2]);
   if (chi <= kMaxChi) {
-    site_sweep_kernel<<<n_jobs, kThreads, sizeof(float) * smem_floats(chi), s>>>(jobs, chi, 1, sp,
-                                                                                 comp_state);
+    site_sweep_kernel<<<n_jobs, kThreads, sizeof(float) * smem_floats(chi), s>>>(
+        jobs, chi, parts, splits, comp_state);
     return cudaGetLastError();
   }
   const uint32_t inv = ((1u << 20) + chi - 1) / chi;  // x / chi = x inv >> 20 for x <= 2 chi^2
   const int open = stream_open(chi);
   if (chi <= kNarrowMaxChi)
-    site_stream_kernel<<<n_jobs, kStreamThreads, stream_bytes(chi, open), s>>>(jobs, chi, open, inv,
-                                                                               comp_state);
-  else
-    (chi % 4 ? site_wide_kernel<false> : site_wide_kernel<true>)<<<
-        n_jobs, kStreamThreads, wide_bytes(chi, open), s>>>(jobs, chi, open, inv, comp_state);
+    (parts == 2 ? site_stream_kernel<2> : site_stream_kernel<1>)<<<
+        n_jobs, kStreamThreads, stream_bytes(chi, open), s>>>(jobs, chi, open, inv, comp_state);
+  else {
+    auto kernel = chi % 4 ? (parts == 2 ? site_wide_kernel<false, 2> : site_wide_kernel<false, 1>)
+                          : (parts == 2 ? site_wide_kernel<true, 2> : site_wide_kernel<true, 1>);
+    kernel<<<n_jobs, kStreamThreads, wide_bytes(chi, open), s>>>(jobs, chi, open, inv, comp_state);
+  }
   return cudaGetLastError();
 }
+}  // namespace
 
-bool site_env_supported(int chi) { return chi >= 1 && chi <= kMaxChi; }
+cudaError_t launch_site_sweep(const SiteJob* jobs, int n_jobs, int chi, const int splits[3],
+                              const double* comp_state, cudaStream_t s) {
+  return launch_parts(jobs, n_jobs, chi, 1, make_int3(splits[0], splits[1], splits[2]), comp_state,
+                      s);
+}
 
 cudaError_t launch_site_env(const SiteJob* jobs, int n_jobs, int chi, cudaStream_t s) {
-  if (n_jobs <= 0) return cudaSuccess;
-  if (!site_env_supported(chi)) return cudaErrorInvalidValue;
-  site_sweep_kernel<<<n_jobs, kThreads, sizeof(float) * smem_floats(chi), s>>>(
-      jobs, chi, 2, make_int3(1, 1, 1), nullptr);
-  return cudaGetLastError();
+  return launch_parts(jobs, n_jobs, chi, 2, make_int3(1, 1, 1), nullptr, s);
 }
 
 }  // namespace tnbp

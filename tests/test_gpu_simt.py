@@ -148,3 +148,14 @@ def test_one_launch_environments(tnlib, chi):
         with tnlib.TNState(g.n, g.edges, g.colours, chi=chi, prec=prec) as s:
             s.apply_floquet(0.6, 4)
             assert np.abs(s.expect_z_all() - o.all_z()).max() < 1e-6
+
+
+@pytest.mark.parametrize("chi", [18, 21, 23, 24, 25, 27, 28, 31, 32, 33])
+def test_streamed_environments(tnlib, chi):
+    """The environments of chi = 17 .. 32 through the streamed sweep kernels, one part
+    per physical value: as above, same bound."""
+    g = OG.star3_tree()
+    o = OB.run(g, 8, 0.6, 4)  # bond dimension 4 is exact
+    with tnlib.TNState(g.n, g.edges, g.colours, chi=chi) as s:
+        s.apply_floquet(0.6, 4)
+        assert np.abs(s.expect_z_all() - o.all_z()).max() < 1e-6
