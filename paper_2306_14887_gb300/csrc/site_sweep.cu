@@ -3,16 +3,16 @@
 // products and the close) through shared memory.
 //
 // At these sizes the contractions of a sweep are a dozen dependent launches of a
-// few microseconds of work each; the site tensor (64 KB at chi = 16) and the
+// few microseconds of work each.  Up to chi = 16 the site tensor (64 KB) and the
 // chain's intermediate fit an SM, so nothing but T is read and nothing but the
-// message is written.  Bound by the shared-memory reads of the products.
-// Measured, a whole sweep with normalisation and stop rule: 127 qubits at chi =
+// message is written; larger chi below.  Bound by the latency of a CTA's phases and
+// the shared-memory reads of the products.  Measured, a whole sweep with normalisation and stop rule: 127 qubits at chi =
 // 16 46 us (147 us as separate GEMM launches), 338 sites at chi = 16 79 us (201),
 // 65 sites at chi = 9 24 us (173 with the GEMM before its rewrite).
 //
-// Up to chi = 16 every sum is taken exactly as the CUDA-core GEMM takes it (16-deep slices of
-// the contraction in the same order, slice sums added by compensated two-sums,
-// split-K parts added in FP64), so the messages are the same bit for bit.
+// Up to chi = 16 every sum is taken exactly as the CUDA-core GEMM takes it (16-deep
+// slices of the contraction in the same order, slice sums added by compensated
+// two-sums, split-K parts added in FP64), so the messages are the same bit for bit.
 //
 // Degree 3, open leg o, first contracted leg f, second g (the chains of the
 // sweep plan): a warp owns a slab (p, o), a chi x chi matrix over (g, f):
