@@ -6,6 +6,7 @@
 
 #include <string>
 
+#include "device_once.cuh"
 #include "tnbp.h"
 
 namespace tnbp {
@@ -100,7 +101,7 @@ __host__ __device__ __forceinline__ int64_t row_off3(int m, int M2, int M3, int6
 // force_splits > 0 replaces the heuristic split count (the autotuner's
 // choice); a count whose partials would not fit part_cap falls back to one.
 int cgemm_plan(const GemmDesc& d, size_t* part_floats, int force_splits = 0);
-cudaError_t simt_prepare();  // kernel attributes, once, before any stream capture
+cudaError_t simt_prepare();  // kernel attributes, once per device, before any stream capture
 cudaError_t launch_cgemm(const GemmDesc& d, cudaStream_t s, float* part = nullptr,
                          size_t part_cap = 0, int* n_kernels = nullptr, int force_splits = 0);
 // One site's chain to one open leg (site_sweep.cu): the message contractions of
@@ -300,14 +301,17 @@ cudaError_t launch_solve(const SolveArgs& a, cudaStream_t s);
 size_t solve_work_doubles(int chi);
 // Shared-memory solve with FP32 rotations (solve32.cu), chi <= 64.
 bool solve32_supported(int chi);
+cudaError_t solve32_prepare();  // kernel attributes, as simt_prepare
 cudaError_t launch_solve32(const SolveArgs& a, cudaStream_t s);
 // The refined solve's FP32 starting basis for 2 chi > 128 (solve32.cu): the
 // bond matrix in the global workspace, one CTA per edge, 16 <= chi <= 256.
+cudaError_t basis_gmem_prepare();
 cudaError_t launch_basis_gmem(const SolveArgs& a, cudaStream_t s);
 // Refined solve (solve_refine.cu): FP64 Cholesky, FP32 starting basis, FP64
 // Newton refinement and FP64 leg matrices; chi <= 64.  work: solve_work_doubles
 // per edge.
 bool solve_refined_supported(int chi);
+cudaError_t refine_prepare();
 cudaError_t launch_solve_refined(const SolveArgs& a, cudaStream_t s);
 // The two halves of launch_solve_refined: the FP64 Cholesky and the FP32
 // starting basis; the FP64 Newton step and leg matrices.

@@ -2,7 +2,6 @@
 // gate, message normalisation with the FP64 residual, the single-site reduced
 // density matrix and a batched block copy.
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -528,13 +527,11 @@ cudaError_t launch_first_leg_last(const float* T, float* TA, const int64_t* site
 // The shared-memory limit of the normalise kernel, raised once to the largest
 // tile the kernel takes (chi with 2 chi (chi + 1) floats <= 200 KB); thread-safe.
 cudaError_t normalise_prepare(int) {
-  static std::once_flag once;
-  static cudaError_t result = cudaSuccess;
-  std::call_once(once, [] {
-    result = cudaFuncSetAttribute(normalise_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  200 * 1024);
+  static DeviceOnce once;
+  return once([] {
+    return cudaFuncSetAttribute(normalise_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                200 * 1024);
   });
-  return result;
 }
 
 cudaError_t launch_bp_loop_init(int n_comp, double* state, unsigned long long* res,

@@ -25,7 +25,6 @@
 // step it took 8.08 ms.  A persistent form, its copies running ahead across
 // tiles, spilled registers and took 2.95 against 2.61 ms.
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
 #include "tnbp.h"
@@ -430,17 +429,16 @@ int cgemm_plan(const GemmDesc& d, size_t* part_floats, int force_splits) {
   return s;
 }
 
-// Kernel attributes, set once before any launch (and before any stream capture).
+// Kernel attributes, set on each device before any launch (and before any stream capture).
 cudaError_t simt_prepare() {
-  static std::once_flag once;
-  static cudaError_t result = cudaSuccess;
-  std::call_once(once, [] {
-    result = prepare_tile<64, 64, 4>();
-    if (result == cudaSuccess) result = prepare_tile<128, 32, 4>();
-    if (result == cudaSuccess) result = prepare_tile<256, 16, 4>();
-    if (result == cudaSuccess) result = prepare_tile<32, 32, 2>();
+  static DeviceOnce once;
+  return once([] {
+    cudaError_t e = prepare_tile<64, 64, 4>();
+    if (e == cudaSuccess) e = prepare_tile<128, 32, 4>();
+    if (e == cudaSuccess) e = prepare_tile<256, 16, 4>();
+    if (e == cudaSuccess) e = prepare_tile<32, 32, 2>();
+    return e;
   });
-  return result;
 }
 
 // Element offsets inside one operand are 32-bit (a site plane holds at most

@@ -29,7 +29,6 @@
 // K = chi^2 is never split and the sums are the GEMM's.  The streamed kernels take
 // the parts as a template argument: as a runtime value they cost the sweep 6 percent.
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
 #include "tnbp.h"
@@ -1000,10 +999,10 @@ bool site_sweep_preferred(int chi, int n_deg3_jobs) {
 int site_sweep_open(int chi) { return chi <= kMaxChi ? std::min(chi, kOpen) : stream_open(chi); }
 
 cudaError_t site_sweep_prepare() {
-  static std::once_flag once;
-  static cudaError_t result = cudaSuccess;
-  std::call_once(once, [] {
-    auto raise = [](auto kernel, size_t bytes) {
+  static DeviceOnce once;
+  return once([] {
+    cudaError_t result = cudaSuccess;
+    auto raise = [&](auto kernel, size_t bytes) {
       if (result == cudaSuccess)
         result = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)bytes);
@@ -1016,8 +1015,8 @@ cudaError_t site_sweep_prepare() {
     raise(site_wide_kernel<true, 2>, wide_bytes(32, kOpen));
     raise(site_wide_kernel<false, 1>, wide_bytes(31, kOpen));
     raise(site_wide_kernel<false, 2>, wide_bytes(31, kOpen));
+    return result;
   });
-  return result;
 }
 
 namespace {

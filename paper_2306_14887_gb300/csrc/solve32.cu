@@ -26,8 +26,6 @@
 //      messages <- diag(S).
 #include <math.h>
 
-#include <mutex>
-
 #include "chol_rows.cuh"
 #include "common.cuh"
 #include "tnbp.h"
@@ -1151,6 +1149,32 @@ size_t smem_bytes(int chi) {
 
 bool solve32_supported(int chi) { return chi >= 1 && chi <= kMaxChi; }
 
+cudaError_t basis_gmem_prepare() {
+  static DeviceOnce once;
+  return once([] {
+    cudaError_t e = cudaFuncSetAttribute(basis_jacobi_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(sizeof(float2) * 2 * kGWarps * kGMaxN));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(basis_jacobi_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed,
+                               1);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(basis_bond_kernel<16>,
+                               cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+  });
+}
+
+// The limit of the largest chi, so that concurrent launches at different chi
+// (the job server) never lower it.
+cudaError_t solve32_prepare() {
+  static DeviceOnce once;
+  return once([] {
+    return cudaFuncSetAttribute(solve32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)smem_bytes(kMaxChi));
+  });
+}
+
 cudaError_t launch_basis_gmem(const SolveArgs& a, cudaStream_t st) {
   if (a.n_edges <= 0) return cudaSuccess;
   const int n = 2 * a.chi;
@@ -1158,19 +1182,8 @@ cudaError_t launch_basis_gmem(const SolveArgs& a, cudaStream_t st) {
   // one pair slot per warp: 8 CTAs (the portable cluster size) hold n <= 256,
   // 16 hold the rest
   const int ctas = n <= 256 ? 8 : 16;
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(basis_jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(sizeof(float2) * 2 * kGWarps * kGMaxN));
-    if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(basis_jacobi_kernel,
-                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(basis_bond_kernel<16>,
-                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  });
-  if (attr != cudaSuccess) return attr;
+  cudaError_t e = basis_gmem_prepare();
+  if (e != cudaSuccess) return e;
   const int per = (n / 2 + ctas - 1) / ctas;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.n_edges * ctas);
@@ -1183,8 +1196,8 @@ cudaError_t launch_basis_gmem(const SolveArgs& a, cudaStream_t st) {
   cfg.attrs = cl;
   cfg.numAttrs = 1;
   cfg.blockDim = dim3(kBThreads);
-  cudaError_t e = n <= 256 ? cudaLaunchKernelEx(&cfg, basis_bond_kernel<8>, a, ctas)
-                           : cudaLaunchKernelEx(&cfg, basis_bond_kernel<16>, a, ctas);
+  e = n <= 256 ? cudaLaunchKernelEx(&cfg, basis_bond_kernel<8>, a, ctas)
+               : cudaLaunchKernelEx(&cfg, basis_bond_kernel<16>, a, ctas);
   if (e != cudaSuccess) return e;
   cfg.blockDim = dim3(kGThreads);
   cfg.dynamicSmemBytes = sizeof(float2) * 2 * (size_t)per * n;
@@ -1196,15 +1209,8 @@ cudaError_t launch_basis_gmem(const SolveArgs& a, cudaStream_t st) {
 cudaError_t launch_solve32(const SolveArgs& a, cudaStream_t st) {
   if (a.n_edges <= 0) return cudaSuccess;
   if (!solve32_supported(a.chi)) return cudaErrorInvalidValue;
-  // the shared-memory limit is raised once, to the largest chi's need, so that
-  // concurrent launches at different chi (the job server) never lower it
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(solve32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_bytes(kMaxChi));
-  });
-  if (attr != cudaSuccess) return attr;
+  const cudaError_t e = solve32_prepare();
+  if (e != cudaSuccess) return e;
   const size_t sm = smem_bytes(a.chi);
   if (!a.basis) {
     solve32_kernel<<<a.n_edges, kThreads, sm, st>>>(a);

@@ -47,7 +47,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "chol_rows.cuh"
 #include "common.cuh"
@@ -737,31 +736,12 @@ __global__ void __launch_bounds__(kThreads, 2) legs_kernel(SolveArgs a, int cwma
   }
 }
 
-// Shared-memory limits of the refined solve's kernels, raised once to the
-// largest request any chi <= kMaxChi makes, so that concurrent launches (the
+// Shared-memory limits of the refined solve's kernels, raised once per device to
+// the largest request any chi <= kMaxChi makes, so that concurrent launches (the
 // job server's slots) never lower a limit another thread relies on.
 constexpr size_t kCholSmemMax = sizeof(double2) * kSmemChi * kSmemChi;
 constexpr size_t kRefineSmemMax = kSmemBudget + 4096;
 constexpr size_t kLegsSmemMax = kSmemBudget / 2 + 8192;
-
-cudaError_t refine_prepare() {
-  static std::once_flag once;
-  static cudaError_t result = cudaSuccess;
-  std::call_once(once, [] {
-    result = cudaFuncSetAttribute(chol64_kernel<2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)kCholSmemMax);
-    if (result == cudaSuccess)
-      for (auto k : {refine_kernel<false>, refine_kernel<true>})
-        if (result == cudaSuccess)
-          result = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)kRefineSmemMax);
-    for (auto k : {legs_kernel<false>, legs_kernel<true>})
-      if (result == cudaSuccess)
-        result = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)kLegsSmemMax);
-  });
-  return result;
-}
 
 int sm_count() {
   int dev = 0, sms = 0;
@@ -771,6 +751,23 @@ int sm_count() {
 }
 
 }  // namespace
+
+cudaError_t refine_prepare() {
+  static DeviceOnce once;
+  return once([] {
+    cudaError_t result = cudaFuncSetAttribute(
+        chol64_kernel<2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCholSmemMax);
+    for (auto k : {refine_kernel<false>, refine_kernel<true>})
+      if (result == cudaSuccess)
+        result = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)kRefineSmemMax);
+    for (auto k : {legs_kernel<false>, legs_kernel<true>})
+      if (result == cudaSuccess)
+        result = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)kLegsSmemMax);
+    return result;
+  });
+}
 
 bool solve_refined_supported(int chi) {
   if (chi >= 1 && chi <= kSmemChi) return solve32_supported(chi);

@@ -29,7 +29,6 @@
 #include <stdint.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -653,19 +652,18 @@ bool tc_plan(const GemmDesc& d, int* quad, int* splits, size_t* part_floats, int
   return true;
 }
 
-// Kernel attributes, set once before any launch (and before any stream capture).
+// Kernel attributes, set on each device before any launch (and before any stream capture).
 cudaError_t tc_prepare() {
-  static std::once_flag once;
-  static cudaError_t result = cudaSuccess;
-  std::call_once(once, [] {
-    result = cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  static DeviceOnce once;
+  return once([] {
+    cudaError_t result = cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)tc_smem_bytes(1));
     // two CTAs per SM: ask for the largest shared-memory carveout
     if (result == cudaSuccess)
       result = cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                     100);
+    return result;
   });
-  return result;
 }
 
 cudaError_t launch_cgemm_tc(const GemmDesc& d, float* part, int* err, cudaStream_t st,

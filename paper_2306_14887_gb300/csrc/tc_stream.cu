@@ -30,6 +30,8 @@
 #include <cuda.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -866,7 +868,7 @@ bool row_levels(const GemmDesc& d, Levels* L) {
   return rem == 1;
 }
 
-int g_num_sms = 0;
+std::atomic<int> g_num_sms{0};
 
 }  // namespace
 
@@ -930,10 +932,9 @@ bool tc_stream_encode(const GemmDesc& d, const float* const* A, const float* con
 size_t tc_stream_map_bytes(int n_outer) { return (size_t)2 * n_outer * sizeof(CUtensorMap); }
 
 cudaError_t tc_stream_prepare() {
-  static std::once_flag once;
-  static cudaError_t result = cudaSuccess;
-  std::call_once(once, [] {
-    result = cudaFuncSetAttribute(tc_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  static DeviceOnce once;
+  return once([] {
+    cudaError_t result = cudaFuncSetAttribute(tc_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   kSmemBytes);
     if (result == cudaSuccess)
       result = cudaFuncSetAttribute(tc_chain_kernel<32>,
@@ -952,8 +953,8 @@ cudaError_t tc_stream_prepare() {
     if (result == cudaSuccess)
       result = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (result == cudaSuccess) g_num_sms = sms;
+    return result;
   });
-  return result;
 }
 
 cudaError_t launch_tc_stream(const GemmDesc& d, const TcStreamPlan& p, int* err, cudaStream_t st) {
@@ -971,7 +972,7 @@ cudaError_t launch_tc_stream(const GemmDesc& d, const TcStreamPlan& p, int* err,
   a.lev1 = p.lev1;
   a.err = err;
   const int total = a.n_outer * a.tiles_per_entry;
-  const int grid = total < g_num_sms ? total : g_num_sms;
+  const int grid = std::min<int>(total, g_num_sms);
   tc_stream_kernel<<<grid, kThreads, kSmemBytes, st>>>(d, a);
   return cudaGetLastError();
 }
@@ -1155,7 +1156,7 @@ cudaError_t launch_tc_chain(const GemmDesc& d1, const GemmDesc& d2, const TcStre
   a.lev1 = p.lev1;
   a.err = err;
   const int total = a.n_outer * a.tiles_per_entry;
-  const int grid = total < g_num_sms ? total : g_num_sms;
+  const int grid = std::min<int>(total, g_num_sms);
   if (d1.N == 64) tc_chain_kernel<64><<<grid, kFThreads, kFSmemBytes, st>>>(d2, a);
   else tc_chain_kernel<32><<<grid, kFThreads, kFSmemBytes, st>>>(d2, a);
   return cudaGetLastError();
