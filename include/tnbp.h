@@ -268,7 +268,10 @@ tn_status tn_bp_components(tn_handle* h, int32_t* comp_of_vertex, int32_t* sweep
  * and the raw messages, so the state is unchanged; the next BP iteration
  * captures its loop again with the new counts, and its results may differ
  * from the untuned ones in the last FP32 bits (the order of the partial
- * sums).  Per (chi, degree, precision) the launch shapes fix the key of a
+ * sums).  A sweep that runs as one launch (FP32 and the split modes under
+ * TN_KERNELS_AUTO up to chi = 32) has no such launches: the rows then give the
+ * time of each at its present count, and neither tuning nor a table changes
+ * the sweep.  Per (chi, degree, precision) the launch shapes fix the key of a
  * table row, so a table tuned on one handle applies to any handle of the same
  * chi, precision and graph shape.
  *   reps       timed launches per candidate, >= 1

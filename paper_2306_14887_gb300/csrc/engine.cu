@@ -942,15 +942,16 @@ tn_status build_site_jobs(tn_handle* h) {
   return upload_site_jobs(h, jobs, &h->site_jobs, &h->n_site_jobs);
 }
 
-// The sweep's contractions at small chi, with the split-K counts the plan's
-// degree-3 closes (launches 2, 4 and 7) have.
+// The sweep's contractions at small chi, with the split-K counts that the plan's
+// degree-3 closes (launches 2, 4 and 7) have untuned: a tuned count comes from the
+// time of a launch that does not run here.
 tn_status run_site_sweep(tn_handle* h) {
   int splits[3] = {1, 1, 1};
   if (!h->sites_by_deg[3].empty())
     for (int j = 0; j < 3; ++j) {
       const HostLaunch& L = h->sweep.L[j == 0 ? 2 : j == 1 ? 4 : 7];
       size_t pf = 0;
-      const int s = cgemm_plan(L.d, &pf, L.tuned);
+      const int s = cgemm_plan(L.d, &pf);
       splits[j] = pf > h->part_floats ? 1 : s;
     }
   TN_CUDA_TRY(launch_site_sweep(h->site_jobs, h->n_site_jobs, h->chi, splits,
@@ -2180,7 +2181,9 @@ tn_status tn_autotune(tn_handle* h, int32_t reps, char* table_out, size_t table_
     // at least 3% faster (timing noise keeps the heuristic's choice)
     int best = now, fastest = 0;
     float now_ms = -1.f, fastest_ms = 0.f;
-    for (int sc = 1; sc <= 64 && !st; sc *= 2) {
+    // A sweep that runs as one launch has no use for the counts: each is reported
+    // as it is.
+    for (int sc = h->n_site_jobs ? now : 1; sc <= 64 && !st; sc = h->n_site_jobs ? 65 : 2 * sc) {
       if (!splits_valid(h, L, kind, sc)) continue;
       set_splits(L, kind, sc);
       st = launch_one(h, L, kind);
