@@ -112,8 +112,9 @@ typedef struct {
   double solve_tol;     /* FP32 Jacobi of the shared and refined solves: it stops when every
                            pair of rows of the bond matrix has |<x_p, x_q>| <= solve_tol
                            ||x_p|| ||x_q||; <= 0 selects the default (refined: 2e-6, the
-                           FP32 floor; shared: 2e-6 for TN_FP32, 1e-4 for TN_TF32, 1e-3 for
-                           TN_BF16, about the relative rounding of the Gram inputs) */
+                           FP32 floor; shared: 2e-6 for FP32 products and TN_TF32X3, 1e-4 for
+                           TN_TF32, 1e-3 for TN_BF16, 1e-5 for the split products of
+                           TN_BF16X3, about the relative rounding of the Gram inputs) */
 } tn_config;
 
 /* Contraction kernels of the tensor-core modes.

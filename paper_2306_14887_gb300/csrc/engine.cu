@@ -1234,14 +1234,19 @@ void rx_matrix(double theta, double u[8]) {
   u[4] = 0; u[5] = -s; u[6] = c; u[7] = 0;
 }
 
+// The arithmetic that the handle's products run in.
+int product_prec(const tn_handle* h) { return cuda_core_mode(h->cfg) ? TN_FP32 : h->cfg.prec; }
+
 // Orthogonality tolerance of the shared solve's Jacobi: about the relative
 // rounding of its Gram inputs, which the contraction precision sets.
 double solve_tol(const tn_handle* h) {
   if (h->cfg.solve_tol > 0) return h->cfg.solve_tol;
-  if (h->cfg.prec == TN_TF32) return 1e-4;
-  if (h->cfg.prec == TN_BF16) return 1e-3;
-  if (h->cfg.prec == TN_BF16X3) return 1e-5;
-  return 2e-6;
+  switch (product_prec(h)) {
+    case TN_TF32: return 1e-4;
+    case TN_BF16: return 1e-3;
+    case TN_BF16X3: return 1e-5;
+    default: return 2e-6;
+  }
 }
 
 double default_svd_cut(const tn_handle* h) {
@@ -1260,10 +1265,10 @@ int solve_kind(int solve, int chi) {
 
 // Residual below which FP32-stored messages can no longer improve.
 double precision_floor(const tn_handle* h) {
-  switch (h->cfg.prec) {
+  switch (product_prec(h)) {
     case TN_TF32: return 2e-3;
     case TN_BF16: return 2e-2;
-    case TN_BF16X3: return 2e-5;  // split BF16: about 16 significant bits per operand
+    case TN_BF16X3: return 2e-5;  // split products: about 16 significant bits per operand
     default: return 2e-6;         // FP32 and split TF32 (about 21 bits)
   }
 }
