@@ -508,19 +508,19 @@ cudaError_t launch_first_leg_last(const float* T, float* TA, const int64_t* site
   if (n_sites <= 0 || d < 2) return cudaSuccess;
   int64_t rest = 1;
   for (int i = 1; i < d; ++i) rest *= chi;
-  if (4LL * n_sites > 65535) return cudaErrorInvalidValue;
+  constexpr int kMaxSites = 65535 / 4;  // four planes a site in the grid's z
   // site offsets are multiples of 4 floats (whole planes of chi^d values, chi
   // even) when chi % 32 == 0; the base pointers come from 256-byte allocations
   const bool wide = !tf32 && rest % 128 == 0 && chi % 32 == 0 &&
                     ((reinterpret_cast<uintptr_t>(T) | reinterpret_cast<uintptr_t>(TA)) & 15) == 0;
-  if (wide) {
-    dim3 grid((unsigned)(rest / 128), (unsigned)(chi / 32), (unsigned)(4 * n_sites));
-    first_leg_last_wide_kernel<<<grid, dim3(32, 8), 0, s>>>(T, TA, site_off, chi, rest);
-    return cudaGetLastError();
+  const int64_t tile = wide ? 128 : 32;
+  for (int i = 0; i < n_sites; i += kMaxSites) {
+    const dim3 grid((unsigned)((rest + tile - 1) / tile), (unsigned)((chi + 31) / 32),
+                    (unsigned)(4 * std::min(n_sites - i, kMaxSites)));
+    auto kernel = wide ? first_leg_last_wide_kernel
+                       : tf32 ? first_leg_last_kernel<true> : first_leg_last_kernel<false>;
+    kernel<<<grid, dim3(32, 8), 0, s>>>(T, TA, site_off + i, chi, rest);
   }
-  dim3 grid((unsigned)((rest + 31) / 32), (unsigned)((chi + 31) / 32), (unsigned)(4 * n_sites));
-  if (tf32) first_leg_last_kernel<true><<<grid, dim3(32, 8), 0, s>>>(T, TA, site_off, chi, rest);
-  else first_leg_last_kernel<false><<<grid, dim3(32, 8), 0, s>>>(T, TA, site_off, chi, rest);
   return cudaGetLastError();
 }
 
