@@ -2269,6 +2269,16 @@ tn_status tn_autotune_apply(tn_handle* h, const char* table, int32_t* n_applied)
   return TN_OK;
 }
 
+// Puts a handle's sweep and gate environments back on the plans' separate launches.
+// Not part of the interface: for comparing the one-launch kernels with them.
+tn_status tnbp_separate_launches(tn_handle* h) {
+  if (!h) { set_error("null handle"); return TN_EINVAL; }
+  h->n_site_jobs = 0;
+  std::fill(h->n_env_jobs.begin(), h->n_env_jobs.end(), 0);
+  if (h->loop_exec) { cudaGraphExecDestroy(h->loop_exec); h->loop_exec = nullptr; }
+  return TN_OK;
+}
+
 tn_status tn_bp_components(tn_handle* h, int32_t* comp_of_vertex, int32_t* sweeps_out,
                            double* residual_out, int32_t cap, int32_t* n_comp_out) {
   if (!h || cap < 0) { set_error("null handle or cap < 0"); return TN_EINVAL; }
