@@ -138,7 +138,8 @@ typedef struct {
  *   kept chi eigenvectors and eigenvalues of H = R_v conj(G_w) R_v^H; FP64 leg
  *   matrices by triangular solves.  Every quantity the outputs are computed
  *   from is FP64; the FP32 phase only chooses the basis the FP64 step starts
- *   from (chi <= 64; larger chi fall back to TN_SOLVE_FP64).
+ *   from (chi <= 64 and multiples of 16 up to 256; other chi fall back to
+ *   TN_SOLVE_FP64).
  * TN_SOLVE_FP64: Hermitian Jacobi eigen-solves of G_v and of H in FP64 on
  *   global-memory workspaces (all arithmetic FP64; slow on GB300, whose FP64
  *   rate is about 1/58 of its FP32 rate).  chi <= 256.
@@ -147,7 +148,7 @@ typedef struct {
  *   K with FP32 rotations, FP32 triangular solves for the leg matrices
  *   (chi <= 64; larger chi fall back to TN_SOLVE_FP64).  Singular values to
  *   about 2e-6 relative; end to end about 1e-5 in <Z> against the FP64 oracle.
- * TN_SOLVE_AUTO: TN_SOLVE_REFINED for chi <= 64, TN_SOLVE_FP64 above. */
+ * TN_SOLVE_AUTO: TN_SOLVE_REFINED, with its fall-back. */
 #define TN_SOLVE_AUTO 0
 #define TN_SOLVE_FP64 1
 #define TN_SOLVE_SHARED 2
@@ -210,8 +211,10 @@ tn_status tn_apply_floquet(tn_handle* h, double theta_h, int32_t steps);
  * RX(theta_v[v]) on site v.  theta_v: n_vertices host doubles (caller-owned,
  * copied at the call).  Used to evolve many independent instances as one
  * graph (their disjoint union): BP and the gates never couple components, so
- * each component evolves as it would alone, while every contraction of every
- * instance runs in the same launches.  Errors: as tn_apply_floquet, plus
+ * each component evolves as it would alone, up to rounding, while every
+ * contraction of every instance runs in the same launches.  (How a launch cuts
+ * its sums, and in FP32 at chi = 28 and 32 whether a sweep runs as one launch,
+ * follows the size of the whole union.)  Errors: as tn_apply_floquet, plus
  * TN_EINVAL for a null or non-finite theta_v.
  */
 tn_status tn_apply_floquet_field(tn_handle* h, const double* theta_v, int32_t steps);
@@ -243,7 +246,8 @@ tn_status tn_bp_converge(tn_handle* h, double tol, int32_t max_iters,
  * regauging in tn_apply_floquet acts on every component separately: a
  * component stops at its own tolerance (or FP32 residual floor, or max_iters)
  * and its messages stay as they are while the others continue, so each
- * instance receives the sweeps it would receive alone.
+ * instance receives the sweeps that the rule gives it alone (on messages that
+ * may differ by rounding, see tn_apply_floquet_field).
  *   comp_of_vertex  n_vertices host int32 (may be NULL): component of each vertex,
  *                   numbered in order of their smallest vertex.
  *   sweeps_out      cap host int32 (may be NULL): sweeps of each component in
@@ -352,17 +356,21 @@ tn_status tn_expect_z_all(tn_handle* h, double* out);
  *         two-site update of exp(sign i pi/4 Z Z);
  *   s_out [edge][chi] FP64 (output): the kept singular values with ||S||_2 = 1
  *         (zeros past the rank or below svd_cutoff * sigma_1).
- * The FP64 workspace (12 (2 chi)^2 doubles per edge) is allocated with
- * cudaMallocAsync on the stream and freed before return.
+ * The FP64 workspace (12 (2 chi)^2 doubles per edge; of the refined solve about
+ * a third) is allocated on the stream from a pool of the library's own and freed
+ * before return; the pool keeps up to 64 MB on a device until the process ends.
+ * (A cudaDeviceReset in the application destroys the pool: make no further call
+ * on that device.)
  * Errors: TN_EINVAL, TN_ENUMERIC (zero or non-finite spectrum), TN_ECUDA.
  */
 tn_status tn_truncation_solve(const float* gram, float* dmat, double* s_out, int32_t n_edges,
                               int32_t chi, int32_t sign, double svd_cutoff, void* cuda_stream);
 
 /* tn_truncation_solve_ex — tn_truncation_solve with the solve variant chosen:
- * TN_SOLVE_FP64 (what tn_truncation_solve runs), TN_SOLVE_REFINED or
- * TN_SOLVE_SHARED (both chi <= 64, TN_EUNSUPPORTED otherwise), or
- * TN_SOLVE_AUTO (TN_SOLVE_REFINED for chi <= 64, TN_SOLVE_FP64 above). */
+ * TN_SOLVE_FP64 (what tn_truncation_solve runs), TN_SOLVE_REFINED (chi <= 64 and
+ * multiples of 16 up to 256) or TN_SOLVE_SHARED (chi <= 64), TN_EUNSUPPORTED at
+ * other chi, or TN_SOLVE_AUTO (TN_SOLVE_REFINED where it runs, else
+ * TN_SOLVE_FP64). */
 tn_status tn_truncation_solve_ex(const float* gram, float* dmat, double* s_out, int32_t n_edges,
                                  int32_t chi, int32_t sign, double svd_cutoff, int32_t solve,
                                  void* cuda_stream);

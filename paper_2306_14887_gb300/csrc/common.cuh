@@ -278,9 +278,10 @@ struct RefineLayout {
   int64_t U1;     // [chi][n] complex: refined kept columns
   int64_t lam0;   // [n]: sigma^2 of the starting basis (decreasing)
   int64_t lam1;   // [chi]: refined eigenvalues of the kept columns
-  int64_t misc;   // [4]: sum of all sigma^2 of the start, FP32 sweeps
+  int64_t misc;   // [4]: sum of all sigma^2 of the start, FP32 sweeps; 2 chi > 128: ||K||_F^2, sweeps
   int64_t ints;   // int32 [2 chi] perm, [2] rank, [1] active columns
-  int64_t S;      // [n][n] float2: FP32 G_w and its Cholesky factor (2 chi > 128 only)
+  int64_t S;      // 2 chi > 128 only: [2][chi][chi] complex, the FP64 Cholesky's rows, then
+                  // [n][n] float2, G_w's FP32 Cholesky factor
   int64_t stride;
 };
 __host__ __device__ inline RefineLayout refine_layout(int chi) {
@@ -304,12 +305,13 @@ bool solve32_supported(int chi);
 cudaError_t solve32_prepare();  // kernel attributes, as simt_prepare
 cudaError_t launch_solve32(const SolveArgs& a, cudaStream_t s);
 // The refined solve's FP32 starting basis for 2 chi > 128 (solve32.cu): the
-// bond matrix in the global workspace, one CTA per edge, 16 <= chi <= 256.
+// bond matrix in the global workspace, one cluster per edge (8 CTAs up to
+// 2 chi = 256, 16 above), chi a multiple of 16 up to 256.
 cudaError_t basis_gmem_prepare();
 cudaError_t launch_basis_gmem(const SolveArgs& a, cudaStream_t s);
 // Refined solve (solve_refine.cu): FP64 Cholesky, FP32 starting basis, FP64
-// Newton refinement and FP64 leg matrices; chi <= 64.  work: solve_work_doubles
-// per edge.
+// Newton refinement and FP64 leg matrices; chi <= 64 and multiples of 16 up to
+// 256.  work: refine_layout(chi).stride per edge.
 bool solve_refined_supported(int chi);
 cudaError_t refine_prepare();
 cudaError_t launch_solve_refined(const SolveArgs& a, cudaStream_t s);

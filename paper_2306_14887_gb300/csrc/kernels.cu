@@ -524,7 +524,7 @@ cudaError_t launch_first_leg_last(const float* T, float* TA, const int64_t* site
   return cudaGetLastError();
 }
 
-// The shared-memory limit of the normalise kernel, raised once to the largest
+// The shared-memory limit of the normalise kernel, raised once per device to the largest
 // tile the kernel takes (chi with 2 chi (chi + 1) floats <= 200 KB); thread-safe.
 cudaError_t normalise_prepare(int) {
   static DeviceOnce once;

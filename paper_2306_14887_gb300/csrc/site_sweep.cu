@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     const int t = st * kStreamWarps + kk / kSlice, k = slice_k(t) + kk % kSlice;
     return t < ns && k < (second(t) ? 2 * K : K) ? k : -1;
   };
-  // stage st: k = 128 st .. + 127 of (p, g, f), as [o'][k]
+  // stage st: k = kStageK st .. + kStageK - 1 of (p, g, f), as [o'][k]
   auto load_stage = [&](int st) {
     float2* dst = sStage + (st & 1) * stage_len;
     if (job.open < 2) {  // contiguous along f
