@@ -141,6 +141,7 @@ struct tn_handle {
   // the same for a gate layer's environments, instead of gate_env
   std::vector<tnbp::SiteJob*> env_jobs;
   std::vector<int> n_env_jobs;
+  std::vector<std::vector<unsigned char>> staged;  // uploads in flight during tn_create
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 
@@ -195,6 +196,16 @@ void* dev_alloc(tn_handle* h, size_t bytes) {
   h->allocations.push_back({p, bytes});
   h->bytes += bytes;
   return p;
+}
+
+// Host data into the handle's memory, in the order of its stream: the allocator
+// hands memory out for that stream, where work on its previous use may still run,
+// and kernels on a non-blocking stream would not wait for a copy elsewhere.  The
+// data are kept until tn_create has waited for the stream.
+cudaError_t upload(tn_handle* h, void* dst, const void* src, size_t bytes) {
+  const unsigned char* p = static_cast<const unsigned char*>(src);
+  h->staged.emplace_back(p, p + bytes);
+  return cudaMemcpyAsync(dst, h->staged.back().data(), bytes, cudaMemcpyHostToDevice, h->stream);
 }
 
 void dev_free(tn_handle* h, void* p) {
@@ -896,8 +907,7 @@ tn_status upload_site_jobs(tn_handle* h, const std::vector<SiteJob>& jobs, SiteJ
   if (jobs.empty()) return TN_OK;
   *dev = (SiteJob*)dev_alloc(h, sizeof(SiteJob) * jobs.size());
   if (!*dev) { set_error("device allocation of the sweep jobs failed"); return TN_ENOMEM; }
-  if (cudaMemcpy(*dev, jobs.data(), sizeof(SiteJob) * jobs.size(), cudaMemcpyHostToDevice) !=
-          cudaSuccess ||
+  if (upload(h, *dev, jobs.data(), sizeof(SiteJob) * jobs.size()) != cudaSuccess ||
       site_sweep_prepare() != cudaSuccess) {
     set_error("preparing the sweep jobs failed");
     return TN_ECUDA;
@@ -971,8 +981,7 @@ tn_status attach_components(tn_handle* h) {
     for (size_t i = 0; i < comp.size(); ++i) comp[i] = h->comp_of_vertex[L.outer_site[i]];
     int* dc = (int*)dev_alloc(h, sizeof(int) * comp.size());
     if (!dc) { set_error("device allocation of the component tables failed"); return TN_ENOMEM; }
-    if (cudaMemcpy(dc, comp.data(), sizeof(int) * comp.size(), cudaMemcpyHostToDevice) !=
-        cudaSuccess) {
+    if (upload(h, dc, comp.data(), sizeof(int) * comp.size()) != cudaSuccess) {
       set_error("upload of the component tables failed");
       return TN_ECUDA;
     }
@@ -1867,7 +1876,12 @@ tn_status tn_create(const tn_graph* graph, const tn_config* cfg, const tn_alloca
   h->t_floats = off;
   const int nmsg = 2 * (int)g.eu.size();
   for (auto& l : g.layers) h->max_layer = std::max(h->max_layer, (int)l.size());
-  auto fail = [&](tn_status s) { dev_free_all(h); delete h; return s; };
+  auto fail = [&](tn_status s) {
+    if (!h->staged.empty()) cudaStreamSynchronize(h->stream);
+    dev_free_all(h);
+    delete h;
+    return s;
+  };
   h->T = (float*)dev_alloc(h, sizeof(float) * off);
   h->Ts = (float*)dev_alloc(h, sizeof(float) * off);
   h->Y1 = (float*)dev_alloc(h, sizeof(float) * off);
@@ -1960,8 +1974,8 @@ tn_status tn_create(const tn_graph* graph, const tn_config* cfg, const tn_alloca
     std::vector<int64_t> offs;
     for (int v : h->sites_by_deg[d]) offs.push_back(h->t_off[v]);
     if (!offs.empty() &&
-        cudaMemcpy(h->site_offs_by_deg[d], offs.data(), sizeof(int64_t) * offs.size(),
-                   cudaMemcpyHostToDevice) != cudaSuccess) {
+        upload(h, h->site_offs_by_deg[d], offs.data(), sizeof(int64_t) * offs.size()) !=
+            cudaSuccess) {
       set_error("upload of site offsets failed");
       return fail(TN_ECUDA);
     }
@@ -1972,8 +1986,7 @@ tn_status tn_create(const tn_graph* graph, const tn_config* cfg, const tn_alloca
       v.push_back(dir_id(g, g.eu[e], e));
       v.push_back(dir_id(g, g.ew[e], e));
     }
-    if (cudaMemcpy(h->d_layer_msg_vw[li], v.data(), sizeof(int32_t) * v.size(),
-                   cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (upload(h, h->d_layer_msg_vw[li], v.data(), sizeof(int32_t) * v.size()) != cudaSuccess) {
       set_error("upload of layer tables failed");
       return fail(TN_ECUDA);
     }
@@ -1981,14 +1994,14 @@ tn_status tn_create(const tn_graph* graph, const tn_config* cfg, const tn_alloca
   {
     std::vector<int> cm(2 * g.eu.size());
     for (size_t e = 0; e < g.eu.size(); ++e) cm[2 * e] = cm[2 * e + 1] = h->comp_of_vertex[g.eu[e]];
-    if (!cm.empty() && cudaMemcpy(h->comp_of_msg, cm.data(), sizeof(int) * cm.size(),
-                                  cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (!cm.empty() &&
+        upload(h, h->comp_of_msg, cm.data(), sizeof(int) * cm.size()) != cudaSuccess) {
       set_error("upload of the component table failed");
       return fail(TN_ECUDA);
     }
   }
-  cudaMemset(h->res_bits, 0, 64);
-  cudaMemset(h->comp_state, 0, sizeof(double) * 4 * std::max(1, h->n_comp));
+  cudaMemsetAsync(h->res_bits, 0, 64, h->stream);
+  cudaMemsetAsync(h->comp_state, 0, sizeof(double) * 4 * std::max(1, h->n_comp), h->stream);
   if (cudaMallocHost(&h->h_status, 8 * sizeof(unsigned long long)) != cudaSuccess) {
     cudaGetLastError();
     set_error("pinned host allocation failed");
@@ -2037,8 +2050,9 @@ tn_status tn_create(const tn_graph* graph, const tn_config* cfg, const tn_alloca
   if (st) { delete[] h->h_stats; return fail(st); }
   st = attach_components(h);
   if (st) { delete[] h->h_stats; return fail(st); }
-  st = init_state(h);
+  st = init_state(h);  // ends with a wait for the stream
   if (st) { delete[] h->h_stats; return fail(st); }
+  h->staged.clear();
   *out = h;
   return TN_OK;
 }
